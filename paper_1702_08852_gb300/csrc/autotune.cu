@@ -69,7 +69,7 @@ wf_status autotune(Plan &P) {
   }
   // inputs are zeros: the kernels' work does not depend on the values
   WF_CUDA(cudaMemsetAsync(P.xs32, 0, sizeof(float2) * P.nalm, P.stream));
-  WF_CUDA(cudaMemsetAsync(P.xs64, 0, sizeof(double2) * P.nalm, P.stream));
+  WF_CUDA(cudaMemsetAsync(P.xtmp, 0, sizeof(double2) * P.nalm, P.stream));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   WF_CUDA(cudaEventCreate(&e0));
   WF_CUDA(cudaEventCreate(&e1));
@@ -91,7 +91,7 @@ wf_status autotune(Plan &P) {
       if (k) P.syn_x2 = ci == 5 ? 2 : (x2 ? 1 : 0);
       float ms = 0.f;
       st = k ? time_synth<float2>(P, P.xs32, P.F32, e0, e1, &ms)
-             : time_synth<double2>(P, P.xs64, P.F64, e0, e1, &ms);
+             : time_synth<double2>(P, P.xtmp, P.F64, e0, e1, &ms);
       if (st != WF_OK) break;
       P.tune_syn_ms[k][ci] = ms;
       if (ms < best) {

@@ -28,6 +28,7 @@ static wf_status arg_error(const char *msg) {
 static void free_plan(wf_plan_s *P) {
   if (!P) return;
   free_group(*P);
+  free_pair_tables(*P);
   for (int i = 0; i < 3; ++i)
     if (P->graph[i]) cudaGraphExecDestroy(P->graph[i]);
   void *bufs[] = {P->pairs, P->cl_d,   P->rc,      P->rg,     P->rc32,   P->seed_l,
@@ -76,10 +77,6 @@ static wf_status alloc_work(Plan &P) {
     // queue-scheduled FP32 analysis: partial sums of tiles of 128 ring pairs
     // (the smallest tile of its variants)
     const long tiles = (P.npairs + 127) / 128;
-    int dev = 0;
-    WF_CUDA(cudaGetDevice(&dev));
-    P.device = dev;
-    WF_CUDA(cudaDeviceGetAttribute(&P.num_sms, cudaDevAttrMultiProcessorCount, dev));
     // 16 bytes per entry: FP32 complex for the FP32 kernels, FP64 complex
     // for the double-float anchor analysis
     // (and the packed analysis' global accumulators: 4 warps x FP32 complex)

@@ -1651,16 +1651,9 @@ static cudaError_t set_big_smem_anal(int big) {
 
 wf_status init_legendre_attributes() {
   const int big = 220 * 1024;
-  WF_CUDA((set_big_smem_synth<double, 1>(big)));
-  WF_CUDA((set_big_smem_synth<double, 2>(big)));
-  WF_CUDA((set_big_smem_synth<double, 4>(big)));
   WF_CUDA((set_big_smem_synth<float, 1>(big)));
   WF_CUDA((set_big_smem_synth<float, 2>(big)));
   WF_CUDA((set_big_smem_synth<float, 4>(big)));
-  WF_CUDA((set_big_smem_anal<double, 2>(big)));
-  WF_CUDA((set_big_smem_anal<double, 4>(big)));
-  WF_CUDA((set_big_smem_anal<double, 8>(big)));
-  WF_CUDA((set_big_smem_anal<double, 16>(big)));
   WF_CUDA((set_big_smem_anal<float, 2>(big)));
   WF_CUDA((set_big_smem_anal<float, 4>(big)));
   WF_CUDA((set_big_smem_anal<float, 8>(big)));
@@ -1727,16 +1720,9 @@ wf_status launch_prescale_dd(const Plan &P, const double2 *x, float4 *xs) {
   return WF_OK;
 }
 
-template wf_status launch_prescale<double2>(const Plan &, const double2 *, double2 *);
 template wf_status launch_prescale<float2>(const Plan &, const double2 *, float2 *);
-template wf_status launch_legendre_synth<double2>(const Plan &, const double2 *,
-                                                  double2 *, const SolverState *,
-                                                  int);
 template wf_status launch_legendre_synth<float2>(const Plan &, const float2 *,
                                                  float2 *, const SolverState *, int);
-template wf_status launch_legendre_anal<double2>(const Plan &, const double2 *,
-                                                 double2 *, const SolverState *,
-                                                 int, int, const double2 *, double2 *);
 template wf_status launch_legendre_anal<float2>(const Plan &, const float2 *,
                                                 double2 *, const SolverState *,
                                                 int, int, const double2 *, float2 *);

@@ -1,0 +1,762 @@
+// legpair.cu -- associated-Legendre synthesis and analysis in the parity-pair
+// basis, with the recurrence restarted from a table of checkpoints.
+//
+// Ring pair k is the north ring k and, but for the equator (k = npairs - 1), the
+// south ring 2 npairs - 2 - k.
+//
+// Basis (Ishioka 2018, J. Meteor. Soc. Japan 96, "A new recurrence formula for
+// efficient computation of spherical harmonic transform").  With
+// eps_l = sqrt((l^2 - m^2) / (4 l^2 - 1)), z lam_l = eps_{l+1} lam_{l+1} +
+// eps_l lam_{l-1}, let Q_j = lam_{m+2j+1} / z (an even function of z, as the
+// lam of even l - m are).  Then
+//   lam_{m+2j+1} = z Q_j,   lam_{m+2j} = eps_{m+2j+1} Q_j + eps_{m+2j} Q_{j-1},
+// so one function serves an even and an odd l, and Q_j steps by two l at once:
+//   eps_{l+1} eps_{l+2} Q_{j+1} = (z^2 - eps_{l+1}^2 - eps_l^2) Q_j
+//                                 - eps_l eps_{l-1} Q_{j-1},   l = m + 2 j + 1.
+// Scaled and sign-folded, Q_j = h_j s_j with h_0 = h_1 = 1 and
+//   s_j = (A_j w + B_j) s_{j-1} + s_{j-2}
+// (tables indexed by the j they produce).  w = z^2 with B, or, for the ring
+// pairs k < kpol near the pole, w = -sin^2 theta with C = A + B in B's place:
+// that form keeps the small angle there (z^2 rounds it away).  The two forms
+// are equal; each CTA or warp takes the one of the pairs it holds.
+//
+// Per (m, ring pair) and j this costs 2 multiply-adds for the recurrence and 4
+// for the two complex sums, 3 per (l, m, pair) term; the one-step recurrence in
+// lam_l needs a multiply and 3 multiply-adds (in FP32, with z in two parts, a
+// multiply and 4).
+//
+// Near the equator Q_j grows like lam / z while neighbouring Q_j cancel in
+// lam_{m+2j}, so rounding in s_j is amplified by up to 1/z there (measured in
+// FP64 at Nside 1024: 1.1e-13 of the map's rms on the rings next to the equator,
+// 1.5e-15 with the one-step recurrence).  The FP64 synthesis therefore gives the
+// ring pairs k >= keq (|z| < ~0.2, where lam_mm itself is the seed for every m)
+// to the one-step recurrence lam_l <- z lam_{l-1}, lam_{l-2}, two l per j, at 8
+// multiply-adds instead of 6.  The analysis, which sums over all rings, does not
+// need it (2.6e-14 of the rms against 3.0e-14 with the one-step recurrence).
+//
+// Bound: the FP64 unit, 2 multiply-adds per clock and SM.  At Nside 1024, lmax 2048
+// (3.14e9 terms) the synthesis takes 16.6 ms (21.4 ms with the one-step recurrence)
+// and the analysis 16.9 ms (29.0 ms), against 15 ms for 3 multiply-adds per term at
+// the unit's measured 1.25 TFLOP/s; at Nside 150, lmax 311, 0.106 and 0.142 ms
+// (0.233 and 0.276 ms).
+//
+// Checkpoints: ck[(block b of 16 j of m)][pair] holds (s_{16b-1}, s_{16b-2}),
+// or, in the block where the pair's first |Q_j| >= 2^-100 lies (j = js), the two
+// seeds (s_js, s_js+1); terms below 2^-100 are dropped.  Any 16 j can therefore
+// be computed on their own: a warp of the analysis owns 16 j of one m, keeps
+// their 64 sums per lane in registers over all ring pairs, and reduces them
+// across the lanes once.
+#include <limits.h>
+#include <math.h>
+
+#include <algorithm>
+#include <type_traits>
+#include <vector>
+
+#include "wf_internal.cuh"
+
+namespace wf {
+
+namespace {
+
+// ------------------------------------------------------------- indexing
+// j of one m: J = (L - m) / 2 + 1; first table entry of m: sum of J over the
+// smaller m.  Blocks of 16 j of one m: (L - m) / 32 + 1.
+__host__ __device__ __forceinline__ long tri_j(long n) { return n + 1 + (n * n) / 4; }
+__host__ __device__ __forceinline__ long pair_base(int lmax, int m) {
+  return tri_j(lmax) - tri_j(lmax - m);
+}
+__host__ __device__ __forceinline__ long tri_b(long n) {
+  const long q = (n + 1) / 32, r = (n + 1) % 32;  // t = 0 .. n: sum of t / 32 + 1
+  return n + 1 + 16 * q * (q - 1) + q * r;
+}
+__host__ __device__ __forceinline__ long block_base(int lmax, int m) {
+  return tri_b(lmax) - tri_b(lmax - m);
+}
+__device__ __forceinline__ long alm_base(int lmax, int m) {  // index of (m, m)
+  return (long)m * (2 * lmax + 1 - m) / 2 + m;
+}
+
+// ------------------------------------------------------------- arithmetic
+template <typename V> struct Cx;  // complex element of F, G and the alm input
+template <> struct Cx<double> { typedef double2 type; };
+template <typename V> struct alignas(16) Quad { V a, b, c, d; };
+template <typename V> struct alignas(2 * sizeof(V)) Pair { V a, b; };
+
+__device__ __forceinline__ double fmav(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ void accv(double &acc, double s, double x) { acc = fma(s, x, acc); }
+
+__device__ __forceinline__ int wmin(int v) { return __reduce_min_sync(0xffffffffu, v); }
+__device__ __forceinline__ int wmax(int v) { return __reduce_max_sync(0xffffffffu, v); }
+
+// v[0..31] per lane -> lane i returns the sum over the lanes of v[i]
+template <typename V>
+__device__ __forceinline__ V lane_sums(V *v, int lane) {
+#pragma unroll
+  for (int s = 16; s >= 1; s >>= 1) {
+    const bool upper = (lane & s) != 0;
+#pragma unroll
+    for (int j = 0; j < s; ++j) {
+      const V send = upper ? v[j] : v[j + s];
+      const V keep = upper ? v[j + s] : v[j];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+    }
+  }
+  return v[0];
+}
+
+}  // namespace
+
+// ------------------------------------------------------------- synthesis
+// One thread per NP ring pairs of one m (grid: tiles of pairs x m), a
+// warp-uniform loop over j.  The CTA stages the m's coefficients in shared
+// memory, combined to the pair basis on the way:
+//   E_j = se_j a_{m+2j} + sn_j a_{m+2j+2},   O_j = so_j a_{m+2j+1}.
+// F_north = sum_j s_j (E_j + z O_j), F_south the difference.
+constexpr int PSYN_THREADS = 64;
+
+template <typename V, int NP>
+__global__ void __launch_bounds__(PSYN_THREADS)
+    k_pair_synth(const PairTab<V> t, int npairs, int lmax,
+                 const typename Cx<V>::type *__restrict__ x,
+                 typename Cx<V>::type *__restrict__ F, const SolverState *__restrict__ st,
+                 int lstatic) {
+  typedef typename Cx<V>::type C;
+  const int m = blockIdx.y;
+  int L = lstatic;
+  if (st) {
+    if (st->done) return;
+    L = st->lcur;
+  }
+  if (m > L) return;  // the ring step ignores m above the band
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int J = (L - m) / 2 + 1;
+  Quad<V> *sx = reinterpret_cast<Quad<V> *>(smraw);
+  Pair<V> *sr = reinterpret_cast<Pair<V> *>(smraw + sizeof(Quad<V>) * J);
+  const int pair00 = blockIdx.x * blockDim.x * NP;
+  const bool polar = pair00 + (int)blockDim.x * NP / 2 <= t.kpol;
+  const bool equator = t.rec_e && pair00 >= t.keq;
+  const V *wt = polar ? t.w + npairs : t.w;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int pair0 = pair00 + warp * 32 * NP;
+  V w[NP];
+  int js[NP];
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {  // in flight while the coefficients are staged
+    const int k = pair0 + lane + 32 * i;
+    w[i] = (V)0;
+    js[i] = INT_MAX / 2;
+    if (k < npairs) {
+      w[i] = wt[k];
+      js[i] = t.js[(long)m * npairs + k];
+    }
+  }
+  {
+    const long q0 = pair_base(lmax, m), a0 = alm_base(lmax, m);
+    const Pair<V> *rec =
+        reinterpret_cast<const Pair<V> *>(equator ? t.rec_e : polar ? t.rec_c : t.rec_b);
+    for (int j = threadIdx.x; j < J; j += blockDim.x) {
+      const int l = m + 2 * j;
+      const C c0 = x[a0 + 2 * j];
+      C c1 = {}, c2 = {};
+      if (l + 1 <= L) c1 = x[a0 + 2 * j + 1];
+      if (l + 2 <= L) c2 = x[a0 + 2 * j + 2];
+      if (equator) {
+        const V ge = t.ge[q0 + j], go = t.go[q0 + j];
+        sx[j] = {ge * c0.x, ge * c0.y, go * c1.x, go * c1.y};
+        sr[j] = rec[q0 + j];
+        continue;
+      }
+      const V se = t.se[q0 + j], sn = t.sn[q0 + j], so = t.so[q0 + j];
+      sx[j] = {fmav(se, c0.x, sn * c2.x), fmav(se, c0.y, sn * c2.y), so * c1.x, so * c1.y};
+      sr[j] = rec[q0 + j];
+    }
+  }
+  __syncthreads();
+  if (pair0 >= npairs) return;
+
+  const long stride = lmax + 1;
+  if (equator) {
+    V z[NP], u[NP], o[NP], er[NP], ei[NP], orr[NP], oi[NP];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const int k = pair0 + lane + 32 * i;
+      u[i] = o[i] = er[i] = ei[i] = orr[i] = oi[i] = z[i] = (V)0;
+      if (k < npairs) {
+        z[i] = t.z[k];
+        u[i] = t.lmm[(long)m * npairs + k];  // lam_mm
+      }
+    }
+#pragma unroll 2
+    for (int j = 0; j < J; ++j) {
+      const Pair<V> r = sr[j];
+      const Quad<V> q = sx[j];
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        u[i] = fmav(r.a * z[i], o[i], u[i]);
+        accv(er[i], u[i], q.a);
+        accv(ei[i], u[i], q.b);
+        o[i] = fmav(r.b * z[i], u[i], o[i]);
+        accv(orr[i], o[i], q.c);
+        accv(oi[i], o[i], q.d);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const int k = pair0 + lane + 32 * i;
+      if (k >= npairs) continue;
+      F[k * stride + m] = {er[i] + orr[i], ei[i] + oi[i]};
+      if (k < npairs - 1)
+        F[(2 * npairs - 2 - k) * stride + m] = {er[i] - orr[i], ei[i] - oi[i]};
+    }
+    return;
+  }
+
+  V s1[NP], s2[NP], d0[NP], d1[NP], er[NP], ei[NP], orr[NP], oi[NP];
+  int jmin = INT_MAX, jinj = -1;
+  const long cb = block_base(lmax, m);
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    const int k = pair0 + lane + 32 * i;
+    s1[i] = s2[i] = d0[i] = d1[i] = er[i] = ei[i] = orr[i] = oi[i] = (V)0;
+    if (js[i] < J) {
+      const C s = t.ck[(cb + (js[i] >> 4)) * npairs + k];
+      d0[i] = s.x;
+      d1[i] = s.y;
+      jmin = min(jmin, js[i]);
+      jinj = max(jinj, js[i] + 1);
+    }
+  }
+  jmin = wmin(jmin);
+  jinj = min(wmax(jinj), J - 1);
+  int j = jmin;
+  for (; j <= jinj; ++j) {  // seeds may still enter
+    const Pair<V> r = sr[j];
+    const Quad<V> q = sx[j];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      V s = fmav(fmav(r.a, w[i], r.b), s1[i], s2[i]);
+      s = j == js[i] ? d0[i] : s;
+      s = j == js[i] + 1 ? d1[i] : s;
+      s2[i] = s1[i];
+      s1[i] = s;
+      accv(er[i], s, q.a);
+      accv(ei[i], s, q.b);
+      accv(orr[i], s, q.c);
+      accv(oi[i], s, q.d);
+    }
+  }
+#pragma unroll 4
+  for (; j < J; ++j) {
+    const Pair<V> r = sr[j];
+    const Quad<V> q = sx[j];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const V s = fmav(fmav(r.a, w[i], r.b), s1[i], s2[i]);
+      s2[i] = s1[i];
+      s1[i] = s;
+      accv(er[i], s, q.a);
+      accv(ei[i], s, q.b);
+      accv(orr[i], s, q.c);
+      accv(oi[i], s, q.d);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    const int k = pair0 + lane + 32 * i;
+    if (k >= npairs) continue;
+    const V z = t.z[k], zr = z * orr[i], zi = z * oi[i];
+    F[k * stride + m] = {er[i] + zr, ei[i] + zi};
+    if (k < npairs - 1) F[(2 * npairs - 2 - k) * stride + m] = {er[i] - zr, ei[i] - zi};
+  }
+}
+
+// ------------------------------------------------------------- analysis
+// One CTA per m.  The m's ring sums P_k = (G_N + G_S, z (G_N - G_S)) are staged
+// in shared memory, in tiles of PANA_TILE pairs; each warp takes blocks of 16 j,
+// holds the block's 64 sums per lane in registers, walks the tile's pairs 32 at a
+// time (one per lane, the recurrence restarted from the checkpoints) and reduces
+// across the lanes into D.  The epilogue goes back to l,
+//   a_{m+2j} = Omega (se_j De_j + sn_{j-1} De_{j-1}),  a_{m+2j+1} = Omega so_j Do_j,
+// with the solver's filter, source term and Cauchy sums fused.
+constexpr int PANA_TILE = 2048;
+constexpr int PANA_MAXWARPS = 8;
+constexpr int CKJ = 16;
+
+// 16 steps of one pair: the recurrence and the four sums of each j.  INJ: the
+// pair's seeds (d0, d1) may enter, at step `rel` and the next.
+template <typename V, bool INJ>
+__device__ __forceinline__ void pair_block(V (&v)[4 * CKJ], const Pair<V> *__restrict__ sr, V w,
+                                           V s1, V s2, const Quad<V> &p, int rel, V d0, V d1) {
+#pragma unroll
+  for (int jj = 0; jj < CKJ; ++jj) {
+    const Pair<V> r = sr[jj];
+    V s = fmav(fmav(r.a, w, r.b), s1, s2);
+    if (INJ) {
+      s = jj == rel ? d0 : s;
+      s = jj == rel + 1 ? d1 : s;
+    }
+    s2 = s1;
+    s1 = s;
+    accv(v[4 * jj], s, p.a);
+    accv(v[4 * jj + 1], s, p.b);
+    accv(v[4 * jj + 2], s, p.c);
+    accv(v[4 * jj + 3], s, p.d);
+  }
+}
+
+// Epilogue of one coefficient (FP64): a = Omega (sr, si), then in ANA_FILTER mode
+// the source term of an anchored stage, the filter f_l = Sbar / (Sbar + xi Omega),
+// Sbar = max(C_l - mu Omega, 0) (Eq. 15, App. B) and the Cauchy partial sums
+// (weight wm = 1 for m = 0, 2 else); writes x.
+__device__ __forceinline__ void pair_finish(long i, int l, double ar, double ai, double wm,
+                                            int mode, const double *__restrict__ cl,
+                                            double omega, double xi, double mu,
+                                            const double2 *__restrict__ src,
+                                            const double2 *__restrict__ xa,
+                                            double2 *__restrict__ x, double &num, double &den,
+                                            double &dx) {
+  if (mode == ANA_FILTER) {
+    const double sbar = fmax(cl[l] - mu * omega, 0.0);
+    const double f = sbar / (sbar + xi * omega);
+    if (src) {  // harmonic source term of a correction solve
+      ar += xi * omega * src[i].x;
+      ai += xi * omega * src[i].y;
+    }
+    ar *= f;
+    ai *= f;
+    const double2 old = x[i];
+    const double dr = ar - old.x, di = ai - old.y;
+    num += wm * (dr * dr + di * di);
+    den += wm * (ar * ar + ai * ai);
+    if (xa) {  // anchored stage: ||x_a + delta||^2
+      const double2 b = xa[i];
+      const double tr = ar + b.x, ti = ai + b.y;
+      dx += wm * (tr * tr + ti * ti);
+    }
+  }
+  x[i] = make_double2(ar, ai);
+}
+
+// block sums of the Cauchy partials -> partials[2m], [2m + 1] and (anchored
+// stages) [2 (lmax + 1) + m], in a fixed order
+__device__ __forceinline__ void pair_partials(double num, double den, double dx, int m, int lmax,
+                                              double *__restrict__ partials) {
+  __shared__ double ws[3][PANA_MAXWARPS];
+  for (int o = 16; o > 0; o >>= 1) {
+    num += __shfl_xor_sync(0xffffffffu, num, o);
+    den += __shfl_xor_sync(0xffffffffu, den, o);
+    dx += __shfl_xor_sync(0xffffffffu, dx, o);
+  }
+  const int warp = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    ws[0][warp] = num;
+    ws[1][warp] = den;
+    ws[2][warp] = dx;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a = 0.0, b = 0.0, c = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+      a += ws[0][w];
+      b += ws[1][w];
+      c += ws[2][w];
+    }
+    partials[2 * m] = a;
+    partials[2 * m + 1] = b;
+    partials[2 * (lmax + 1) + m] = c;
+  }
+}
+
+template <typename V>
+__global__ void __launch_bounds__(32 * PANA_MAXWARPS)
+    k_pair_anal(const PairTab<V> t, int npairs, int lmax,
+                const double *__restrict__ cl, double omega,
+                const typename Cx<V>::type *__restrict__ G, double2 *__restrict__ x,
+                double *__restrict__ partials, const double2 *__restrict__ src,
+                const SolverState *__restrict__ st, int mode, int lstatic) {
+  typedef typename Cx<V>::type C;
+  const int m = blockIdx.x;
+  int L = lstatic;
+  double xi = 0.0, mu = 0.0;
+  const double2 *xa = nullptr;  // anchored stage: the anchor iterate x_a
+  if (st) {
+    if (st->done) return;
+    L = st->lcur;
+    xi = st->xi;
+    mu = filter_mu(*st, st->mu);
+    xa = st->xa;
+  }
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = blockDim.x >> 5;
+  const long a0 = alm_base(lmax, m);
+  const double wm = (m == 0) ? 1.0 : 2.0;
+  double num = 0.0, den = 0.0, dx = 0.0;
+
+  if (m <= L) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int J = (L - m) / 2 + 1, nb = (J + CKJ - 1) / CKJ, J16 = nb * CKJ;
+    const int tile = min(npairs, PANA_TILE);
+    Quad<V> *sp = reinterpret_cast<Quad<V> *>(smraw);                 // [tile]
+    Quad<V> *sd = sp + tile;                                          // [J16]
+    Pair<V> *srb = reinterpret_cast<Pair<V> *>(sd + J16);             // [J16]
+    Pair<V> *src_ = srb + J16;                                        // [J16]
+    const long q0 = pair_base(lmax, m), cb = block_base(lmax, m);
+    for (int j = tid; j < J16; j += blockDim.x) {
+      const Pair<V> zero = {(V)0, (V)0};
+      srb[j] = j < J ? reinterpret_cast<const Pair<V> *>(t.rec_b)[q0 + j] : zero;
+      src_[j] = j < J ? reinterpret_cast<const Pair<V> *>(t.rec_c)[q0 + j] : zero;
+    }
+    const long stride = lmax + 1;
+    for (int t0 = 0; t0 < npairs; t0 += PANA_TILE) {
+      const int nt = min(PANA_TILE, npairs - t0);
+      __syncthreads();  // the previous tile's reads are done
+      for (int k = tid; k < nt; k += blockDim.x) {
+        const int kk = t0 + k;
+        const C gn = G[kk * stride + m];
+        C gs = {};
+        if (kk < npairs - 1) gs = G[(2 * npairs - 2 - kk) * stride + m];
+        const V z = t.z[kk];
+        sp[k] = {gn.x + gs.x, gn.y + gs.y, z * (gn.x - gs.x), z * (gn.y - gs.y)};
+      }
+      __syncthreads();
+      for (int b = warp; b < nb; b += nwarps) {
+        const int j0 = b * CKJ;
+        V v[4 * CKJ];
+#pragma unroll
+        for (int i = 0; i < 4 * CKJ; ++i) v[i] = (V)0;
+        for (int g = 0; g < nt; g += 32) {
+          const int k = t0 + g + lane;
+          int js = INT_MAX / 2;
+          if (g + lane < nt) js = t.js[(long)m * npairs + k];
+          const bool on = js < j0 + CKJ;
+          if (!__any_sync(0xffffffffu, on)) continue;
+          const bool polar = t0 + g < t.kpol;
+          const Pair<V> *sr = (polar ? src_ : srb) + j0;
+          C c = {};
+          V w = (V)0;
+          Quad<V> p = {(V)0, (V)0, (V)0, (V)0};
+          if (on) {
+            c = t.ck[(cb + b) * npairs + k];
+            w = t.w[polar ? npairs + k : k];
+            p = sp[g + lane];
+          }
+          const bool inj = on && js >= j0;
+          if (__any_sync(0xffffffffu, inj || !on)) {
+            const V s1 = inj ? (V)0 : c.x, s2 = inj ? (V)0 : c.y;
+            pair_block<V, true>(v, sr, w, s1, s2, p, inj ? js - j0 : -2, c.x, c.y);
+          } else {
+            pair_block<V, false>(v, sr, w, c.x, c.y, p, 0, c.x, c.y);
+          }
+        }
+        V *d = reinterpret_cast<V *>(sd) + 4 * j0 + lane;
+        const V lo = lane_sums(v, lane), hi = lane_sums(v + 32, lane);
+        d[0] = t0 ? d[0] + lo : lo;
+        d[32] = t0 ? d[32] + hi : hi;
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i <= L - m; i += blockDim.x) {
+      const int j = i >> 1;
+      V sr, si;
+      if (i & 1) {
+        const V f = t.so[q0 + j];
+        sr = f * sd[j].c;
+        si = f * sd[j].d;
+      } else {
+        const V f = t.se[q0 + j];
+        sr = f * sd[j].a;
+        si = f * sd[j].b;
+        if (j > 0) {
+          const V g = t.sn[q0 + j - 1];
+          sr = fmav(g, sd[j - 1].a, sr);
+          si = fmav(g, sd[j - 1].b, si);
+        }
+      }
+      pair_finish(a0 + i, m + i, omega * sr, omega * si, wm, mode, cl, omega, xi, mu, src, xa, x,
+                  num, den, dx);
+    }
+  }
+  // coefficients of this m above the band are zero
+  for (int l = max(m, L + 1) + tid; l <= lmax; l += blockDim.x) {
+    const long i = a0 + (l - m);
+    if (mode == ANA_FILTER) {
+      const double2 old = x[i];
+      num += wm * (old.x * old.x + old.y * old.y);
+    }
+    x[i] = make_double2(0.0, 0.0);
+  }
+  if (mode == ANA_FILTER) pair_partials(num, den, dx, m, lmax, partials);
+}
+
+// ------------------------------------------------------------- launch
+static size_t synth_smem(size_t v, int lmax) { return 6 * v * (lmax / 2 + 1); }
+static size_t anal_smem(size_t v, int npairs, int lmax) {
+  const size_t j16 = (size_t)(lmax / 32 + 1) * CKJ;
+  return 4 * v * std::min(npairs, PANA_TILE) + 8 * v * j16;
+}
+
+template <int NP>
+static void synth64(const Plan &P, const double2 *x, double2 *F, const SolverState *st,
+                    int lstatic, int threads) {
+  const dim3 grid((P.npairs + threads * NP - 1) / (threads * NP), P.lmax + 1);
+  k_pair_synth<double, NP><<<grid, threads, synth_smem(8, P.lmax), P.stream>>>(
+      P.pt64, P.npairs, P.lmax, x, F, st, lstatic);
+}
+
+template <>
+wf_status launch_legendre_synth<double2>(const Plan &P, const double2 *x, double2 *F,
+                                         const SolverState *st, int lstatic) {
+  ++P.nlaunch;
+  // one or two warps per CTA: an SM's FP64 unit (2 lanes per clock) is full with a
+  // few warps, and small CTAs spread small maps over the SMs
+  const int threads = (long)P.npairs * (P.lmax + 1) <= 64L * 4 * P.num_sms ? 32 : PSYN_THREADS;
+  switch (P.syn_np[0]) {
+    case 2: synth64<2>(P, x, F, st, lstatic, threads); break;
+    case 4: synth64<4>(P, x, F, st, lstatic, threads); break;
+    default: synth64<1>(P, x, F, st, lstatic, threads); break;
+  }
+  WF_CUDA(cudaGetLastError());
+  return WF_OK;
+}
+
+template <>
+wf_status launch_legendre_anal<double2>(const Plan &P, const double2 *G, double2 *x,
+                                        const SolverState *st, int mode, int lstatic,
+                                        const double2 *src, double2 *) {
+  ++P.nlaunch;
+  const int warps = std::max(2, std::min(PANA_MAXWARPS, P.lmax / 32 + 1));
+  k_pair_anal<double><<<P.lmax + 1, 32 * warps, anal_smem(8, P.npairs, P.lmax), P.stream>>>(
+      P.pt64, P.npairs, P.lmax, P.cl_d, P.omega, G, x, P.partials, src, st, mode,
+      lstatic);
+  WF_CUDA(cudaGetLastError());
+  return WF_OK;
+}
+
+wf_status init_pair_attributes() {
+  const int big = 220 * 1024;
+  WF_CUDA(cudaFuncSetAttribute(k_pair_synth<double, 1>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  WF_CUDA(cudaFuncSetAttribute(k_pair_synth<double, 2>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  WF_CUDA(cudaFuncSetAttribute(k_pair_synth<double, 4>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  WF_CUDA(cudaFuncSetAttribute(k_pair_anal<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               big));
+  return WF_OK;
+}
+
+// ------------------------------------------------------------- tables
+// s of every (m, pair): a walk from lam_mm (mantissa, exponent) in scaled FP64
+// until |Q_j| reaches 2^-100, then plainly to the last j, leaving the seeds and
+// the state before each block.
+__global__ void k_pair_walk(int npairs, int lmax, int kpol, const double *__restrict__ w64,
+                            const double2 *__restrict__ rec_b,
+                            const double2 *__restrict__ rec_c, const double *__restrict__ so,
+                            const double *__restrict__ mant, const int *__restrict__ expo,
+                            int *__restrict__ js_out, double2 *__restrict__ ck) {
+  const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (long)npairs * (lmax + 1)) return;
+  const int m = (int)(t / npairs), k = (int)(t % npairs);
+  const int J = (lmax - m) / 2 + 1;
+  const long q0 = pair_base(lmax, m), cb = block_base(lmax, m);
+  const double2 *rec = (k < kpol ? rec_c : rec_b) + q0;
+  const double w = w64[k < kpol ? npairs + k : k];
+  double v = mant[t] * sqrt(2.0 * m + 3.0), vp = 0.0;  // Q_0 = lam_mm / eps_{m+1}
+  int e = expo[t], j = 0;                              // value v 2^e
+  bool found = false;
+  for (;;) {
+    const double a = fabs(v * so[q0 + j]);
+    if (e == 0 ? a >= 0x1p-100 : (e == -200 && a >= 0x1p+100)) {
+      found = true;
+      break;
+    }
+    if (j == J - 1) break;
+    ++j;
+    const double2 r = rec[j];
+    const double vn = fma(fma(r.x, w, r.y), v, vp);
+    vp = v;
+    v = vn;
+    if (e < 0 && fabs(v) > 0x1p+200) {
+      v *= 0x1p-200;
+      vp *= 0x1p-200;
+      e += 200;
+    }
+  }
+  js_out[t] = found ? j : INT_MAX / 2;
+  if (!found) return;
+  double s1 = ldexp(v, e), s2 = ldexp(vp, e);
+  {
+    double nx = 0.0;
+    if (j + 1 < J) {
+      const double2 r = rec[j + 1];
+      nx = fma(fma(r.x, w, r.y), s1, s2);
+    }
+    ck[(cb + (j >> 4)) * npairs + k] = make_double2(s1, nx);
+  }
+  for (;;) {
+    if ((j & 15) == 15 && j + 1 < J) ck[(cb + (j >> 4) + 1) * npairs + k] = make_double2(s1, s2);
+    if (++j >= J) break;
+    const double2 r = rec[j];
+    const double s = fma(fma(r.x, w, r.y), s1, s2);
+    s2 = s1;
+    s1 = s;
+  }
+}
+
+// double-double on the device, for the coefficient tables only: their errors
+// would add up along j
+struct d2 {
+  double h, l;
+};
+__device__ __forceinline__ d2 d2_norm(double s, double e) {
+  const double h = __dadd_rn(s, e);
+  return {h, __dsub_rn(e, __dsub_rn(h, s))};
+}
+__device__ __forceinline__ d2 d2_mul(d2 a, d2 b) {
+  const double p = __dmul_rn(a.h, b.h);
+  return d2_norm(p, fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
+}
+__device__ __forceinline__ d2 d2_div(d2 a, d2 b) {
+  const double q = a.h / b.h;
+  const d2 p = d2_mul({q, 0.0}, b);
+  return d2_norm(q, ((a.h - p.h) - p.l + a.l) / b.h);
+}
+__device__ __forceinline__ d2 d2_sqrt(d2 a) {
+  const double r = sqrt(a.h);
+  const double p = __dmul_rn(r, r);
+  return d2_norm(r, ((a.h - p) - fma(r, r, -p) + a.l) / (2.0 * r));
+}
+__device__ __forceinline__ d2 d2_add(d2 a, d2 b) {  // |a| >= |b|
+  const double s = __dadd_rn(a.h, b.h);
+  return d2_norm(s, (b.h - (s - a.h)) + (a.l + b.l));
+}
+// eps_l^2 = (l - m) (l + m) / ((2 l - 1) (2 l + 1)); the integers are exact
+__device__ __forceinline__ d2 eps2(double l, int m) {
+  return d2_div({(l - m) * (l + m), 0.0}, {(2.0 * l - 1.0) * (2.0 * l + 1.0), 0.0});
+}
+
+// One thread per m.  Pair basis: with up_j = eps_{l+1} eps_{l+2} (l = m + 2j + 1),
+// h_{j+1} = h_{j-1} up_{j-1} / up_j and A = h_j / (h_{j+1} up_j).  One-step
+// recurrence (equator): lam = g u, g_l = g_{l-2} eps_{l-1} / eps_l,
+// u_l = c_l z u_{l-1} - u_{l-2}, c_l = g_{l-1} / (g_l eps_l), sign-folded
+// likewise (signs (-1)^floor((l - m) / 2)).
+__global__ void k_pair_coefs(int lmax, PairTab<double> t) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m > lmax) return;
+  const long q0 = pair_base(lmax, m);
+  const int J = (lmax - m) / 2 + 1;
+  const d2 one = {1.0, 0.0};
+  d2 h0 = one, h1 = one, up0 = one;             // h_{j-1}, h_j, up_{j-1}
+  d2 e_l = eps2(m + 1.0, m), r_l = d2_sqrt(e_l);  // eps^2 and eps of l = m + 2j + 1
+  d2 g0 = one, g1 = one, rm = one;              // g_{2j-1}, g_{2j}, eps_{m+2j}
+  for (int j = 0; j < J; ++j) {
+    const double l = m + 2.0 * j + 1.0;
+    const double fold = ((j >> 1) & 1) ? -1.0 : 1.0;
+    const d2 e1 = eps2(l + 1.0, m), e2 = eps2(l + 2.0, m);
+    const d2 r1 = d2_sqrt(e1), r2 = d2_sqrt(e2);
+    t.se[q0 + j] = fold * d2_mul(h1, r_l).h;
+    t.sn[q0 + j] = fold * d2_mul(h1, r1).h;
+    t.so[q0 + j] = fold * h1.h;
+    const d2 up = d2_mul(r1, r2);
+    const d2 hn = j == 0 ? one : d2_div(d2_mul(h0, up0), up);
+    if (j == 0) t.rec_b[q0] = t.rec_c[q0] = make_double2(0.0, 0.0);
+    if (j + 1 < J) {
+      const double sg = (j & 1) ? -1.0 : 1.0;
+      const d2 A = d2_div(h1, d2_mul(hn, up));
+      const d2 e = e_l.h > e1.h ? d2_add(e_l, e1) : d2_add(e1, e_l);
+      const d2 B = d2_mul(A, e), C = d2_mul(A, d2_add(one, {-e.h, -e.l}));
+      t.rec_b[q0 + j + 1] = make_double2(sg * A.h, -sg * B.h);
+      t.rec_c[q0 + j + 1] = make_double2(sg * A.h, sg * C.h);
+    }
+    // one-step: l - m = 2 j (g1, c0 from the last j) and 2 j + 1
+    const double f2 = (j & 1) ? -1.0 : 1.0;
+    const d2 go = j == 0 ? one : d2_div(d2_mul(g0, rm), r_l);  // g_{2j+1}
+    t.ge[q0 + j] = f2 * g1.h;
+    t.go[q0 + j] = f2 * go.h;
+    t.rec_e[q0 + j].y = d2_div(g1, d2_mul(go, r_l)).h;
+    if (j == 0) t.rec_e[q0].x = 0.0;
+    const d2 ge = d2_div(d2_mul(g1, r_l), r1);                 // g_{2j+2}
+    if (j + 1 < J) t.rec_e[q0 + j + 1].x = -d2_div(go, d2_mul(ge, r1)).h;
+    g0 = go;
+    g1 = ge;
+    rm = r1;
+    h0 = h1;
+    h1 = hn;
+    up0 = up;
+    e_l = e2;
+    r_l = r2;
+  }
+}
+
+// lam_mm of the pairs from keq on (mantissa and exponent 0 there)
+__global__ void k_pair_lmm(int npairs, int lmax, int keq, const double *__restrict__ mant,
+                           const int *__restrict__ expo, double *__restrict__ lmm) {
+  const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int n = npairs - keq;
+  if (t >= (long)n * (lmax + 1)) return;
+  const long i = t / n * npairs + keq + t % n;
+  lmm[i] = ldexp(mant[i], expo[i]);
+}
+
+// The tables and the checkpoints.  mant, expo: lam_mm of every (m, pair).
+wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
+  const int lmax = P.lmax;
+  const long nq = pair_base(lmax, lmax) + 1;
+  const long nb = block_base(lmax, lmax) + 1;
+  std::vector<double> w(2 * (size_t)P.npairs), z(P.npairs);
+  // rings with z > 0.7 use the polar form, in whole warps of pairs
+  int np = 0;
+  for (int k = 0; k < P.npairs; ++k) {
+    z[k] = P.pairs_h[k].z;
+    if (z[k] > 0.7) np = k + 1;
+  }
+  const int kpol = (np / 32) * 32;
+  for (int k = 0; k < P.npairs; ++k) {
+    w[k] = z[k] * z[k];
+    w[P.npairs + k] = -(1.0 - z[k]) * (1.0 + z[k]);
+  }
+  auto up = [](auto **dst, const auto &v) {
+    WF_CUDA(cudaMalloc(dst, sizeof(v[0]) * v.size()));
+    WF_CUDA(cudaMemcpy(*dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice));
+    return WF_OK;
+  };
+  // the equatorial pairs, in whole CTAs of the synthesis
+  int keq = P.npairs;
+  while (keq > 0 && z[keq - 1] < 0.2 && lmax * log2(P.pairs_h[keq - 1].sth) > -90.0) --keq;
+  keq = (keq + PSYN_THREADS - 1) / PSYN_THREADS * PSYN_THREADS;
+  PairTab<double> &t = P.pt64;
+  t.kpol = kpol;
+  t.keq = keq;
+  WF_TRY(up(&t.w, w));
+  WF_TRY(up(&t.z, z));
+  for (double2 **a : {&t.rec_b, &t.rec_c, &t.rec_e})
+    WF_CUDA(cudaMalloc(a, sizeof(double2) * nq));
+  for (double **a : {&t.se, &t.sn, &t.so, &t.ge, &t.go})
+    WF_CUDA(cudaMalloc(a, sizeof(double) * nq));
+  k_pair_coefs<<<(lmax + 32) / 32, 32, 0, P.stream>>>(lmax, t);
+  WF_CUDA(cudaGetLastError());
+  if (keq < P.npairs) {
+    const long ne = (long)(P.npairs - keq) * (lmax + 1);
+    WF_CUDA(cudaMalloc(&t.lmm, sizeof(double) * (size_t)P.npairs * (lmax + 1)));
+    k_pair_lmm<<<(unsigned)((ne + 255) / 256), 256, 0, P.stream>>>(P.npairs, lmax, keq, mant,
+                                                                   expo, t.lmm);
+    WF_CUDA(cudaGetLastError());
+  }
+  const long n = (long)P.npairs * (lmax + 1);
+  WF_CUDA(cudaMalloc(&t.js, sizeof(int) * n));
+  WF_CUDA(cudaMalloc(&t.ck, sizeof(double2) * nb * P.npairs));
+  k_pair_walk<<<(unsigned)((n + 127) / 128), 128, 0, P.stream>>>(
+      P.npairs, lmax, kpol, t.w, t.rec_b, t.rec_c, t.so, mant, expo, t.js, t.ck);
+  WF_CUDA(cudaGetLastError());
+  return WF_OK;
+}
+
+void free_pair_tables(Plan &P) {
+  PairTab<double> &t = P.pt64;
+  void *b[] = {t.rec_b, t.rec_c, t.rec_e, t.se, t.sn, t.so, t.ge, t.go, t.w, t.z, t.lmm, t.js,
+               t.ck};
+  for (void *p : b)
+    if (p) cudaFree(p);
+}
+
+}  // namespace wf

@@ -170,8 +170,7 @@ wf_status residual_static(Plan &P, const double *d, const double *alm, double *r
                             cudaMemcpyHostToDevice, P.stream));
     WF_CUDA(cudaMemcpyAsync(P.xtmp, x, sizeof(double2) * P.nalm, cudaMemcpyDeviceToDevice,
                             P.stream));
-    WF_TRY(launch_prescale<double2>(P, x, P.xs64));
-    WF_TRY(launch_legendre_synth<double2>(P, P.xs64, P.F64, nullptr, P.lmax));
+    WF_TRY(launch_legendre_synth<double2>(P, x, P.F64, nullptr, P.lmax));
     WF_TRY(launch_ring<double2>(P, RING_FUSED, P.F64, P.G64, P.dmap, nullptr, P.state,
                                 P.lmax));
     WF_TRY(launch_legendre_anal<double2>(P, P.G64, P.xtmp, P.state, ANA_FILTER, P.lmax));

@@ -362,6 +362,10 @@ __global__ void k_seed_walk(const RingPair *pairs, int npairs, int lmax,
 }
 
 static wf_status make_seeds(Plan &P) {
+  int dev = 0;
+  WF_CUDA(cudaGetDevice(&dev));
+  P.device = dev;
+  WF_CUDA(cudaDeviceGetAttribute(&P.num_sms, cudaDevAttrMultiProcessorCount, dev));
   const long n = (long)P.npairs * (P.lmax + 1);
   double *mant = nullptr;
   int *expo = nullptr;
@@ -376,6 +380,7 @@ static wf_status make_seeds(Plan &P) {
   k_seed_walk<<<(unsigned)((n + 255) / 256), 256, 0, P.stream>>>(
       P.pairs, P.npairs, P.lmax, mant, expo, P.rg, P.seed_l, P.seed_u, P.seed_s32);
   WF_CUDA(cudaGetLastError());
+  WF_TRY(build_pair_tables(P, mant, expo));
   WF_CUDA(cudaStreamSynchronize(P.stream));
   WF_CUDA(cudaFree(mant));
   WF_CUDA(cudaFree(expo));
@@ -384,6 +389,7 @@ static wf_status make_seeds(Plan &P) {
 
 wf_status build_tables(Plan &P) {
   WF_TRY(init_legendre_attributes());
+  WF_TRY(init_pair_attributes());
   WF_TRY(init_ring_attributes());
   make_pairs(P);
   WF_TRY(make_fft_tables(P));

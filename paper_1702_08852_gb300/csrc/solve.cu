@@ -307,8 +307,7 @@ wf_status alm_dot_host(Plan &P, const double2 *a, const double2 *b, double *res)
 // ---------------------------------------------------------------- transforms
 wf_status alm2map(Plan &P, const double *alm, double *map) {
   const double2 *a = reinterpret_cast<const double2 *>(alm);
-  WF_TRY(launch_prescale<double2>(P, a, P.xs64));
-  WF_TRY(launch_legendre_synth<double2>(P, P.xs64, P.F64, nullptr, P.lmax));
+  WF_TRY(launch_legendre_synth<double2>(P, a, P.F64, nullptr, P.lmax));
   WF_TRY(launch_ring<double2>(P, RING_SYNTH, P.F64, nullptr, nullptr, map, nullptr,
                               P.lmax));
   return WF_OK;
@@ -429,7 +428,7 @@ SolverState initial_state(const Plan &P) {
 
 template <typename T2> struct Scaled;
 template <> struct Scaled<double2> {
-  static double2 *get(Plan &P) { return P.xs64; }
+  static double2 *get(Plan &P) { return P.x; }  // read as it is
 };
 template <> struct Scaled<float2> {
   static float2 *get(Plan &P) { return P.xs32; }
@@ -652,10 +651,7 @@ static wf_status fp64_step(Plan &P, const double2 *x, double2 *gx, double *num,
                           cudaMemcpyHostToDevice, P.stream));
   WF_CUDA(cudaMemcpyAsync(gx, x, sizeof(double2) * P.nalm, cudaMemcpyDeviceToDevice,
                           P.stream));
-  if (dd)
-    WF_TRY(launch_prescale_dd(P, x, dd_view(P.xs64)));
-  else
-    WF_TRY(launch_prescale<double2>(P, x, P.xs64));
+  if (dd) WF_TRY(launch_prescale_dd(P, x, dd_view(P.xs64)));
   // opts.timing: events around the double-float synthesis, ring step and
   // analysis (kernels 3, 5, 4 of wf_kernel_stats)
   const bool timed = dd && P.opts.timing;
@@ -666,7 +662,7 @@ static wf_status fp64_step(Plan &P, const double2 *x, double2 *gx, double *num,
     WF_TRY(launch_legendre_synth_dd(P, dd_view(P.xs64), dd_view(P.F64), nullptr,
                                     std::max(L, 0)));
   else
-    WF_TRY(launch_legendre_synth<double2>(P, P.xs64, P.F64, nullptr, std::max(L, 0)));
+    WF_TRY(launch_legendre_synth<double2>(P, x, P.F64, nullptr, std::max(L, 0)));
   if (timed) WF_CUDA(cudaEventRecord(P.dd_ev[1], P.stream));
   if (dd)
     WF_TRY(launch_ring_dd(P, RING_FUSED, dd_view(P.F64), dd_view(P.G64), nullptr, nullptr,
@@ -1258,8 +1254,7 @@ wf_status residual(Plan &P, const double *d, const double *alm, double *res_wf,
                       P.stream);
       cudaMemcpyAsync(P.xtmp, x, sizeof(double2) * P.nalm, cudaMemcpyDeviceToDevice,
                       P.stream);
-      if ((status = launch_prescale<double2>(P, x, P.xs64)) != WF_OK) break;
-      if ((status = launch_legendre_synth<double2>(P, P.xs64, P.F64, nullptr, P.lmax)) !=
+      if ((status = launch_legendre_synth<double2>(P, x, P.F64, nullptr, P.lmax)) !=
           WF_OK)
         break;
       if ((status = launch_ring<double2>(P, RING_FUSED, P.F64, P.G64, P.dmap, nullptr,

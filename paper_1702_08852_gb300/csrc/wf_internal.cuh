@@ -44,6 +44,26 @@ struct Tab32 {
   const float *cl;
 };
 
+// Tables of the Legendre kernels in the parity-pair basis (legpair.cu), V the
+// arithmetic; indexed by (m, j) except where noted
+template <typename V> struct PairVec;
+template <> struct PairVec<double> { typedef double2 type; };
+template <typename V>
+struct PairTab {
+  typename PairVec<V>::type *rec_b = nullptr, *rec_c = nullptr;  // (A, B), (A, A + B)
+  V *se = nullptr, *sn = nullptr, *so = nullptr;  // basis change, scales and signs included
+  V *w = nullptr;                                 // [2][npairs]: z^2, -sin^2 theta
+  V *z = nullptr;                                 // [npairs]
+  int *js = nullptr;                              // [lmax+1][npairs] first j, |Q_j| >= 2^-100
+  typename PairVec<V>::type *ck = nullptr;        // [block of 16 j of m][npairs]
+  int kpol = 0;                                   // pairs below it: the polar form
+  // the pairs k >= keq in the synthesis: the one-step recurrence's coefficients
+  // (l - m even, odd), its scales, and lam_mm [lmax+1][npairs]
+  int keq = 0;
+  typename PairVec<V>::type *rec_e = nullptr;
+  V *ge = nullptr, *go = nullptr, *lmm = nullptr;
+};
+
 struct RingPair {
   double z;        // z of the north ring
   double sth;      // sin(theta) of the north ring
@@ -150,6 +170,7 @@ struct Plan {
   // geometry / Legendre tables
   RingPair *pairs = nullptr;     // [npairs]
   double *cl_d = nullptr;        // [lmax+1]
+  PairTab<double> pt64;          // parity-pair basis, FP64
   double *rc = nullptr;          // [nalm] recurrence coefficient c_lm
   double *rg = nullptr;          // [nalm] scale g_lm (lambda = g u)
   float *rc32 = nullptr;         // [nalm] FP32 copy of rc
@@ -167,7 +188,7 @@ struct Plan {
 
   // launch variants (ring pairs per thread), [0] = FP64, [1] = FP32; set by
   // the autotuner (opts.autotune) or the defaults below
-  int syn_np[2] = {2, 2};
+  int syn_np[2] = {1, 2};
   int ana_np[2] = {4, 8};
   // FP32 analysis scheduling: 0 = one CTA per m, 1 = warps take (m, tile)
   // items from a queue and a combine kernel sums the tiles (ana_scratch)
@@ -215,7 +236,7 @@ struct Plan {
   double2 *x = nullptr;          // [nalm] current iterate
   double2 *xtmp = nullptr;       // [nalm]
   double2 *xacc = nullptr;       // [nalm] refined solution (mixed precision)
-  double2 *xs64 = nullptr;       // [nalm] g_lm x_lm, synthesis input (FP64)
+  double2 *xs64 = nullptr;       // [nalm] g_lm x_lm as double-float pairs, synthesis input
   float2 *xs32 = nullptr;        // [nalm] g_lm x_lm, synthesis input (FP32)
   double2 *src = nullptr;        // [nalm] harmonic source of a correction solve
   // mixed solver, stage boundaries between anchored stages: the unfiltered
@@ -275,8 +296,8 @@ struct Plan {
 // Legendre transforms (legendre.cu).  Modes of the analysis:
 enum AnalysisMode { ANA_PLAIN = 0, ANA_FILTER = 1 };
 
-// The synthesis reads xs = g_lm a_lm in its own precision (written by the
-// analysis of the previous iteration, or by launch_prescale).
+// The FP32 synthesis reads xs = g_lm a_lm (written by the analysis of the previous
+// iteration, or by launch_prescale), the FP64 one the coefficients themselves.
 template <typename T2>
 wf_status launch_prescale(const Plan &P, const double2 *x, T2 *xs);
 template <typename T2>
@@ -284,11 +305,16 @@ wf_status launch_legendre_synth(const Plan &P, const T2 *xs, T2 *F,
                                 const SolverState *st, int lstatic);
 // src (optional, FP64 alm): adds the harmonic source f_l xi Omega src_lm of an
 // anchored stage to the filtered coefficients (ANA_FILTER only).
-// xs_out (optional): also write g_lm a_lm in the transform precision.
+// xs_out (optional, FP32): also write the synthesis input g_lm a_lm.
 template <typename T2>
 wf_status launch_legendre_anal(const Plan &P, const T2 *G, double2 *x,
                                const SolverState *st, int mode, int lstatic,
                                const double2 *src = nullptr, T2 *xs_out = nullptr);
+
+// tables and attributes of the parity-pair kernels (legpair.cu)
+wf_status init_pair_attributes();
+wf_status build_pair_tables(Plan &P, const double *mant, const int *expo);
+void free_pair_tables(Plan &P);
 
 // Double-float (pairs of FP32) Legendre transforms with FP64 inputs and
 // outputs, for the anchor steps of the mixed solver (legendre.cu): the same
