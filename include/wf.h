@@ -372,26 +372,18 @@ wf_status wf_kernel_stats(wf_plan_t plan, int kernel, double *ms, long *launches
                           double *gflop, int reset);
 
 /* Launch variants of the Legendre kernels in use by a plan, and the times
- * the autotuner measured for each candidate (opts.autotune = 1; a choice
- * cached for the geometry reports the timings it was made from; -1 where a
- * candidate was not timed, and everywhere with autotune = 0).
- * Index [0] = FP64 kernels, [1] = FP32 kernels.
- *  syn_np      ring pairs per thread of the synthesis.
- *  syn_packed  FP32 synthesis on packed f32x2 pairs of rings (1: syn_np 2, 4;
- *              2: syn_np 2 with duplicated shared-memory tables).
- *  ana_np      ring pairs per lane of the analysis.
- *  ana_queue   FP32 analysis scheduling: 0 = one CTA per m, 1 = warps take
- *              (m, tile) items from a queue, then a per-m combine kernel.
- *  ana_packed  FP32 per-m analysis on packed f32x2 pairs (ana_np 4, 6, 8).
- *  ana_global_acc  with ana_packed: the per-warp accumulators in global
- *              scratch instead of shared memory (more CTAs/SM); 1: ana_np 4,
- *              6 with 16-l chunks, 2: ana_np 4, 6, 8 with 8-l chunks, 3:
- *              ana_np 8 with 8-l chunks and the seeds in shared memory.
- *  syn_ms      candidates 1, 2, 4 pairs per thread, then (FP32) packed 2, 4
- *              and packed with duplicated tables 2: ms for two launches.
- *  ana_ms      candidates 2, 4, 8, 16 pairs per lane, then (FP32 only) queue
- *              4, 8, packed 4, 8, 6, packed with global accumulators 4, 6
- *              and the same with 8-l chunks 8, 6, 4 and with shared seeds 8:
+ * the autotuner measured (opts.autotune = 1; a choice cached for the geometry
+ * reports the timings it was made from; -1 where a candidate was not timed, and
+ * everywhere with autotune = 0).  Index [0] = FP64 kernels, [1] = FP32 kernels.
+ *  syn_np      ring pairs per thread of the synthesis (FP32 with 2 or 4: on
+ *              packed f32x2 pairs of rings).
+ *  syn_packed, ana_np, ana_queue, ana_packed, ana_global_acc
+ *              kept for callers that set them: the analysis is one kernel (a
+ *              warp per 16 recurrence steps of one m over all rings), and these
+ *              fields are checked, stored and reported but select nothing.
+ *  syn_ms      candidates 1, 2, 4 pairs per thread, then (FP32) 2, 4 and 2
+ *              again: ms for two launches.
+ *  ana_ms      the analysis, the same figure in slots 0 .. 2 (FP32: 0 .. 14):
  *              ms for two launches. */
 typedef struct {
   int syn_np[2], syn_packed, ana_np[2], ana_queue, ana_packed, ana_global_acc;

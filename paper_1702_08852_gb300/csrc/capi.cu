@@ -31,14 +31,14 @@ static void free_plan(wf_plan_s *P) {
   free_pair_tables(*P);
   for (int i = 0; i < 3; ++i)
     if (P->graph[i]) cudaGraphExecDestroy(P->graph[i]);
-  void *bufs[] = {P->pairs, P->cl_d,   P->rc,      P->rg,     P->rc32,   P->seed_l,
+  void *bufs[] = {P->pairs, P->cl_d,   P->rc,      P->rg,     P->seed_l,
                   P->seed_u, P->tw64,  P->tw32,    P->chirp64, P->chirp32, P->bhat64,
                   P->bhat32, P->nvar,  P->F64,     P->G64,    P->F32,    P->G32,
                   P->x,      P->xtmp,  P->dmap,    P->mtmp,   P->partials, P->red,
                   P->state,  P->trace, P->xacc,  P->src, P->xs64, P->xs32,
                   P->nvar32, P->dmap32, P->ana_scratch, P->ana_lstart,
                   P->ana_counter, P->uacc[0], P->uacc[1],
-                  P->seed_s32, P->zs32, P->rg32, P->cl32, P->twdd, P->chirpdd, P->bhatdd,
+                  P->cl32, P->twdd, P->chirpdd, P->bhatdd,
                   P->phasedd, P->rcdd, P->nvardd, P->dmapdd};
   for (void *b : bufs)
     if (b) cudaFree(b);
@@ -59,7 +59,7 @@ static wf_status alloc_work(Plan &P) {
   WF_CUDA(cudaStreamCreateWithFlags(&P.side_stream, cudaStreamNonBlocking));
   WF_CUDA(cudaEventCreateWithFlags(&P.fork_ev, cudaEventDisableTiming));
   WF_CUDA(cudaEventCreateWithFlags(&P.join_ev, cudaEventDisableTiming));
-  const size_t nF = (size_t)P.nring * (P.lmax + 1);
+  const size_t nF = 2 * (size_t)P.npairs * (P.lmax + 1);
   WF_CUDA(cudaMalloc(&P.F64, sizeof(double2) * nF));
   WF_CUDA(cudaMalloc(&P.G64, sizeof(double2) * nF));
   WF_CUDA(cudaMalloc(&P.F32, sizeof(float2) * nF));

@@ -1,8 +1,10 @@
 // legpair.cu -- associated-Legendre synthesis and analysis in the parity-pair
 // basis, with the recurrence restarted from a table of checkpoints.
 //
-// Ring pair k is the north ring k and, but for the equator (k = npairs - 1), the
-// south ring 2 npairs - 2 - k.
+// F and G hold the two rings of a pair side by side, [m][pair][north, south]: the
+// lanes of a warp (one pair each) read and write whole lines, and the ring kernels
+// touch one (north, south) element per m.  The equator (the last pair) has no south
+// ring.
 //
 // Basis (Ishioka 2018, J. Meteor. Soc. Japan 96, "A new recurrence formula for
 // efficient computation of spherical harmonic transform").  With
@@ -15,10 +17,12 @@
 //                                 - eps_l eps_{l-1} Q_{j-1},   l = m + 2 j + 1.
 // Scaled and sign-folded, Q_j = h_j s_j with h_0 = h_1 = 1 and
 //   s_j = (A_j w + B_j) s_{j-1} + s_{j-2}
-// (tables indexed by the j they produce).  w = z^2 with B, or, for the ring
-// pairs k < kpol near the pole, w = -sin^2 theta with C = A + B in B's place:
-// that form keeps the small angle there (z^2 rounds it away).  The two forms
-// are equal; each CTA or warp takes the one of the pairs it holds.
+// (tables indexed by the j they produce) with w = z^2 - w0 and B_j taken at w0:
+// three equal forms, w0 = 1, 1/2 and 0, for the pairs below kform[0] (near the
+// pole, where -sin^2 theta keeps the small angle that z^2 rounds away), below
+// kform[1], and the others.  Each keeps |B| at or below the size of the sum, so
+// that rounding B does not add to the phase; a CTA or warp takes the form of the
+// pairs it holds.
 //
 // Per (m, ring pair) and j this costs 2 multiply-adds for the recurrence and 4
 // for the two complex sums, 3 per (l, m, pair) term; the one-step recurrence in
@@ -38,14 +42,20 @@
 // (3.14e9 terms) the synthesis takes 16.6 ms (21.4 ms with the one-step recurrence)
 // and the analysis 16.9 ms (29.0 ms), against 15 ms for 3 multiply-adds per term at
 // the unit's measured 1.25 TFLOP/s; at Nside 150, lmax 311, 0.106 and 0.142 ms
-// (0.233 and 0.276 ms).
+// (0.233 and 0.276 ms).  FP32: the FMA pipe takes 6 clocks per warp and step, 0.26 ms
+// at Nside 1024; measured 0.435 ms (synthesis, from 0.645) and 0.597 ms (analysis,
+// from 0.891), at Nside 256 17.7 and 23 us (from 23 and 38): what is left is the
+// reductions, the loads between the blocks and, on small maps, the largest m's chain.
 //
-// Checkpoints: ck[(block b of 16 j of m)][pair] holds (s_{16b-1}, s_{16b-2}),
-// or, in the block where the pair's first |Q_j| >= 2^-100 lies (j = js), the two
-// seeds (s_js, s_js+1); terms below 2^-100 are dropped.  Any 16 j can therefore
-// be computed on their own: a warp of the analysis owns 16 j of one m, keeps
-// their 64 sums per lane in registers over all ring pairs, and reduces them
-// across the lanes once.
+// Checkpoints: ck[(block b of 16 j of m)][pair] holds (s_{16b-1}, s_{16b-2}), so any 16
+// j can be computed on their own: a warp of the analysis owns 16 j of one m, keeps
+// their 64 sums per lane in registers over all ring pairs, and reduces them across the
+// lanes once.  The terms start at the first |Q_j| >= 2^-100 (j = js); in the block that
+// holds js the checkpoint is, where the state before the block is out of the
+// arithmetic's range, the seeds (s_js, s_js+1) instead, which enter at j = js (jin).
+// FP64 always has that state; FP32 where it is above 2^-120, and a block that ends
+// below 2^-80 without it is left out (an FP32 sum does not see such terms beside the
+// O(1) ones).
 #include <limits.h>
 #include <math.h>
 
@@ -80,11 +90,24 @@ __device__ __forceinline__ long alm_base(int lmax, int m) {  // index of (m, m)
 // ------------------------------------------------------------- arithmetic
 template <typename V> struct Cx;  // complex element of F, G and the alm input
 template <> struct Cx<double> { typedef double2 type; };
+template <> struct Cx<float> { typedef float2 type; };
 template <typename V> struct alignas(16) Quad { V a, b, c, d; };
 template <typename V> struct alignas(2 * sizeof(V)) Pair { V a, b; };
 
 __device__ __forceinline__ double fmav(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ void accv(double &acc, double s, double x) { acc = fma(s, x, acc); }
+
+__device__ __forceinline__ float fmav(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ void accv(float &acc, float s, float x) { acc = fmaf(s, x, acc); }
+// (dx, dy) = (ax, ay) (bx, by) + (cx, cy): one packed instruction (f32x2), each half
+// rounded as the scalar one
+__device__ __forceinline__ void fma2(float &dx, float &dy, float ax, float ay, float bx, float by,
+                                     float cx, float cy) {
+  asm("{\n .reg .b64 ra, rb, rc, rd;\n mov.b64 ra, {%2, %3};\n mov.b64 rb, {%4, %5};\n"
+      " mov.b64 rc, {%6, %7};\n fma.rn.f32x2 rd, ra, rb, rc;\n mov.b64 {%0, %1}, rd;\n}"
+      : "=f"(dx), "=f"(dy)
+      : "f"(ax), "f"(ay), "f"(bx), "f"(by), "f"(cx), "f"(cy));
+}
 
 __device__ __forceinline__ int wmin(int v) { return __reduce_min_sync(0xffffffffu, v); }
 __device__ __forceinline__ int wmax(int v) { return __reduce_max_sync(0xffffffffu, v); }
@@ -109,14 +132,17 @@ __device__ __forceinline__ V lane_sums(V *v, int lane) {
 
 // ------------------------------------------------------------- synthesis
 // One thread per NP ring pairs of one m (grid: tiles of pairs x m), a
-// warp-uniform loop over j.  The CTA stages the m's coefficients in shared
+// warp-uniform loop over j.  FP32 with NP even runs two pairs per packed instruction
+// (f32x2); its shared-memory inputs hold every value twice, so that a packed operand
+// is one load.  The CTA stages the m's coefficients in shared
 // memory, combined to the pair basis on the way:
 //   E_j = se_j a_{m+2j} + sn_j a_{m+2j+2},   O_j = so_j a_{m+2j+1}.
 // F_north = sum_j s_j (E_j + z O_j), F_south the difference.
-constexpr int PSYN_THREADS = 64;
+constexpr int PSYN_THREADS = 64;     // FP64
+constexpr int PSYN_THREADS32 = 128;  // FP32
 
 template <typename V, int NP>
-__global__ void __launch_bounds__(PSYN_THREADS)
+__global__ void __launch_bounds__(PSYN_THREADS32)
     k_pair_synth(const PairTab<V> t, int npairs, int lmax,
                  const typename Cx<V>::type *__restrict__ x,
                  typename Cx<V>::type *__restrict__ F, const SolverState *__restrict__ st,
@@ -130,15 +156,21 @@ __global__ void __launch_bounds__(PSYN_THREADS)
   }
   if (m > L) return;  // the ring step ignores m above the band
   extern __shared__ __align__(16) unsigned char smraw[];
+  constexpr bool PK = std::is_same<V, float>::value && NP % 2 == 0;
   const int J = (L - m) / 2 + 1;
+  // per j a quad (E_re, E_im, O_re, O_im), or, PK, two: (E_re, E_re, E_im, E_im),
+  // (O_re, O_re, O_im, O_im); then the forms' (A, B), [NF][J]
   Quad<V> *sx = reinterpret_cast<Quad<V> *>(smraw);
-  Pair<V> *sr = reinterpret_cast<Pair<V> *>(smraw + sizeof(Quad<V>) * J);
+  Pair<V> *srec = reinterpret_cast<Pair<V> *>(smraw + sizeof(Quad<V>) * J * (PK ? 2 : 1));
   const int pair00 = blockIdx.x * blockDim.x * NP;
-  const bool polar = pair00 + (int)blockDim.x * NP / 2 <= t.kpol;
+  // FP32 CTAs span several forms: all three are staged and each warp takes its own;
+  // FP64 CTAs (at most 64 pairs) stage one
+  constexpr int NF = std::is_same<V, float>::value ? 3 : 1;
   const bool equator = t.rec_e && pair00 >= t.keq;
-  const V *wt = polar ? t.w + npairs : t.w;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int pair0 = pair00 + warp * 32 * NP;
+  const int form = t.form(NF == 1 ? pair00 + (int)blockDim.x / 2 - 1 : pair0 + 16 * NP - 1);
+  const V *wt = t.w + form * t.stride;
   V w[NP];
   int js[NP];
 #pragma unroll
@@ -148,13 +180,12 @@ __global__ void __launch_bounds__(PSYN_THREADS)
     js[i] = INT_MAX / 2;
     if (k < npairs) {
       w[i] = wt[k];
-      js[i] = t.js[(long)m * npairs + k];
+      js[i] = t.js[(long)m * t.stride + k];
     }
   }
   {
     const long q0 = pair_base(lmax, m), a0 = alm_base(lmax, m);
-    const Pair<V> *rec =
-        reinterpret_cast<const Pair<V> *>(equator ? t.rec_e : polar ? t.rec_c : t.rec_b);
+    const Pair<V> *rec = reinterpret_cast<const Pair<V> *>(equator ? t.rec_e : t.rec[form]);
     for (int j = threadIdx.x; j < J; j += blockDim.x) {
       const int l = m + 2 * j;
       const C c0 = x[a0 + 2 * j];
@@ -164,18 +195,32 @@ __global__ void __launch_bounds__(PSYN_THREADS)
       if (equator) {
         const V ge = t.ge[q0 + j], go = t.go[q0 + j];
         sx[j] = {ge * c0.x, ge * c0.y, go * c1.x, go * c1.y};
-        sr[j] = rec[q0 + j];
+        srec[j] = rec[q0 + j];
         continue;
       }
       const V se = t.se[q0 + j], sn = t.sn[q0 + j], so = t.so[q0 + j];
-      sx[j] = {fmav(se, c0.x, sn * c2.x), fmav(se, c0.y, sn * c2.y), so * c1.x, so * c1.y};
-      sr[j] = rec[q0 + j];
+      const V xr = fmav(se, c0.x, sn * c2.x), xi = fmav(se, c0.y, sn * c2.y);
+      const V yr = so * c1.x, yi = so * c1.y;
+      if constexpr (PK) {
+        sx[2 * j] = {xr, xr, xi, xi};
+        sx[2 * j + 1] = {yr, yr, yi, yi};
+      } else {
+        sx[j] = {xr, xi, yr, yi};
+      }
+      if constexpr (NF == 1) {
+        srec[j] = rec[q0 + j];
+      } else {
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+          srec[f * J + j] = reinterpret_cast<const Pair<V> *>(t.rec[f])[q0 + j];
+      }
     }
   }
   __syncthreads();
   if (pair0 >= npairs) return;
+  const Pair<V> *sr = srec + (NF == 1 ? 0 : form * J);
 
-  const long stride = lmax + 1;
+  Quad<V> *out = reinterpret_cast<Quad<V> *>(F) + (long)m * npairs;
   if (equator) {
     V z[NP], u[NP], o[NP], er[NP], ei[NP], orr[NP], oi[NP];
 #pragma unroll
@@ -205,22 +250,19 @@ __global__ void __launch_bounds__(PSYN_THREADS)
     for (int i = 0; i < NP; ++i) {
       const int k = pair0 + lane + 32 * i;
       if (k >= npairs) continue;
-      F[k * stride + m] = {er[i] + orr[i], ei[i] + oi[i]};
-      if (k < npairs - 1)
-        F[(2 * npairs - 2 - k) * stride + m] = {er[i] - orr[i], ei[i] - oi[i]};
+      out[k] = {er[i] + orr[i], ei[i] + oi[i], er[i] - orr[i], ei[i] - oi[i]};
     }
     return;
   }
 
   V s1[NP], s2[NP], d0[NP], d1[NP], er[NP], ei[NP], orr[NP], oi[NP];
   int jmin = INT_MAX, jinj = -1;
-  const long cb = block_base(lmax, m);
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
     const int k = pair0 + lane + 32 * i;
     s1[i] = s2[i] = d0[i] = d1[i] = er[i] = ei[i] = orr[i] = oi[i] = (V)0;
     if (js[i] < J) {
-      const C s = t.ck[(cb + (js[i] >> 4)) * npairs + k];
+      const C s = t.seed[(long)m * t.stride + k];
       d0[i] = s.x;
       d1[i] = s.y;
       jmin = min(jmin, js[i]);
@@ -230,44 +272,63 @@ __global__ void __launch_bounds__(PSYN_THREADS)
   jmin = wmin(jmin);
   jinj = min(wmax(jinj), J - 1);
   int j = jmin;
-  for (; j <= jinj; ++j) {  // seeds may still enter
-    const Pair<V> r = sr[j];
-    const Quad<V> q = sx[j];
+  if constexpr (PK) {
+    auto step = [&](int jj, bool inj) {
+      const Pair<V> r = sr[jj];
+      const Quad<V> xe = sx[2 * jj], xo = sx[2 * jj + 1];
 #pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      V s = fmav(fmav(r.a, w[i], r.b), s1[i], s2[i]);
-      s = j == js[i] ? d0[i] : s;
-      s = j == js[i] + 1 ? d1[i] : s;
-      s2[i] = s1[i];
-      s1[i] = s;
-      accv(er[i], s, q.a);
-      accv(ei[i], s, q.b);
-      accv(orr[i], s, q.c);
-      accv(oi[i], s, q.d);
-    }
-  }
+      for (int i = 0; i < NP; i += 2) {
+        V c0, c1, a0, a1;
+        fma2(c0, c1, r.a, r.a, w[i], w[i + 1], r.b, r.b);
+        fma2(a0, a1, c0, c1, s1[i], s1[i + 1], s2[i], s2[i + 1]);
+        if (inj) {
+          a0 = jj == js[i] ? d0[i] : a0;
+          a0 = jj == js[i] + 1 ? d1[i] : a0;
+          a1 = jj == js[i + 1] ? d0[i + 1] : a1;
+          a1 = jj == js[i + 1] + 1 ? d1[i + 1] : a1;
+        }
+        s2[i] = s1[i];
+        s2[i + 1] = s1[i + 1];
+        s1[i] = a0;
+        s1[i + 1] = a1;
+        fma2(er[i], er[i + 1], a0, a1, xe.a, xe.b, er[i], er[i + 1]);
+        fma2(ei[i], ei[i + 1], a0, a1, xe.c, xe.d, ei[i], ei[i + 1]);
+        fma2(orr[i], orr[i + 1], a0, a1, xo.a, xo.b, orr[i], orr[i + 1]);
+        fma2(oi[i], oi[i + 1], a0, a1, xo.c, xo.d, oi[i], oi[i + 1]);
+      }
+    };
+    for (; j <= jinj; ++j) step(j, true);  // seeds may still enter
 #pragma unroll 4
-  for (; j < J; ++j) {
-    const Pair<V> r = sr[j];
-    const Quad<V> q = sx[j];
+    for (; j < J; ++j) step(j, false);
+  } else {
+    auto step = [&](int jj, bool inj) {
+      const Pair<V> r = sr[jj];
+      const Quad<V> q = sx[jj];
 #pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      const V s = fmav(fmav(r.a, w[i], r.b), s1[i], s2[i]);
-      s2[i] = s1[i];
-      s1[i] = s;
-      accv(er[i], s, q.a);
-      accv(ei[i], s, q.b);
-      accv(orr[i], s, q.c);
-      accv(oi[i], s, q.d);
-    }
+      for (int i = 0; i < NP; ++i) {
+        V s = fmav(fmav(r.a, w[i], r.b), s1[i], s2[i]);
+        if (inj) {
+          s = jj == js[i] ? d0[i] : s;
+          s = jj == js[i] + 1 ? d1[i] : s;
+        }
+        s2[i] = s1[i];
+        s1[i] = s;
+        accv(er[i], s, q.a);
+        accv(ei[i], s, q.b);
+        accv(orr[i], s, q.c);
+        accv(oi[i], s, q.d);
+      }
+    };
+    for (; j <= jinj; ++j) step(j, true);  // seeds may still enter
+#pragma unroll 4
+    for (; j < J; ++j) step(j, false);
   }
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
     const int k = pair0 + lane + 32 * i;
     if (k >= npairs) continue;
     const V z = t.z[k], zr = z * orr[i], zi = z * oi[i];
-    F[k * stride + m] = {er[i] + zr, ei[i] + zi};
-    if (k < npairs - 1) F[(2 * npairs - 2 - k) * stride + m] = {er[i] - zr, ei[i] - zi};
+    out[k] = {er[i] + zr, ei[i] + zi, er[i] - zr, ei[i] - zi};
   }
 }
 
@@ -283,25 +344,45 @@ constexpr int PANA_TILE = 2048;
 constexpr int PANA_MAXWARPS = 8;
 constexpr int CKJ = 16;
 
-// 16 steps of one pair: the recurrence and the four sums of each j.  INJ: the
-// pair's seeds (d0, d1) may enter, at step `rel` and the next.
-template <typename V, bool INJ>
-__device__ __forceinline__ void pair_block(V (&v)[4 * CKJ], const Pair<V> *__restrict__ sr, V w,
-                                           V s1, V s2, const Quad<V> &p, int rel, V d0, V d1) {
+// 16 steps of R pairs (one lane's): the recurrence and the four sums of each j; in
+// FP32 the real and the imaginary sum of one parity are one packed accumulator.
+// INJ: a pair's seeds c may enter, at step `rel` and the next (else c is the state
+// before the block), and the pairs may differ in their form (table sr[i]).
+template <typename V, int R, bool INJ>
+__device__ __forceinline__ void pair_block(V (&v)[4 * CKJ], const Pair<V> *const (&sr)[R],
+                                           const V (&w)[R], const typename Cx<V>::type (&c)[R],
+                                           const Quad<V> (&p)[R], const int (&rel)[R]) {
+  V s1[R], s2[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const bool inj = INJ && (unsigned)rel[i] < (unsigned)CKJ;
+    s1[i] = inj ? (V)0 : c[i].x;
+    s2[i] = inj ? (V)0 : c[i].y;
+  }
 #pragma unroll
   for (int jj = 0; jj < CKJ; ++jj) {
-    const Pair<V> r = sr[jj];
-    V s = fmav(fmav(r.a, w, r.b), s1, s2);
-    if (INJ) {
-      s = jj == rel ? d0 : s;
-      s = jj == rel + 1 ? d1 : s;
+    Pair<V> r = sr[0][jj];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      if (INJ && i > 0) r = sr[i][jj];
+      V s = fmav(fmav(r.a, w[i], r.b), s1[i], s2[i]);
+      if (INJ) {
+        s = jj == rel[i] ? c[i].x : s;
+        if (jj > 0) s = jj == rel[i] + 1 ? c[i].y : s;
+      }
+      s2[i] = s1[i];
+      s1[i] = s;
+      V *x = v + 4 * jj;
+      if constexpr (std::is_same<V, float>::value) {
+        fma2(x[0], x[1], s, s, p[i].a, p[i].b, x[0], x[1]);
+        fma2(x[2], x[3], s, s, p[i].c, p[i].d, x[2], x[3]);
+      } else {
+        accv(x[0], s, p[i].a);
+        accv(x[1], s, p[i].b);
+        accv(x[2], s, p[i].c);
+        accv(x[3], s, p[i].d);
+      }
     }
-    s2 = s1;
-    s1 = s;
-    accv(v[4 * jj], s, p.a);
-    accv(v[4 * jj + 1], s, p.b);
-    accv(v[4 * jj + 2], s, p.c);
-    accv(v[4 * jj + 3], s, p.d);
   }
 }
 
@@ -338,6 +419,43 @@ __device__ __forceinline__ void pair_finish(long i, int l, double ar, double ai,
   x[i] = make_double2(ar, ai);
 }
 
+// The same in FP32 (this part's FP64 unit runs at 1/64 of the FP32 rate): the filter
+// from the FP32 C_l, om = Omega, xio = xi Omega, muo = mu Omega.  Only the Cauchy
+// differences against the FP64 iterate stay in FP64 (unweighted: the caller
+// multiplies by wm once).  xs (optional): the coefficient in FP32, the next
+// synthesis' input.
+__device__ __forceinline__ void pair_finish32(long i, int l, float sr, float si, int mode,
+                                              const float *__restrict__ cl, float om, float xio,
+                                              float muo, const double2 *__restrict__ src,
+                                              const double2 *__restrict__ xa,
+                                              double2 *__restrict__ x, float2 *__restrict__ xs,
+                                              double &num, double &den, double &dx) {
+  float ar = om * sr, ai = om * si;
+  if (mode == ANA_FILTER) {
+    const float sbar = fmaxf(cl[l] - muo, 0.f);
+    const float f = sbar > 0.f ? sbar / (sbar + xio) : 0.f;
+    if (src) {  // harmonic source term of a correction solve
+      const double2 sv = src[i];
+      ar = fmaf(xio, (float)sv.x, ar);
+      ai = fmaf(xio, (float)sv.y, ai);
+    }
+    ar *= f;
+    ai *= f;
+    const double2 old = x[i];
+    const double ard = ar, aid = ai;
+    const double dr = ard - old.x, di = aid - old.y;
+    num = fma(dr, dr, fma(di, di, num));
+    den = fma(ard, ard, fma(aid, aid, den));
+    if (xa) {  // anchored stage: ||x_a + delta||^2
+      const double2 b = xa[i];
+      const double tr = ard + b.x, ti = aid + b.y;
+      dx = fma(tr, tr, fma(ti, ti, dx));
+    }
+  }
+  x[i] = make_double2(ar, ai);
+  if (xs) xs[i] = make_float2(ar, ai);
+}
+
 // block sums of the Cauchy partials -> partials[2m], [2m + 1] and (anchored
 // stages) [2 (lmax + 1) + m], in a fixed order
 __device__ __forceinline__ void pair_partials(double num, double den, double dx, int m, int lmax,
@@ -369,13 +487,15 @@ __device__ __forceinline__ void pair_partials(double num, double den, double dx,
 }
 
 template <typename V>
-__global__ void __launch_bounds__(32 * PANA_MAXWARPS)
+__global__ void __launch_bounds__(32 * PANA_MAXWARPS, sizeof(V) == 4 ? 2 : 1)
     k_pair_anal(const PairTab<V> t, int npairs, int lmax,
                 const double *__restrict__ cl, double omega,
                 const typename Cx<V>::type *__restrict__ G, double2 *__restrict__ x,
                 double *__restrict__ partials, const double2 *__restrict__ src,
+                typename Cx<V>::type *__restrict__ xs, const float *__restrict__ cl32,
                 const SolverState *__restrict__ st, int mode, int lstatic) {
   typedef typename Cx<V>::type C;
+  constexpr int R = std::is_same<V, float>::value ? 2 : 1;  // pairs in flight per lane
   const int m = blockIdx.x;
   int L = lstatic;
   double xi = 0.0, mu = 0.0;
@@ -395,63 +515,77 @@ __global__ void __launch_bounds__(32 * PANA_MAXWARPS)
   if (m <= L) {
     extern __shared__ __align__(16) unsigned char smraw[];
     const int J = (L - m) / 2 + 1, nb = (J + CKJ - 1) / CKJ, J16 = nb * CKJ;
-    const int tile = min(npairs, PANA_TILE);
+    const int tile = min((npairs + 63) / 64 * 64, PANA_TILE);
     Quad<V> *sp = reinterpret_cast<Quad<V> *>(smraw);                 // [tile]
     Quad<V> *sd = sp + tile;                                          // [J16]
-    Pair<V> *srb = reinterpret_cast<Pair<V> *>(sd + J16);             // [J16]
-    Pair<V> *src_ = srb + J16;                                        // [J16]
+    Pair<V> *srec = reinterpret_cast<Pair<V> *>(sd + J16);            // [3][J16]
     const long q0 = pair_base(lmax, m), cb = block_base(lmax, m);
-    for (int j = tid; j < J16; j += blockDim.x) {
-      const Pair<V> zero = {(V)0, (V)0};
-      srb[j] = j < J ? reinterpret_cast<const Pair<V> *>(t.rec_b)[q0 + j] : zero;
-      src_[j] = j < J ? reinterpret_cast<const Pair<V> *>(t.rec_c)[q0 + j] : zero;
-    }
-    const long stride = lmax + 1;
+    for (int j = tid; j < J16; j += blockDim.x) sd[j] = {(V)0, (V)0, (V)0, (V)0};
+    for (int f = 0; f < 3; ++f)
+      for (int j = tid; j < J16; j += blockDim.x) {
+        const Pair<V> zero = {(V)0, (V)0};
+        srec[f * J16 + j] = j < J ? reinterpret_cast<const Pair<V> *>(t.rec[f])[q0 + j] : zero;
+      }
     for (int t0 = 0; t0 < npairs; t0 += PANA_TILE) {
       const int nt = min(PANA_TILE, npairs - t0);
       __syncthreads();  // the previous tile's reads are done
-      for (int k = tid; k < nt; k += blockDim.x) {
-        const int kk = t0 + k;
-        const C gn = G[kk * stride + m];
-        C gs = {};
-        if (kk < npairs - 1) gs = G[(2 * npairs - 2 - kk) * stride + m];
-        const V z = t.z[kk];
-        sp[k] = {gn.x + gs.x, gn.y + gs.y, z * (gn.x - gs.x), z * (gn.y - gs.y)};
+      for (int k = tid; k < (nt + 63) / 64 * 64; k += blockDim.x) {
+        Quad<V> q = {(V)0, (V)0, (V)0, (V)0};
+        if (k < nt) q = reinterpret_cast<const Quad<V> *>(G)[(long)m * npairs + t0 + k];
+        if (t0 + k == npairs - 1) q.c = q.d = (V)0;  // the equator
+        const V z = t.z[t0 + k];
+        sp[k] = {q.a + q.c, q.b + q.d, z * (q.a - q.c), z * (q.b - q.d)};
       }
       __syncthreads();
+      // js, the checkpoints and w are loaded one step (32 R pairs) ahead
+      const int *jrow = t.jin + (long)m * t.stride + t0 + lane;
       for (int b = warp; b < nb; b += nwarps) {
         const int j0 = b * CKJ;
+        const C *crow = t.ck + (cb + b) * t.stride + t0 + lane;
+        int rel[R], form[R];
+        C c[R];
+        V w[R];
+        auto load = [&](int g) {
+#pragma unroll
+          for (int i = 0; i < R; ++i) {
+            form[i] = t.form(t0 + g + 32 * i);
+            rel[i] = R == 2 ? jrow[g + 32 * i] - j0 : -1;  // FP64: no seeds enter
+            c[i] = crow[g + 32 * i];
+            w[i] = t.w[form[i] * t.stride + t0 + lane + g + 32 * i];
+          }
+        };
         V v[4 * CKJ];
 #pragma unroll
         for (int i = 0; i < 4 * CKJ; ++i) v[i] = (V)0;
-        for (int g = 0; g < nt; g += 32) {
-          const int k = t0 + g + lane;
-          int js = INT_MAX / 2;
-          if (g + lane < nt) js = t.js[(long)m * npairs + k];
-          const bool on = js < j0 + CKJ;
-          if (!__any_sync(0xffffffffu, on)) continue;
-          const bool polar = t0 + g < t.kpol;
-          const Pair<V> *sr = (polar ? src_ : srb) + j0;
-          C c = {};
-          V w = (V)0;
-          Quad<V> p = {(V)0, (V)0, (V)0, (V)0};
-          if (on) {
-            c = t.ck[(cb + b) * npairs + k];
-            w = t.w[polar ? npairs + k : k];
-            p = sp[g + lane];
+        // below its first warp of pairs a block is zero
+        int g = max(0, t.gfirst[cb + b] - t0) / (32 * R) * (32 * R);
+        if (g < nt) load(g);
+        for (; g < nt; g += 32 * R) {
+          const Pair<V> *sr[R];
+          V wc[R];
+          C d[R];
+          Quad<V> p[R];
+          int rl[R];
+          bool slow = R == 2 && form[0] != form[R - 1];
+#pragma unroll
+          for (int i = 0; i < R; ++i) {
+            sr[i] = srec + form[i] * J16 + j0;
+            wc[i] = w[i];
+            d[i] = c[i];
+            rl[i] = rel[i];
+            p[i] = sp[g + 32 * i + lane];
+            slow |= (unsigned)rel[i] < (unsigned)CKJ;
           }
-          const bool inj = on && js >= j0;
-          if (__any_sync(0xffffffffu, inj || !on)) {
-            const V s1 = inj ? (V)0 : c.x, s2 = inj ? (V)0 : c.y;
-            pair_block<V, true>(v, sr, w, s1, s2, p, inj ? js - j0 : -2, c.x, c.y);
-          } else {
-            pair_block<V, false>(v, sr, w, c.x, c.y, p, 0, c.x, c.y);
-          }
+          if (g + 32 * R < nt) load(g + 32 * R);
+          if (R == 2 && __any_sync(0xffffffffu, slow))
+            pair_block<V, R, true>(v, sr, wc, d, p, rl);
+          else
+            pair_block<V, R, false>(v, sr, wc, d, p, rl);
         }
-        V *d = reinterpret_cast<V *>(sd) + 4 * j0 + lane;
+        V *dd = reinterpret_cast<V *>(sd) + 4 * j0 + lane;
         const V lo = lane_sums(v, lane), hi = lane_sums(v + 32, lane);
-        d[0] = t0 ? d[0] + lo : lo;
-        d[32] = t0 ? d[32] + hi : hi;
+        dd[0] += lo;
+        dd[32] += hi;
       }
     }
     __syncthreads();
@@ -472,8 +606,17 @@ __global__ void __launch_bounds__(32 * PANA_MAXWARPS)
           si = fmav(g, sd[j - 1].b, si);
         }
       }
-      pair_finish(a0 + i, m + i, omega * sr, omega * si, wm, mode, cl, omega, xi, mu, src, xa, x,
-                  num, den, dx);
+      if constexpr (std::is_same<V, float>::value)
+        pair_finish32(a0 + i, m + i, sr, si, mode, cl32, (float)omega, (float)(xi * omega),
+                      (float)(mu * omega), src, xa, x, xs, num, den, dx);
+      else
+        pair_finish(a0 + i, m + i, omega * sr, omega * si, wm, mode, cl, omega, xi, mu, src, xa,
+                    x, num, den, dx);
+    }
+    if constexpr (std::is_same<V, float>::value) {
+      num *= wm;
+      den *= wm;
+      dx *= wm;
     }
   }
   // coefficients of this m above the band are zero
@@ -484,15 +627,21 @@ __global__ void __launch_bounds__(32 * PANA_MAXWARPS)
       num += wm * (old.x * old.x + old.y * old.y);
     }
     x[i] = make_double2(0.0, 0.0);
+    if constexpr (std::is_same<V, float>::value) {
+      if (xs) xs[i] = make_float2(0.f, 0.f);
+    }
   }
   if (mode == ANA_FILTER) pair_partials(num, den, dx, m, lmax, partials);
 }
 
 // ------------------------------------------------------------- launch
-static size_t synth_smem(size_t v, int lmax) { return 6 * v * (lmax / 2 + 1); }
+// per j: a quad (packed FP32: two) and one form's pair (FP32: three)
+static size_t synth_smem(size_t v, int lmax, bool packed = false) {
+  return ((packed ? 8 : 4) + (v == 4 ? 6 : 2)) * v * (lmax / 2 + 1);
+}
 static size_t anal_smem(size_t v, int npairs, int lmax) {
   const size_t j16 = (size_t)(lmax / 32 + 1) * CKJ;
-  return 4 * v * std::min(npairs, PANA_TILE) + 8 * v * j16;
+  return 4 * v * std::min((npairs + 63) / 64 * 64, PANA_TILE) + 10 * v * j16;
 }
 
 template <int NP>
@@ -526,7 +675,43 @@ wf_status launch_legendre_anal<double2>(const Plan &P, const double2 *G, double2
   ++P.nlaunch;
   const int warps = std::max(2, std::min(PANA_MAXWARPS, P.lmax / 32 + 1));
   k_pair_anal<double><<<P.lmax + 1, 32 * warps, anal_smem(8, P.npairs, P.lmax), P.stream>>>(
-      P.pt64, P.npairs, P.lmax, P.cl_d, P.omega, G, x, P.partials, src, st, mode,
+      P.pt64, P.npairs, P.lmax, P.cl_d, P.omega, G, x, P.partials, src, nullptr, nullptr, st,
+      mode, lstatic);
+  WF_CUDA(cudaGetLastError());
+  return WF_OK;
+}
+
+template <int NP>
+static void synth32(const Plan &P, const float2 *x, float2 *F, const SolverState *st,
+                    int lstatic) {
+  const int tile = PSYN_THREADS32 * NP;
+  const dim3 grid((P.npairs + tile - 1) / tile, P.lmax + 1);
+  k_pair_synth<float, NP>
+      <<<grid, PSYN_THREADS32, synth_smem(4, P.lmax, NP % 2 == 0), P.stream>>>(
+          P.pt32, P.npairs, P.lmax, x, F, st, lstatic);
+}
+
+template <>
+wf_status launch_legendre_synth<float2>(const Plan &P, const float2 *xs, float2 *F,
+                                        const SolverState *st, int lstatic) {
+  ++P.nlaunch;
+  switch (P.syn_np[1]) {
+    case 1: synth32<1>(P, xs, F, st, lstatic); break;
+    case 4: synth32<4>(P, xs, F, st, lstatic); break;
+    default: synth32<2>(P, xs, F, st, lstatic); break;
+  }
+  WF_CUDA(cudaGetLastError());
+  return WF_OK;
+}
+
+template <>
+wf_status launch_legendre_anal<float2>(const Plan &P, const float2 *G, double2 *x,
+                                       const SolverState *st, int mode, int lstatic,
+                                       const double2 *src, float2 *xs_out) {
+  ++P.nlaunch;
+  const int warps = std::max(2, std::min(PANA_MAXWARPS, P.lmax / 32 + 1));
+  k_pair_anal<float><<<P.lmax + 1, 32 * warps, anal_smem(4, P.npairs, P.lmax), P.stream>>>(
+      P.pt32, P.npairs, P.lmax, P.cl_d, P.omega, G, x, P.partials, src, xs_out, P.cl32, st, mode,
       lstatic);
   WF_CUDA(cudaGetLastError());
   return WF_OK;
@@ -540,6 +725,14 @@ wf_status init_pair_attributes() {
                                cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   WF_CUDA(cudaFuncSetAttribute(k_pair_synth<double, 4>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  WF_CUDA(cudaFuncSetAttribute(k_pair_synth<float, 1>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  WF_CUDA(cudaFuncSetAttribute(k_pair_synth<float, 2>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  WF_CUDA(cudaFuncSetAttribute(k_pair_synth<float, 4>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  WF_CUDA(cudaFuncSetAttribute(k_pair_anal<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               big));
   WF_CUDA(cudaFuncSetAttribute(k_pair_anal<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                big));
   return WF_OK;
@@ -547,31 +740,38 @@ wf_status init_pair_attributes() {
 
 // ------------------------------------------------------------- tables
 // s of every (m, pair): a walk from lam_mm (mantissa, exponent) in scaled FP64
-// until |Q_j| reaches 2^-100, then plainly to the last j, leaving the seeds and
-// the state before each block.
-__global__ void k_pair_walk(int npairs, int lmax, int kpol, const double *__restrict__ w64,
-                            const double2 *__restrict__ rec_b,
-                            const double2 *__restrict__ rec_c, const double *__restrict__ so,
-                            const double *__restrict__ mant, const int *__restrict__ expo,
-                            int *__restrict__ js_out, double2 *__restrict__ ck) {
+// until |Q_j| reaches 2^-100, then plainly to the last j, leaving the seeds, the state
+// before each block and, in FP32, the blocks where the seeds enter.
+__global__ void k_pair_walk(int npairs, int lmax, const PairTab<double> t_,
+                            const PairTab<float> u, const double *__restrict__ mant,
+                            const int *__restrict__ expo) {
   const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long)npairs * (lmax + 1)) return;
   const int m = (int)(t / npairs), k = (int)(t % npairs);
-  const int J = (lmax - m) / 2 + 1;
-  const long q0 = pair_base(lmax, m), cb = block_base(lmax, m);
-  const double2 *rec = (k < kpol ? rec_c : rec_b) + q0;
-  const double w = w64[k < kpol ? npairs + k : k];
+  const int J = (lmax - m) / 2 + 1, stride = t_.stride;
+  const long q0 = pair_base(lmax, m), cb = block_base(lmax, m), mk = (long)m * stride + k;
+  const int form = t_.form(k);
+  const double2 *rec = t_.rec[form] + q0;
+  const double w = t_.w[form * stride + k];
   double v = mant[t] * sqrt(2.0 * m + 3.0), vp = 0.0;  // Q_0 = lam_mm / eps_{m+1}
   int e = expo[t], j = 0;                              // value v 2^e
+  // the state before the block of j: rec[0] = (0, 0), so (0, s_0) yields s_0 at j = 0
+  double b1 = 0.0, b2 = v;
+  int be = e;
   bool found = false;
   for (;;) {
-    const double a = fabs(v * so[q0 + j]);
+    const double a = fabs(v * t_.so[q0 + j]);
     if (e == 0 ? a >= 0x1p-100 : (e == -200 && a >= 0x1p+100)) {
       found = true;
       break;
     }
     if (j == J - 1) break;
     ++j;
+    if ((j & 15) == 0) {
+      b1 = v;
+      b2 = vp;
+      be = e;
+    }
     const double2 r = rec[j];
     const double vn = fma(fma(r.x, w, r.y), v, vp);
     vp = v;
@@ -582,19 +782,34 @@ __global__ void k_pair_walk(int npairs, int lmax, int kpol, const double *__rest
       e += 200;
     }
   }
-  js_out[t] = found ? j : INT_MAX / 2;
-  if (!found) return;
-  double s1 = ldexp(v, e), s2 = ldexp(vp, e);
-  {
-    double nx = 0.0;
-    if (j + 1 < J) {
-      const double2 r = rec[j + 1];
-      nx = fma(fma(r.x, w, r.y), s1, s2);
-    }
-    ck[(cb + (j >> 4)) * npairs + k] = make_double2(s1, nx);
+  if (!found) return;  // the tables are zero, js and jin beyond every block
+  const int js = j, bj = j >> 4;
+  t_.js[mk] = js;
+  for (int b = bj; b < (J + 15) / 16; ++b)
+    if (k / 32 * 32 < t_.gfirst[cb + b]) atomicMin(t_.gfirst + cb + b, k / 32 * 32);
+  double s1 = ldexp(v, e), s2 = ldexp(vp, e), nx = 0.0;
+  if (j + 1 < J) {
+    const double2 r = rec[j + 1];
+    nx = fma(fma(r.x, w, r.y), s1, s2);
   }
+  t_.seed[mk] = make_double2(s1, nx);
+  u.seed[mk] = make_float2((float)s1, (float)nx);
+  const double2 st = make_double2(ldexp(b1, be), ldexp(b2, be));
+  t_.ck[(cb + bj) * stride + k] = st;
+  const bool fits = fmax(fabs(st.x), fabs(st.y)) >= 0x1p-120;
+  if (fits) u.ck[(cb + bj) * stride + k] = make_float2((float)st.x, (float)st.y);
+  const double seed0 = s1;
   for (;;) {
-    if ((j & 15) == 15 && j + 1 < J) ck[(cb + (j >> 4) + 1) * npairs + k] = make_double2(s1, s2);
+    if ((j & 15) == 15 || j + 1 == J) {
+      if (!fits && (j >> 4) == bj && fmax(fabs(s1), fabs(s2)) >= 0x1p-80) {
+        u.ck[(cb + bj) * stride + k] = make_float2((float)seed0, (float)nx);
+        u.jin[mk] = js;
+      }
+      if (j + 1 < J) {
+        t_.ck[(cb + (j >> 4) + 1) * stride + k] = make_double2(s1, s2);
+        u.ck[(cb + (j >> 4) + 1) * stride + k] = make_float2((float)s1, (float)s2);
+      }
+    }
     if (++j >= J) break;
     const double2 r = rec[j];
     const double s = fma(fma(r.x, w, r.y), s1, s2);
@@ -630,6 +845,9 @@ __device__ __forceinline__ d2 d2_add(d2 a, d2 b) {  // |a| >= |b|
   const double s = __dadd_rn(a.h, b.h);
   return d2_norm(s, (b.h - (s - a.h)) + (a.l + b.l));
 }
+__device__ __forceinline__ d2 d2_sum(d2 a, d2 b) {  // any order
+  return fabs(a.h) >= fabs(b.h) ? d2_add(a, b) : d2_add(b, a);
+}
 // eps_l^2 = (l - m) (l + m) / ((2 l - 1) (2 l + 1)); the integers are exact
 __device__ __forceinline__ d2 eps2(double l, int m) {
   return d2_div({(l - m) * (l + m), 0.0}, {(2.0 * l - 1.0) * (2.0 * l + 1.0), 0.0});
@@ -659,14 +877,16 @@ __global__ void k_pair_coefs(int lmax, PairTab<double> t) {
     t.so[q0 + j] = fold * h1.h;
     const d2 up = d2_mul(r1, r2);
     const d2 hn = j == 0 ? one : d2_div(d2_mul(h0, up0), up);
-    if (j == 0) t.rec_b[q0] = t.rec_c[q0] = make_double2(0.0, 0.0);
+    if (j == 0) t.rec[0][q0] = t.rec[1][q0] = t.rec[2][q0] = make_double2(0.0, 0.0);
     if (j + 1 < J) {
       const double sg = (j & 1) ? -1.0 : 1.0;
       const d2 A = d2_div(h1, d2_mul(hn, up));
       const d2 e = e_l.h > e1.h ? d2_add(e_l, e1) : d2_add(e1, e_l);
-      const d2 B = d2_mul(A, e), C = d2_mul(A, d2_add(one, {-e.h, -e.l}));
-      t.rec_b[q0 + j + 1] = make_double2(sg * A.h, -sg * B.h);
-      t.rec_c[q0 + j + 1] = make_double2(sg * A.h, sg * C.h);
+      const d2 me = {-e.h, -e.l};
+      t.rec[0][q0 + j + 1] = make_double2(sg * A.h, sg * d2_mul(A, d2_add(one, me)).h);
+      t.rec[1][q0 + j + 1] =
+          make_double2(sg * A.h, sg * d2_mul(A, d2_sum({0.5, 0.0}, me)).h);
+      t.rec[2][q0 + j + 1] = make_double2(sg * A.h, sg * d2_mul(A, me).h);
     }
     // one-step: l - m = 2 j (g1, c0 from the last j) and 2 j + 1
     const double f2 = (j & 1) ? -1.0 : 1.0;
@@ -698,22 +918,24 @@ __global__ void k_pair_lmm(int npairs, int lmax, int keq, const double *__restri
   lmm[i] = ldexp(mant[i], expo[i]);
 }
 
+static wf_status build_pair_tables32(Plan &P, long nq);
+
 // The tables and the checkpoints.  mant, expo: lam_mm of every (m, pair).
 wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
   const int lmax = P.lmax;
   const long nq = pair_base(lmax, lmax) + 1;
   const long nb = block_base(lmax, lmax) + 1;
-  std::vector<double> w(2 * (size_t)P.npairs), z(P.npairs);
-  // rings with z > 0.7 use the polar form, in whole warps of pairs
-  int np = 0;
+  const int stride = (P.npairs + 63) / 64 * 64;  // rows padded to whole steps
+  std::vector<double> w(3 * (size_t)stride, 0.0), z(stride, 0.0);
+  // the forms' limits z^2 = 3/4 and 1/4, in whole warps of pairs
+  int kform[2] = {0, 0};
   for (int k = 0; k < P.npairs; ++k) {
     z[k] = P.pairs_h[k].z;
-    if (z[k] > 0.7) np = k + 1;
-  }
-  const int kpol = (np / 32) * 32;
-  for (int k = 0; k < P.npairs; ++k) {
-    w[k] = z[k] * z[k];
-    w[P.npairs + k] = -(1.0 - z[k]) * (1.0 + z[k]);
+    for (int f = 0; f < 2; ++f)
+      if (z[k] * z[k] > (f ? 0.25 : 0.75)) kform[f] = k + 1;
+    w[k] = -(1.0 - z[k]) * (1.0 + z[k]);
+    w[stride + k] = fma(z[k], z[k], -0.5);
+    w[2L * stride + k] = z[k] * z[k];
   }
   auto up = [](auto **dst, const auto &v) {
     WF_CUDA(cudaMalloc(dst, sizeof(v[0]) * v.size()));
@@ -725,11 +947,12 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
   while (keq > 0 && z[keq - 1] < 0.2 && lmax * log2(P.pairs_h[keq - 1].sth) > -90.0) --keq;
   keq = (keq + PSYN_THREADS - 1) / PSYN_THREADS * PSYN_THREADS;
   PairTab<double> &t = P.pt64;
-  t.kpol = kpol;
+  for (int f = 0; f < 2; ++f) t.kform[f] = (kform[f] + 16) / 32 * 32;
   t.keq = keq;
+  t.stride = stride;
   WF_TRY(up(&t.w, w));
   WF_TRY(up(&t.z, z));
-  for (double2 **a : {&t.rec_b, &t.rec_c, &t.rec_e})
+  for (double2 **a : {&t.rec[0], &t.rec[1], &t.rec[2], &t.rec_e})
     WF_CUDA(cudaMalloc(a, sizeof(double2) * nq));
   for (double **a : {&t.se, &t.sn, &t.so, &t.ge, &t.go})
     WF_CUDA(cudaMalloc(a, sizeof(double) * nq));
@@ -742,19 +965,70 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
                                                                    expo, t.lmm);
     WF_CUDA(cudaGetLastError());
   }
+  WF_TRY(build_pair_tables32(P, nq));
+  PairTab<float> &u = P.pt32;
+  // no seed: js and jin beyond every block; no checkpoint: zero (also the rows'
+  // padding)
+  const size_t mk = (size_t)stride * (lmax + 1), ck = (size_t)nb * stride;
+  WF_CUDA(cudaMalloc(&t.js, sizeof(int) * mk));
+  WF_CUDA(cudaMalloc(&u.jin, sizeof(int) * mk));
+  WF_CUDA(cudaMalloc(&t.seed, sizeof(double2) * mk));
+  WF_CUDA(cudaMalloc(&u.seed, sizeof(float2) * mk));
+  WF_CUDA(cudaMalloc(&t.ck, sizeof(double2) * ck));
+  WF_CUDA(cudaMalloc(&u.ck, sizeof(float2) * ck));
+  WF_CUDA(cudaMalloc(&t.gfirst, sizeof(int) * nb));
+  WF_CUDA(cudaMemsetAsync(t.js, 0x3f, sizeof(int) * mk, P.stream));
+  WF_CUDA(cudaMemsetAsync(u.jin, 0x3f, sizeof(int) * mk, P.stream));
+  WF_CUDA(cudaMemsetAsync(t.ck, 0, sizeof(double2) * ck, P.stream));
+  WF_CUDA(cudaMemsetAsync(u.ck, 0, sizeof(float2) * ck, P.stream));
+  WF_CUDA(cudaMemsetAsync(t.gfirst, 0x7f, sizeof(int) * nb, P.stream));  // none
+  u.js = t.js;
+  u.gfirst = t.gfirst;
   const long n = (long)P.npairs * (lmax + 1);
-  WF_CUDA(cudaMalloc(&t.js, sizeof(int) * n));
-  WF_CUDA(cudaMalloc(&t.ck, sizeof(double2) * nb * P.npairs));
-  k_pair_walk<<<(unsigned)((n + 127) / 128), 128, 0, P.stream>>>(
-      P.npairs, lmax, kpol, t.w, t.rec_b, t.rec_c, t.so, mant, expo, t.js, t.ck);
+  k_pair_walk<<<(unsigned)((n + 127) / 128), 128, 0, P.stream>>>(P.npairs, lmax, t, u, mant,
+                                                                 expo);
   WF_CUDA(cudaGetLastError());
   return WF_OK;
 }
 
+// FP32 copies of the FP64 tables
+__global__ void k_pair_round(const double *__restrict__ in, long n, float *__restrict__ out) {
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long)gridDim.x * blockDim.x)
+    out[i] = (float)in[i];
+}
+
+static wf_status build_pair_tables32(Plan &P, long nq) {
+  const PairTab<double> &t = P.pt64;
+  PairTab<float> &u = P.pt32;
+  auto round = [&P](auto **dst, const void *src, long n) {
+    WF_CUDA(cudaMalloc(dst, sizeof(float) * n));
+    const unsigned grid = (unsigned)std::min((n + 255) / 256, 4096L);
+    k_pair_round<<<grid, 256, 0, P.stream>>>(static_cast<const double *>(src), n,
+                                             reinterpret_cast<float *>(*dst));
+    WF_CUDA(cudaGetLastError());
+    return WF_OK;
+  };
+  for (int f = 0; f < 3; ++f) WF_TRY(round(&u.rec[f], t.rec[f], 2 * nq));
+  WF_TRY(round(&u.se, t.se, nq));
+  WF_TRY(round(&u.sn, t.sn, nq));
+  WF_TRY(round(&u.so, t.so, nq));
+  WF_TRY(round(&u.w, t.w, 3L * t.stride));
+  WF_TRY(round(&u.z, t.z, t.stride));
+  u.stride = t.stride;
+  for (int f = 0; f < 2; ++f) u.kform[f] = t.kform[f];
+  u.keq = P.npairs;
+  return WF_OK;
+}
+
 void free_pair_tables(Plan &P) {
+  PairTab<float> &u = P.pt32;
+  void *f[] = {u.rec[0], u.rec[1], u.rec[2], u.se, u.sn, u.so, u.w, u.z, u.ck, u.jin, u.seed};
+  for (void *p : f)
+    if (p) cudaFree(p);
   PairTab<double> &t = P.pt64;
-  void *b[] = {t.rec_b, t.rec_c, t.rec_e, t.se, t.sn, t.so, t.ge, t.go, t.w, t.z, t.lmm, t.js,
-               t.ck};
+  void *b[] = {t.rec[0], t.rec[1], t.rec[2], t.rec_e, t.se, t.sn, t.so, t.ge, t.go, t.w, t.z,
+               t.lmm, t.js, t.seed, t.ck, t.gfirst};
   for (void *p : b)
     if (p) cudaFree(p);
 }

@@ -359,29 +359,30 @@ __device__ __forceinline__ T2 ring_phase(int k, int num, int den, int tstep,
 //     = e^{i k phi0} (sum_j sgn^j F[k + j n] + sum_{j >= 1} sgn^j conj F[j n - k])
 // When n > L each sum has at most one term (every equatorial ring, the outer
 // polar rings): the two loads are issued together, not in dependent loops.
+// ms: distance of consecutive m.
 template <typename T2>
-__device__ __forceinline__ T2 fold(const typename CT<T2>::G *__restrict__ Fr, int k, int n,
-                                   int L, typename CT<T2>::T sgn, T2 ph) {
+__device__ __forceinline__ T2 fold(const typename CT<T2>::G *__restrict__ Fr, int ms, int k,
+                                   int n, int L, typename CT<T2>::T sgn, T2 ph) {
   typedef typename CT<T2>::T T;
   T2 acc = CT<T2>::mk((T)0, (T)0);
   if (n > L) {
     const T2 zero = CT<T2>::mk((T)0, (T)0);
-    const T2 a = k <= L ? CT<T2>::ld(Fr + k) : zero;
-    const T2 b = n - k <= L ? CT<T2>::ld(Fr + (n - k)) : zero;
+    const T2 a = k <= L ? CT<T2>::ld(Fr + (long)k * ms) : zero;
+    const T2 b = n - k <= L ? CT<T2>::ld(Fr + (long)(n - k) * ms) : zero;
     acc = CT<T2>::mk(a.x + sgn * b.x, a.y - sgn * b.y);
     return cmul(acc, ph);
   }
   T s = (T)1;
 #pragma unroll 4
   for (int m = k; m <= L; m += n) {
-    const T2 f = CT<T2>::ld(Fr + m);
+    const T2 f = CT<T2>::ld(Fr + (long)m * ms);
     acc = CT<T2>::mk(acc.x + s * f.x, acc.y + s * f.y);
     s *= sgn;
   }
   s = sgn;
 #pragma unroll 4
   for (int m = n - k; m <= L; m += n) {  // m >= 1 since k < n
-    const T2 f = CT<T2>::ld(Fr + m);
+    const T2 f = CT<T2>::ld(Fr + (long)m * ms);
     acc = CT<T2>::mk(acc.x + s * f.x, acc.y - s * f.y);
     s *= sgn;
   }
@@ -396,7 +397,7 @@ constexpr int RING_THREADS_BIG = 512;
 
 template <typename T2, int MODE>
 __global__ void __launch_bounds__(RING_THREADS_BIG)
-    k_ring(const RingPair *__restrict__ pairs, int pair_base, int lmax,
+    k_ring(const RingPair *__restrict__ pairs, int pair_base, int npairs, int lmax,
            const typename CT<T2>::G *__restrict__ F, typename CT<T2>::G *__restrict__ G,
            const double *__restrict__ in_map, double *__restrict__ out_map,
            const double *__restrict__ nvar, const typename CT<T2>::W *__restrict__ tw,
@@ -461,15 +462,19 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
   const WT *chirp = blue ? chirp_all + rp.chirp_ofs : nullptr;
   const WT *bhat = blue ? bhat_all + rp.bhat_ofs : nullptr;
   const WT *phs = (blue && phase_all) ? phase_all + rp.chirp_ofs : nullptr;
-  const long stride = lmax + 1;
   const bool south = rp.ringS >= 0;
+  // F and G: [m][pair][north, south] with `npairs` pairs, or (0: the grouped
+  // transforms) [ring][m]
+  const int ms = npairs ? 2 * npairs : 1;
+  const long rowN = npairs ? 2L * (pair_base + blk) : (long)rp.ringN * (lmax + 1);
+  const long rowS = npairs ? rowN + 1 : (long)rp.ringS * (lmax + 1);
   const T2 zero = CT<T2>::mk((T)0, (T)0);
   const T sgn = rp.phi_num ? (T)-1 : (T)1;  // e^{i n phi0}
   const int tstep = (rp.phi_num && Mmax % (2 * rp.phi_den) == 0) ? Mmax / (2 * rp.phi_den) : 0;
 
   if (MODE != RING_ANALYSIS) {
-    const GT *FN = F + rp.ringN * stride;
-    const GT *FS = south ? F + rp.ringS * stride : nullptr;
+    const GT *FN = F + rowN;
+    const GT *FS = south ? F + rowS : nullptr;
     if (n < (int)blockDim.x) {
       // small rings (n < threads): each k's sums over j are split across
       // P = threads / n threads (j = part mod P), whose partials are added
@@ -481,19 +486,19 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
         if (Lf >= 0) {
           for (int j = part; k + j * n <= Lf; j += P) {  // m = k + j n
             const T s = (sgn < (T)0 && (j & 1)) ? (T)-1 : (T)1;
-            const T2 f = CT<T2>::ld(FN + (k + j * n));
+            const T2 f = CT<T2>::ld(FN + (long)(k + j * n) * ms);
             pN = CT<T2>::mk(pN.x + s * f.x, pN.y + s * f.y);
             if (south) {
-              const T2 g = CT<T2>::ld(FS + (k + j * n));
+              const T2 g = CT<T2>::ld(FS + (long)(k + j * n) * ms);
               pS = CT<T2>::mk(pS.x + s * g.x, pS.y + s * g.y);
             }
           }
           for (int j = 1 + part; j * n - k <= Lf; j += P) {  // m = j n - k, conj
             const T s = (sgn < (T)0 && (j & 1)) ? (T)-1 : (T)1;
-            const T2 f = CT<T2>::ld(FN + (j * n - k));
+            const T2 f = CT<T2>::ld(FN + (long)(j * n - k) * ms);
             pN = CT<T2>::mk(pN.x + s * f.x, pN.y - s * f.y);
             if (south) {
-              const T2 g = CT<T2>::ld(FS + (j * n - k));
+              const T2 g = CT<T2>::ld(FS + (long)(j * n - k) * ms);
               pS = CT<T2>::mk(pS.x + s * g.x, pS.y - s * g.y);
             }
           }
@@ -520,8 +525,8 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
         T2 cN = zero, cS = zero;
         if (Lf >= 0 && (k <= Lf || n - k <= Lf)) {
           const T2 ph = ring_phase<T2>(k, rp.phi_num, rp.phi_den, tstep, tw, phs);
-          cN = fold(FN, k, n, Lf, sgn, ph);
-          if (south) cS = fold(FS, k, n, Lf, sgn, ph);
+          cN = fold(FN, ms, k, n, Lf, sgn, ph);
+          if (south) cS = fold(FS, ms, k, n, Lf, sgn, ph);
         }
         const T2 Zk = CT<T2>::mk(cN.x - cS.y, cN.y + cS.x);  // cN + i cS
         buf[sw(k)] = blue ? cmulc(cconj(Zk), CT<T2>::ldw(chirp + k)) : Zk;
@@ -616,8 +621,8 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
     fft_dit<T2, false>(buf, M, tw, Mmax);
   // split the two real rings and apply e^{-i m phi0}: for m = k + j n,
   // G[m] = sgn^j e^{-i k phi0} X_k (X^N or X^S)
-  GT *GN = G + rp.ringN * stride;
-  GT *GS = south ? G + rp.ringS * stride : nullptr;
+  GT *GN = G + rowN;
+  GT *GS = south ? G + rowS : nullptr;
   const T half = (T)0.5;
   const int kmax = min(n - 1, Lg);
   // small rings: the copies m = k + j n of each k are split across
@@ -639,8 +644,8 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
       for (int j = part; k + j * n <= Lg; j += P) {
         const int m = k + j * n;
         const T s = (sgn < (T)0 && (j & 1)) ? (T)-1 : (T)1;
-        CT<T2>::st(GN + m, CT<T2>::mk(s * tN.x, s * tN.y));
-        if (south) CT<T2>::st(GS + m, CT<T2>::mk(s * tS.x, s * tS.y));
+        CT<T2>::st(GN + (long)m * ms, CT<T2>::mk(s * tN.x, s * tN.y));
+        if (south) CT<T2>::st(GS + (long)m * ms, CT<T2>::mk(s * tS.x, s * tS.y));
       }
     }
   }
@@ -671,7 +676,8 @@ static wf_status launch_ring_mode(const Plan &P, const typename CT<T2>::G *F,
                                   typename CT<T2>::G *G, const double *in_map,
                                   double *out_map, const SolverState *st, int lstatic,
                                   const float *in32, const float2 *in_dd = nullptr,
-                                  int nbatch = 1, long bstride_f = 0, long bstride_m = 0) {
+                                  int nbatch = 1, long bstride_f = 0, long bstride_m = 0,
+                                  bool rows = false) {
   auto kern = k_ring<T2, MODE>;
   // two launches: the polar rings (pairs 0 .. nside-2, Bluestein unless n is
   // a power of two) and the equatorial belt (pairs nside-1 .. 2 nside-1);
@@ -699,7 +705,7 @@ static wf_status launch_ring_mode(const Plan &P, const typename CT<T2>::G *F,
     cudaStream_t s = (fork && g == 1) ? P.side_stream : P.stream;
     ++P.nlaunch;
     kern<<<dim3(e - b, nbatch), threads, smem, s>>>(
-        P.pairs, b, P.lmax, F, G, in_map, out_map, P.nvar, Tables<T2>::tw(P),
+        P.pairs, b, rows ? 0 : P.npairs, P.lmax, F, G, in_map, out_map, P.nvar, Tables<T2>::tw(P),
         P.fftMmax, Tables<T2>::ch(P), Tables<T2>::bh(P), st, lstatic, g == 0, in32,
         P.nvar32, red_ofs, Tables<T2>::ph(P), in_dd, P.nvardd, bstride_f, bstride_m);
     WF_CUDA(cudaGetLastError());
@@ -735,11 +741,12 @@ wf_status launch_ring_batch32(const Plan &P, int mode, const float2 *F, float2 *
                              long fstride, long mstride) {
   if (mode == RING_SYNTH)
     return launch_ring_mode<float2, RING_SYNTH>(P, F, G, in_map, out_map, nullptr, P.lmax,
-                                                nullptr, nullptr, nbatch, fstride, mstride);
+                                                nullptr, nullptr, nbatch, fstride, mstride,
+                                                true);
   if (mode == RING_ANALYSIS)
     return launch_ring_mode<float2, RING_ANALYSIS>(P, F, G, in_map, out_map, nullptr,
                                                    P.lmax, nullptr, nullptr, nbatch, fstride,
-                                                   mstride);
+                                                   mstride, true);
   set_error("batched ring transform: synthesis or analysis only");
   return WF_ERR_ARG;
 }

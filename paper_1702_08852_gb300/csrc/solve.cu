@@ -323,7 +323,7 @@ wf_status map2alm(Plan &P, const double *map, double *alm) {
 
 wf_status alm2map_f32(Plan &P, const double *alm, double *map) {
   const double2 *a = reinterpret_cast<const double2 *>(alm);
-  WF_TRY(launch_prescale<float2>(P, a, P.xs32));
+  WF_TRY(launch_to_f32(P, a, P.xs32));
   WF_TRY(launch_legendre_synth<float2>(P, P.xs32, P.F32, nullptr, P.lmax));
   WF_TRY(launch_ring<float2>(P, RING_SYNTH, P.F32, nullptr, nullptr, map, nullptr,
                              P.lmax));
@@ -536,7 +536,7 @@ static wf_status run_loop(Plan &P, int which, T2 *F, T2 *G, const double *tinit,
     WF_TRY(launch_ring<T2>(P, RING_ANALYSIS, nullptr, G, tinit, nullptr, nullptr,
                            P.lmax));
   } else {
-    WF_CUDA(cudaMemsetAsync(G, 0, sizeof(T2) * (size_t)P.nring * (P.lmax + 1),
+    WF_CUDA(cudaMemsetAsync(G, 0, sizeof(T2) * 2 * (size_t)P.npairs * (P.lmax + 1),
                             P.stream));
   }
   WF_TRY(capture_graph<T2>(P, which, F, G, data, src));

@@ -33,30 +33,25 @@ void set_error_static(const char *msg);
   } while (0)
 
 // ---------------------------------------------------------------- geometry
-// One iso-latitude ring pair: the north ring and its mirror image in the
-// south (the equator ring is a "pair" with no south ring).  Both rings share
-// nphi, |z| and phi0.
-// the FP32 tables as one kernel argument
-struct Tab32 {
-  const float2 *seed_s;
-  const float *zh, *zl;
-  const float *rg;
-  const float *cl;
-};
-
 // Tables of the Legendre kernels in the parity-pair basis (legpair.cu), V the
 // arithmetic; indexed by (m, j) except where noted
 template <typename V> struct PairVec;
 template <> struct PairVec<double> { typedef double2 type; };
+template <> struct PairVec<float> { typedef float2 type; };
 template <typename V>
 struct PairTab {
-  typename PairVec<V>::type *rec_b = nullptr, *rec_c = nullptr;  // (A, B), (A, A + B)
+  typename PairVec<V>::type *rec[3] = {};  // (A, B) of the three forms
   V *se = nullptr, *sn = nullptr, *so = nullptr;  // basis change, scales and signs included
-  V *w = nullptr;                                 // [2][npairs]: z^2, -sin^2 theta
-  V *z = nullptr;                                 // [npairs]
-  int *js = nullptr;                              // [lmax+1][npairs] first j, |Q_j| >= 2^-100
-  typename PairVec<V>::type *ck = nullptr;        // [block of 16 j of m][npairs]
-  int kpol = 0;                                   // pairs below it: the polar form
+  int stride = 0;                  // row length: npairs rounded up to 64
+  V *w = nullptr;                  // [3][stride]: z^2 - 1, z^2 - 1/2, z^2
+  V *z = nullptr;                  // [stride]
+  int *js = nullptr;               // [lmax+1][stride] first j with |Q_j| >= 2^-100
+  typename PairVec<V>::type *ck = nullptr;  // [block of 16 j of m][stride]
+  typename PairVec<V>::type *seed = nullptr;  // [lmax+1][stride] (s_js, s_js+1)
+  int *jin = nullptr;              // [lmax+1][stride] FP32: j where ck holds the seeds
+  int *gfirst = nullptr;           // [block]: first warp of pairs with a term in it
+  int kform[2] = {0, 0};           // pairs below kform[f]: form f (multiples of 32)
+  __host__ __device__ int form(int k) const { return k < kform[0] ? 0 : k < kform[1] ? 1 : 2; }
   // the pairs k >= keq in the synthesis: the one-step recurrence's coefficients
   // (l - m even, odd), its scales, and lam_mm [lmax+1][npairs]
   int keq = 0;
@@ -64,6 +59,9 @@ struct PairTab {
   V *ge = nullptr, *go = nullptr, *lmm = nullptr;
 };
 
+// One iso-latitude ring pair: the north ring and its mirror image in the
+// south (the equator ring is a "pair" with no south ring).  Both rings share
+// nphi, |z| and phi0.
 struct RingPair {
   double z;        // z of the north ring
   double sth;      // sin(theta) of the north ring
@@ -171,36 +169,22 @@ struct Plan {
   RingPair *pairs = nullptr;     // [npairs]
   double *cl_d = nullptr;        // [lmax+1]
   PairTab<double> pt64;          // parity-pair basis, FP64
+  PairTab<float> pt32;           // and FP32
   double *rc = nullptr;          // [nalm] recurrence coefficient c_lm
   double *rg = nullptr;          // [nalm] scale g_lm (lambda = g u)
-  float *rc32 = nullptr;         // [nalm] FP32 copy of rc
   float2 *rcdd = nullptr;        // [nalm] rc as double-float pairs (hi, lo)
   int *seed_l = nullptr;         // [lmax+1][npairs] first l with |lambda| >= 2^-100
   double2 *seed_u = nullptr;     // [lmax+1][npairs] (u_ls, u_ls+1)
-  // FP32 kernels' tables (no FP64 arithmetic left in their tile loads and
-  // epilogues): seeds in s-units (eps_ls u_ls, eps_ls+1 u_ls+1), z of each
-  // pair split as zh + zl (two arrays: the packed kernels pair the zh of two
-  // rings, so each value is loaded on its own), g_lm eps_l, C_l
-  float2 *seed_s32 = nullptr;    // [lmax+1][npairs]
-  float *zs32 = nullptr;         // [2][npairs]: zh, then zl
-  float *rg32 = nullptr;         // [nalm]
-  float *cl32 = nullptr;         // [lmax+1]
+  float *cl32 = nullptr;         // [lmax+1] C_l in FP32 (the FP32 analysis' filter)
 
-  // launch variants (ring pairs per thread), [0] = FP64, [1] = FP32; set by
-  // the autotuner (opts.autotune) or the defaults below
-  int syn_np[2] = {1, 2};
+  // ring pairs per thread of the synthesis, [0] = FP64, [1] = FP32 (make_seeds, or the
+  // autotuner: opts.autotune).  The other variants of wf_set_tuning are one kernel now:
+  // kept as they were set, for wf_get_tuning
+  int syn_np[2] = {1, 1};
   int ana_np[2] = {4, 8};
-  // FP32 analysis scheduling: 0 = one CTA per m, 1 = warps take (m, tile)
-  // items from a queue and a combine kernel sums the tiles (ana_scratch)
-  int ana_queue = 0;
-  // FP32 kernels on packed f32x2 pairs of rings (NP even): 0 / 1 (synthesis:
-  // 2 = packed with duplicated shared-memory tables)
-  int syn_x2 = 0, ana_x2 = 0;
-  // packed per-m FP32 analysis with its per-warp accumulators in global
-  // scratch (ana_scratch rows [warp][alm]) instead of shared memory: 1 with
-  // 16-l chunks, 2 with 8-l chunks
-  int ana_gacc = 0;
-  float *ana_scratch = nullptr;  // [tiles of 128 pairs][nalm] float2
+  int ana_queue = 0, syn_x2 = 0, ana_x2 = 0, ana_gacc = 0;
+  // double-float analysis: per-tile sums, first l of each item, the queue's next item
+  float *ana_scratch = nullptr;  // [tiles of 128 pairs][nalm] double2
   int *ana_lstart = nullptr;     // [lmax+1][tiles] first l written per item
   int *ana_counter = nullptr;    // the queue's next item (reset by the combine)
   int num_sms = 0;
@@ -231,13 +215,13 @@ struct Plan {
   float2 *nvardd = nullptr;      // [npix] sigma^2 as double-float (hi, lo); (+inf, 0) masked
 
   // work buffers
-  double2 *F64 = nullptr, *G64 = nullptr;   // [nring][lmax+1]
+  double2 *F64 = nullptr, *G64 = nullptr;   // [lmax+1][npairs][north, south]
   float2 *F32 = nullptr, *G32 = nullptr;
   double2 *x = nullptr;          // [nalm] current iterate
   double2 *xtmp = nullptr;       // [nalm]
   double2 *xacc = nullptr;       // [nalm] refined solution (mixed precision)
   double2 *xs64 = nullptr;       // [nalm] g_lm x_lm as double-float pairs, synthesis input
-  float2 *xs32 = nullptr;        // [nalm] g_lm x_lm, synthesis input (FP32)
+  float2 *xs32 = nullptr;        // [nalm] x_lm, synthesis input (FP32)
   double2 *src = nullptr;        // [nalm] harmonic source of a correction solve
   // mixed solver, stage boundaries between anchored stages: the unfiltered
   // FP64 analysis U = Omega Y^T t_a of the last two anchors and the next
@@ -296,16 +280,15 @@ struct Plan {
 // Legendre transforms (legendre.cu).  Modes of the analysis:
 enum AnalysisMode { ANA_PLAIN = 0, ANA_FILTER = 1 };
 
-// The FP32 synthesis reads xs = g_lm a_lm (written by the analysis of the previous
-// iteration, or by launch_prescale), the FP64 one the coefficients themselves.
-template <typename T2>
-wf_status launch_prescale(const Plan &P, const double2 *x, T2 *xs);
+// The synthesis reads the coefficients in its own precision: the FP32 ones are written
+// by the analysis of the previous iteration or by launch_to_f32.
+wf_status launch_to_f32(const Plan &P, const double2 *x, float2 *xs);
 template <typename T2>
 wf_status launch_legendre_synth(const Plan &P, const T2 *xs, T2 *F,
                                 const SolverState *st, int lstatic);
 // src (optional, FP64 alm): adds the harmonic source f_l xi Omega src_lm of an
 // anchored stage to the filtered coefficients (ANA_FILTER only).
-// xs_out (optional, FP32): also write the synthesis input g_lm a_lm.
+// xs_out (optional, FP32): also write the coefficients in FP32, the synthesis input.
 template <typename T2>
 wf_status launch_legendre_anal(const Plan &P, const T2 *G, double2 *x,
                                const SolverState *st, int mode, int lstatic,
@@ -328,7 +311,7 @@ wf_status launch_legendre_synth_dd(const Plan &P, const float4 *xs, float4 *F,
                                    const SolverState *st, int lstatic);
 wf_status launch_legendre_anal_dd(const Plan &P, const float4 *G, double2 *x,
                                   const SolverState *st, int mode, int lstatic,
-                                  const double2 *src = nullptr, double2 *xs_out = nullptr);
+                                  const double2 *src = nullptr);
 
 // Ring transforms (ringfft.cu).  Modes:
 enum RingMode {
