@@ -89,7 +89,8 @@ typedef struct {
                         test is FP64 either way. */
   int band_limit;    /* 1: restrict each stage's transforms to the band where
                         the truncated spectrum is nonzero (exact; default 1) */
-  int graph_chunk;   /* iterations per captured CUDA graph launch; 0 = auto */
+  int graph_chunk;   /* iterations per pass of the captured loop (timing = 1: per
+                        graph launch); 0 = auto */
   int refine_max;    /* WF_PREC_MIXED: max FP64 refinement steps (default 8) */
   int timing;        /* 1: time the Legendre kernels of every iteration with
                         CUDA events recorded inside the captured graphs

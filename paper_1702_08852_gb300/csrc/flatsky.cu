@@ -227,7 +227,7 @@ static SolverState flat_initial_state(const FlatPlan &F) {
 
 static int flat_ncols(const FlatPlan &F) { return F.n / FLAT_CB; }
 
-static wf_status flat_enqueue_iteration(FlatPlan &F, cudaStream_t st) {
+static wf_status flat_enqueue_iteration(FlatPlan &F, cudaStream_t st, LoopHandle loop) {
   F.nlaunch += 3;
   k_flat_cols<<<flat_ncols(F), FLAT_THREADS, F.smem_cols, st>>>(
       F.n, F.logn, F.omega, F.ck, F.T1, F.S, F.T2, F.tw, F.state, F.partials, FLAT_ITER);
@@ -235,44 +235,25 @@ static wf_status flat_enqueue_iteration(FlatPlan &F, cudaStream_t st) {
                                                       F.nvar, nullptr, F.tw, F.state,
                                                       FLAT_ITER);
   k_control<<<1, CONTROL_THREADS, 0, st>>>(F.state, F.partials, flat_ncols(F) - 1, nullptr,
-                                           F.trace);
+                                           F.trace, loop);
   WF_CUDA(cudaGetLastError());
   return WF_OK;
 }
 
 static wf_status flat_capture(FlatPlan &F) {
   if (F.graph) return WF_OK;
-  F.chunk = F.opts.graph_chunk > 0 ? F.opts.graph_chunk
-                                   : (int)std::max(8L, std::min(256L, (1L << 22) / ((long)F.n * F.n)));
+  // iterations per pass of the device loop (loop_unroll in solve.cu)
+  F.chunk = F.opts.graph_chunk > 0 ? F.opts.graph_chunk : 16;
   if (!F.capture_stream)
     WF_CUDA(cudaStreamCreateWithFlags(&F.capture_stream, cudaStreamNonBlocking));
-  cudaError_t e = cudaStreamBeginCapture(F.capture_stream, cudaStreamCaptureModeThreadLocal);
-  if (e != cudaSuccess) {
-    set_error(std::string("wf_flat: graph capture: ") + cudaGetErrorString(e));
-    return WF_ERR_CUDA;
-  }
   const long n0 = F.nlaunch;
-  wf_status s = WF_OK;
-  for (int i = 0; i < F.chunk && s == WF_OK; ++i) s = flat_enqueue_iteration(F, F.capture_stream);
+  const wf_status s = capture_loop(F.capture_stream, &F.graph, [&](LoopHandle loop) {
+    for (int i = 0; i < F.chunk; ++i)
+      WF_TRY(flat_enqueue_iteration(F, F.capture_stream, loop));
+    return WF_OK;
+  });
   F.nlaunch = n0;
-  cudaGraph_t g = nullptr;
-  e = cudaStreamEndCapture(F.capture_stream, &g);
-  if (s != WF_OK) {
-    if (g) cudaGraphDestroy(g);
-    return s;
-  }
-  if (e != cudaSuccess) {
-    set_error(std::string("wf_flat: graph capture: ") + cudaGetErrorString(e));
-    return WF_ERR_CUDA;
-  }
-  e = cudaGraphInstantiate(&F.graph, g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) {
-    F.graph = nullptr;
-    set_error(std::string("wf_flat: graph instantiate: ") + cudaGetErrorString(e));
-    return WF_ERR_CUDA;
-  }
-  return WF_OK;
+  return s;
 }
 
 static wf_status flat_solve(FlatPlan &F, const double *d, double *s_out, wf_stats *stats) {
@@ -291,15 +272,11 @@ static wf_status flat_solve(FlatPlan &F, const double *d, double *s_out, wf_stat
                                                             nullptr, FLAT_FWD);
   WF_CUDA(cudaGetLastError());
   WF_TRY(flat_capture(F));
-  long graph_nodes = 3L * F.chunk;
-  for (;;) {
-    WF_CUDA(cudaGraphLaunch(F.graph, F.stream));
-    F.nlaunch += graph_nodes;
-    WF_CUDA(cudaMemcpyAsync(F.state_h, F.state, sizeof(SolverState), cudaMemcpyDeviceToHost,
-                            F.stream));
-    WF_CUDA(cudaStreamSynchronize(F.stream));
-    if (F.state_h->done) break;
-  }
+  WF_CUDA(cudaGraphLaunch(F.graph, F.stream));
+  WF_CUDA(cudaMemcpyAsync(F.state_h, F.state, sizeof(SolverState), cudaMemcpyDeviceToHost,
+                          F.stream));
+  WF_CUDA(cudaStreamSynchronize(F.stream));
+  F.nlaunch += 3L * ((F.state_h->iter + F.chunk - 1) / F.chunk) * F.chunk;
   // s of the last iteration: the inverse transforms of its filtered spectrum
   F.nlaunch += 2;
   k_flat_cols<<<flat_ncols(F), FLAT_THREADS, F.smem_cols, F.stream>>>(

@@ -64,11 +64,14 @@ constexpr int MAX_REANCHORS = 4096;
 
 __global__ void __launch_bounds__(CTRL_THREADS)
     k_control(SolverState *st, const double *__restrict__ partials, int lmax,
-              const double *__restrict__ cl, TraceEntry *trace) {
+              const double *__restrict__ cl, TraceEntry *trace, LoopHandle loop) {
   __shared__ double snum[CTRL_THREADS], sden[CTRL_THREADS];
   __shared__ int sh[CTRL_THREADS];
   __shared__ int advance;
-  if (st->done) return;
+  if (st->done) {
+    if (loop.on && threadIdx.x == 0) cudaGraphSetConditional(loop.h, 0);
+    return;
+  }
   __shared__ double sdx[CTRL_THREADS];
   double num = 0.0, den = 0.0, dx = 0.0;
   const bool anchored = st->xa != nullptr;
@@ -200,6 +203,7 @@ __global__ void __launch_bounds__(CTRL_THREADS)
       st->reanchor = 1;
     }
     if (!st->done && st->iter >= st->max_iter) st->done = 1;
+    if (st->done && loop.on) cudaGraphSetConditional(loop.h, 0);
     advance = adv;
   }
   __syncthreads();
@@ -438,7 +442,7 @@ template <> struct Scaled<float2> {
 // harmonic source `src`
 template <typename T2>
 static wf_status enqueue_iteration(Plan &P, T2 *F, T2 *G, const double *data,
-                                   const double2 *src, int slot) {
+                                   const double2 *src, int slot, LoopHandle loop) {
   const bool timed = slot >= 0 && P.tev_chunk > 0;
   const int C = P.tev_chunk;
   if (timed) WF_CUDA(cudaEventRecordWithFlags(P.tev[0 * C + slot], P.stream, cudaEventRecordExternal));
@@ -455,24 +459,35 @@ static wf_status enqueue_iteration(Plan &P, T2 *F, T2 *G, const double *data,
   if (timed) WF_CUDA(cudaEventRecordWithFlags(P.tev[5 * C + slot], P.stream, cudaEventRecordExternal));
   ++P.nlaunch;
   k_control<<<1, CTRL_THREADS, 0, P.stream>>>(P.state, P.partials, P.lmax, P.cl_d,
-                                              P.trace);
+                                              P.trace, loop);
   WF_CUDA(cudaGetLastError());
   return WF_OK;
 }
 
-// Iterations per graph launch: ~2^24 / Npix (fewer host polls for small
-// maps), at least 8 (at Nside 1024 a poll every ~11 ms of work instead of
-// every 2 iterations; iterations past `done` return at once).
+// Iterations per graph launch of a timed solve: ~2^24 / Npix (fewer host polls for
+// small maps), at least 8; iterations past `done` return at once.
 static int auto_chunk(const Plan &P) {
   long k = (1L << 24) / std::max(1L, P.npix);
   return (int)std::max(8L, std::min(128L, k));
+}
+
+// Iterations per pass of the device loop: the loop's own step costs ~2 us, an
+// iteration past `done` five launches that return at once (~8 us).  Runs of whole
+// stages and solves (graph 0) take up to 16, the short runs between anchors up to 4;
+// large maps 1.
+static int loop_unroll(const Plan &P, int which) {
+  const long most = which == 0 ? 16 : 4;
+  return (int)std::max(1L, std::min(most, most * (1L << 20) / std::max(1L, P.npix)));
 }
 
 template <typename T2>
 static wf_status capture_graph(Plan &P, int which, T2 *F, T2 *G, const double *data,
                                const double2 *src) {
   if (P.graph[which]) return WF_OK;
-  const int chunk = P.opts.graph_chunk > 0 ? P.opts.graph_chunk : auto_chunk(P);
+  const bool timed = P.opts.timing != 0;
+  const int chunk = P.opts.graph_chunk > 0 ? P.opts.graph_chunk
+                    : timed                ? auto_chunk(P)
+                                           : loop_unroll(P, which);
   cudaGraph_t g = nullptr;
   // capture on the plan's private stream (the caller's stream may be the
   // legacy default stream, which cannot be captured); launch on P.stream
@@ -490,6 +505,19 @@ static wf_status capture_graph(Plan &P, int which, T2 *F, T2 *G, const double *d
   }
   cudaStream_t user = P.stream;
   P.stream = P.capture_stream;
+  if (!timed) {  // one launch runs the iterations to the end, on the device
+    const long l0 = P.nlaunch;
+    const wf_status st = capture_loop(P.stream, &P.graph[which], [&](LoopHandle loop) {
+      for (int i = 0; i < chunk; ++i)
+        WF_TRY(enqueue_iteration<T2>(P, F, G, data, src, -1, loop));
+      return WF_OK;
+    });
+    P.graph_kernels[which] = P.nlaunch - l0;
+    P.nlaunch = l0;
+    P.stream = user;
+    P.graph_chunk[which] = chunk;
+    return st;
+  }
   cudaError_t eb = cudaStreamBeginCapture(P.stream, cudaStreamCaptureModeThreadLocal);
   if (eb != cudaSuccess) {
     P.stream = user;
@@ -499,7 +527,7 @@ static wf_status capture_graph(Plan &P, int which, T2 *F, T2 *G, const double *d
   wf_status s = WF_OK;
   const long n0 = P.nlaunch;
   for (int i = 0; i < chunk && s == WF_OK; ++i)
-    s = enqueue_iteration<T2>(P, F, G, data, src, P.opts.timing ? i : -1);
+    s = enqueue_iteration<T2>(P, F, G, data, src, i, LoopHandle{});
   P.graph_kernels[which] = P.nlaunch - n0;  // nodes of the graph, not yet run
   P.nlaunch = n0;
   cudaError_t e = cudaStreamEndCapture(P.stream, &g);
@@ -543,10 +571,12 @@ static wf_status run_loop(Plan &P, int which, T2 *F, T2 *G, const double *tinit,
   int it0 = P.state_h->iter;
   for (;;) {
     WF_CUDA(cudaGraphLaunch(P.graph[which], P.stream));
-    P.nlaunch += P.graph_kernels[which];
     WF_CUDA(cudaMemcpyAsync(P.state_h, P.state, sizeof(SolverState),
                             cudaMemcpyDeviceToHost, P.stream));
     WF_CUDA(cudaStreamSynchronize(P.stream));
+    const int chunk = P.graph_chunk[which];
+    const int passes = P.opts.timing ? 1 : (P.state_h->iter - it0 + chunk - 1) / chunk;
+    P.nlaunch += passes * P.graph_kernels[which];
     if (P.opts.timing && timed) {
       // iterations that did work in this launch: the first (iter - it0)
       const int active = std::min(P.state_h->iter - it0, P.graph_chunk[which]);

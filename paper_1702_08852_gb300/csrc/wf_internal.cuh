@@ -244,7 +244,7 @@ struct Plan {
   // graphs (one per precision), captured lazily
   // 0: FP64 with data, 1: FP32 with data, 2: FP32 correction (harmonic source)
   cudaGraphExec_t graph[3] = {nullptr, nullptr, nullptr};
-  int graph_chunk[3] = {0, 0, 0};
+  int graph_chunk[3] = {0, 0, 0};  // iterations per launch (opts.timing) or loop pass
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
 
   // kernel launches issued for this plan (graph launches count their kernel
@@ -389,9 +389,54 @@ wf_status pcg(Plan &P, const double *d, double *alm, double *map, double tol, in
 // j <= nslots - 1 (passed as lmax), stage test, cooling, trace; cl may be
 // NULL when the state's band_limit is 0
 constexpr int CONTROL_THREADS = 256;
+// the condition of a graph's loop node, which k_control ends when it sets `done`
+struct LoopHandle {
+  cudaGraphConditionalHandle h{};
+  int on = 0;
+};
 __global__ void __launch_bounds__(CONTROL_THREADS)
     k_control(SolverState *st, const double *__restrict__ partials, int lmax,
-              const double *__restrict__ cl, TraceEntry *trace);
+              const double *__restrict__ cl, TraceEntry *trace, LoopHandle loop);
+
+// Captures `pass` (the launches of one loop pass, on `stream`) as the body of a
+// while node and instantiates the graph: one launch iterates on the device until
+// k_control sets `done` (every run ends at max_iter).
+template <typename Pass>
+wf_status capture_loop(cudaStream_t stream, cudaGraphExec_t *out, Pass pass) {
+  cudaGraph_t g = nullptr, body = nullptr;
+  WF_CUDA(cudaGraphCreate(&g, 0));
+  LoopHandle loop;
+  loop.on = 1;
+  cudaError_t e = cudaGraphConditionalHandleCreate(&loop.h, g, 1, cudaGraphCondAssignDefault);
+  if (e == cudaSuccess) {
+    cudaGraphNodeParams np{};
+    np.type = cudaGraphNodeTypeConditional;
+    np.conditional.handle = loop.h;
+    np.conditional.type = cudaGraphCondTypeWhile;
+    np.conditional.size = 1;
+    cudaGraphNode_t node;
+    e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &np);
+    if (e == cudaSuccess) body = np.conditional.phGraph_out[0];
+  }
+  if (e == cudaSuccess)
+    e = cudaStreamBeginCaptureToGraph(stream, body, nullptr, nullptr, 0,
+                                      cudaStreamCaptureModeThreadLocal);
+  wf_status s = WF_OK;
+  if (e == cudaSuccess) {
+    s = pass(loop);
+    cudaGraph_t same = nullptr;
+    e = cudaStreamEndCapture(stream, &same);
+  }
+  if (s == WF_OK && e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
+  cudaGraphDestroy(g);
+  if (s != WF_OK) return s;
+  if (e != cudaSuccess) {
+    *out = nullptr;
+    set_error(std::string("graph capture: ") + cudaGetErrorString(e));
+    return WF_ERR_CUDA;
+  }
+  return WF_OK;
+}
 
 // helper kernels of solve.cu shared with noalloc.cu
 __global__ void k_mask_data(const double *d, const double *nvar, long npix, double *out);
