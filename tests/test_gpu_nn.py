@@ -117,3 +117,30 @@ def test_training_lowers_the_loss_and_warm_solve_is_exact(torch_cuda, osht, odm)
     a = alm.cpu().numpy()
     assert st["converged"] == 1
     assert osht.alm_norm(a - ref, p.lmax) / osht.alm_norm(ref, p.lmax) < 1e-9
+
+
+# the kernels' edges: a 15-tap window wider than the polar rings (4 pixels), more than
+# 256 (output, input) channel pairs, channel counts beside the groups of 8, a 1-tap
+# kernel, rings longer than one tile of the weight gradient (64 quads)
+@pytest.mark.parametrize("nside,H,K,Hm", [(2, 32, 15, 64), (3, 9, 1, 3), (70, 9, 7, 5)])
+def test_gradient_at_the_kernels_edges(torch_cuda, osht, nside, H, K, Hm):
+    torch = torch_cuda
+    from oracle import nn as onn
+    from paper_1702_08852_gb300 import inputs, wf
+    p = inputs.lognormal_problem(nside, lmax=min(2 * nside, 24), seed=7, band_deg=20.0, discs=3)
+    d = p.data(osht.alm2map(p.alm_true, p.nside, p.lmax))
+    _, n = onn.layout(H, K, Hm)
+    theta = (0.3 / np.sqrt(K) * np.random.default_rng(8).standard_normal(n)).astype(np.float32)
+    target = (0.8 * p.alm_true).astype(np.complex128)
+    nv = torch.from_numpy(p.noise_var).cuda()
+    mk = torch.from_numpy(p.mask.astype(np.uint8)).cuda()
+    with wf.Plan(p.nside, p.lmax, p.cl, nv, mk) as plan:
+        net = wf.Net(plan, H, K, Hm, bf16=False)
+        net.set_params(theta)
+        loss, g = net.loss_grad(torch.from_numpy(d).cuda(), torch.from_numpy(target).cuda(),
+                                want_grad=True)
+        net.close()
+    ref_loss, ref_g = onn.loss_grad(theta.astype(np.float64), H, K, Hm, p.nside, p.lmax, p.cl,
+                                    p.noise_var, p.mask, d, target)
+    assert loss == pytest.approx(ref_loss, rel=1e-5)
+    assert np.linalg.norm(g - ref_g) <= 1e-3 * np.linalg.norm(ref_g)
