@@ -18,12 +18,21 @@
 //   k_flat_rows  one row per CTA: inverse row FFT -> s, the pixel update ->
 //                t, forward row FFT for the next iteration.
 // Rows and columns are radix-2 FFTs in shared memory (n a power of two).
+//
+// A spectrum with C_k = C_-k (any isotropic one) keeps the maps' row transforms
+// Hermitian: the h kernels then hold only the n / 2 + 1 columns kx >= 0, transform two
+// real rows as one complex row, and keep the filtered spectrum and C in the
+// bit-reversed ky order that the forward column transform leaves, so no permutation
+// pass is made.  FP64 arithmetic (2 multiply-adds per clock and SM) bounds both forms:
+// per iteration at n = 256 it is ~9 us of the h form.  Other spectra run the general
+// kernels.
 #include <math.h>
 
 #include <algorithm>
 #include <string>
 #include <vector>
 
+#include "fft.cuh"
 #include "wf_internal.cuh"
 
 namespace wf {
@@ -170,9 +179,131 @@ __global__ void __launch_bounds__(FLAT_THREADS)
   for (int x = tid; x < n; x += FLAT_THREADS) T1[row + x] = buf[x];
 }
 
+// ------------------------------------------------------- Hermitian spectra
+// T1, T2: [row pair][kx <= n / 2][2 rows]; S and C: [kx][ky bit-reversed].
+//
+// Columns kx0 .. kx0 + cb - 1: as k_flat_cols; the columns 0 < kx < n / 2 stand for two
+// in the Cauchy sums.
+__global__ void __launch_bounds__(FLAT_THREADS)
+    k_flat_hcols(int n, int cb, double omega, const double *__restrict__ ck,
+                 const double2 *__restrict__ T1, double2 *__restrict__ S,
+                 double2 *__restrict__ T2, const double2 *__restrict__ tw,
+                 const SolverState *__restrict__ st, double *__restrict__ partials, int mode) {
+  extern __shared__ __align__(16) unsigned char flat_smem[];
+  double2 *buf = reinterpret_cast<double2 *>(flat_smem);  // [cb][n]
+  __shared__ double red[2][FLAT_THREADS / 32];
+  if (mode == FLAT_ITER && st->done) return;
+  const int nk = n / 2 + 1, kx0 = blockIdx.x * cb, nc = min(cb, nk - kx0);
+  const int tid = threadIdx.x, nt = blockDim.x;
+  if (mode == FLAT_ITER) {
+    for (int e = tid; e < nc * n; e += nt) {  // two rows of a column are adjacent
+      const int c = (e >> 1) % nc, y = (e >> 1) / nc * 2 + (e & 1);
+      buf[c * n + sw(y)] = T1[((long)(y >> 1) * nk + kx0 + c) * 2 + (y & 1)];
+    }
+    __syncthreads();
+    for (int c = 0; c < nc; ++c) fft_dif<double2, false>(buf + c * n, n, tw, n);
+    double num = 0.0, den = 0.0;
+    const double mo = st->mu * omega, xo = st->xi * omega;
+    for (int e = tid; e < nc * n; e += nt) {
+      const int c = e / n, q = e - c * n;
+      const long k = (long)(kx0 + c) * n + q;
+      const double sbar = fmax(ck[k] - mo, 0.0);
+      const double f = sbar > 0.0 ? sbar / (sbar + xo) : 0.0;
+      const double2 v = buf[c * n + sw(q)], old = S[k];
+      const double2 sh = make_double2(f * v.x, f * v.y);
+      const double dr = sh.x - old.x, di = sh.y - old.y;
+      const double w = kx0 + c == 0 || kx0 + c == nk - 1 ? 1.0 : 2.0;
+      num += w * (dr * dr + di * di);
+      den += w * (sh.x * sh.x + sh.y * sh.y);
+      S[k] = sh;
+      buf[c * n + sw(q)] = sh;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      num += __shfl_xor_sync(0xffffffffu, num, o);
+      den += __shfl_xor_sync(0xffffffffu, den, o);
+    }
+    if ((tid & 31) == 0) {
+      red[0][tid >> 5] = num;
+      red[1][tid >> 5] = den;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      for (int w = 1; w < nt / 32; ++w) {
+        num += red[0][w];
+        den += red[1][w];
+      }
+      partials[2 * blockIdx.x] = num;
+      partials[2 * blockIdx.x + 1] = den;
+    }
+  } else {
+    for (int e = tid; e < nc * n; e += nt) {
+      const int c = e / n, q = e - c * n;
+      buf[c * n + sw(q)] = S[(long)(kx0 + c) * n + q];
+    }
+    __syncthreads();
+  }
+  for (int c = 0; c < nc; ++c) fft_dit<double2, true>(buf + c * n, n, tw, n);
+  for (int e = tid; e < nc * n; e += nt) {
+    const int c = (e >> 1) % nc, y = (e >> 1) / nc * 2 + (e & 1);
+    T2[((long)(y >> 1) * nk + kx0 + c) * 2 + (y & 1)] = buf[c * n + sw(y)];
+  }
+}
+
+// Rows 2 r and 2 r + 1 as the real and imaginary part of one row: as k_flat_rows.
+__global__ void __launch_bounds__(FLAT_THREADS)
+    k_flat_hrows(int n, int logn, const double2 *__restrict__ T2, double2 *__restrict__ T1,
+                 const double *__restrict__ in, const double *__restrict__ d,
+                 const double *__restrict__ nvar, double *__restrict__ out,
+                 const double2 *__restrict__ tw, const SolverState *__restrict__ st, int mode) {
+  extern __shared__ __align__(16) unsigned char flat_smem[];
+  double2 *buf = reinterpret_cast<double2 *>(flat_smem);  // [n]
+  if (mode == FLAT_ITER && st->done) return;
+  const int nk = n / 2 + 1, tid = threadIdx.x, nt = blockDim.x;
+  const long row = 2L * blockIdx.x * n, trow = 2L * blockIdx.x * nk;
+  if (mode == FLAT_FWD) {
+    for (int x = tid; x < n; x += nt) buf[sw(x)] = make_double2(in[row + x], in[row + n + x]);
+    __syncthreads();
+  } else {
+    for (int k = tid; k < nk; k += nt) {
+      double2 a = T2[trow + 2 * k], b = T2[trow + 2 * k + 1];
+      if (k == 0 || k == n / 2) a.y = b.y = 0.0;  // real up to rounding
+      buf[sw(bitrev_n(k, logn))] = make_double2(a.x - b.y, a.y + b.x);
+      if (k > 0 && k < n / 2)
+        buf[sw(bitrev_n(n - k, logn))] = make_double2(a.x + b.y, b.x - a.y);
+    }
+    __syncthreads();
+    fft_dit<double2, true>(buf, n, tw, n);
+    const double scale = 1.0 / ((double)n * (double)n);
+    if (mode == FLAT_FINAL) {
+      for (int x = tid; x < n; x += nt) {
+        const double2 v = buf[sw(x)];
+        out[row + x] = v.x * scale;
+        out[row + n + x] = v.y * scale;
+      }
+      return;
+    }
+    const double xi = st->xi, mu = st->mu;
+    for (int x = tid; x < n; x += nt) {
+      const double2 v = buf[sw(x)];
+      const double s0 = v.x * scale, s1 = v.y * scale;
+      const double v0 = nvar[row + x], v1 = nvar[row + n + x];
+      const double w0 = isinf(v0) ? 0.0 : xi / (v0 + mu), w1 = isinf(v1) ? 0.0 : xi / (v1 + mu);
+      buf[sw(x)] = make_double2(s0 + w0 * (d[row + x] - s0), s1 + w1 * (d[row + n + x] - s1));
+    }
+    __syncthreads();
+  }
+  fft_dif<double2, false>(buf, n, tw, n);
+  for (int k = tid; k < nk; k += nt) {
+    const double2 z = buf[sw(bitrev_n(k, logn))], m = buf[sw(bitrev_n((n - k) & (n - 1), logn))];
+    T1[trow + 2 * k] = make_double2(0.5 * (z.x + m.x), 0.5 * (z.y - m.y));
+    T1[trow + 2 * k + 1] = make_double2(0.5 * (z.y + m.y), 0.5 * (m.x - z.x));
+  }
+}
+
 // ------------------------------------------------------------------ plan
 struct FlatPlan {
   int n = 0, logn = 0;
+  bool herm = false;  // C_k = C_-k: the h kernels
   double omega = 0.0, alpha = 0.0, ck_max = 0.0;
   wf_opts opts{};
   cudaStream_t stream = nullptr, capture_stream = nullptr;
@@ -225,15 +356,41 @@ static SolverState flat_initial_state(const FlatPlan &F) {
   return s;
 }
 
-static int flat_ncols(const FlatPlan &F) { return F.n / FLAT_CB; }
+// columns per CTA of the h kernel: one on small grids (more CTAs), two above (whole
+// 64-byte accesses)
+static int flat_cb(const FlatPlan &F) { return F.herm ? (F.n < 512 ? 1 : 2) : FLAT_CB; }
+static int flat_ncols(const FlatPlan &F) {
+  return F.herm ? (F.n / 2 + flat_cb(F)) / flat_cb(F) : F.n / FLAT_CB;
+}
+
+// the column kernel; st NULL: FLAT_FINAL
+static void flat_cols(FlatPlan &F, cudaStream_t s, const SolverState *st) {
+  const int mode = st ? FLAT_ITER : FLAT_FINAL;
+  ++F.nlaunch;
+  if (F.herm)
+    k_flat_hcols<<<flat_ncols(F), std::max(32, std::min(FLAT_THREADS, F.n / 4)), F.smem_cols, s>>>(
+        F.n, flat_cb(F), F.omega, F.ck, F.T1, F.S, F.T2, F.tw, st, F.partials, mode);
+  else
+    k_flat_cols<<<flat_ncols(F), FLAT_THREADS, F.smem_cols, s>>>(
+        F.n, F.logn, F.omega, F.ck, F.T1, F.S, F.T2, F.tw, st, F.partials, mode);
+}
+
+// the row kernel
+static void flat_rows(FlatPlan &F, cudaStream_t s, const double *in, double *out,
+                      const SolverState *st, int mode) {
+  ++F.nlaunch;
+  if (F.herm)
+    k_flat_hrows<<<F.n / 2, std::max(32, std::min(FLAT_THREADS, F.n / 4)), F.smem_rows, s>>>(
+        F.n, F.logn, F.T2, F.T1, in, F.d, F.nvar, out, F.tw, st, mode);
+  else
+    k_flat_rows<<<F.n, FLAT_THREADS, F.smem_rows, s>>>(F.n, F.logn, F.T2, F.T1, in, F.d, F.nvar,
+                                                       out, F.tw, st, mode);
+}
 
 static wf_status flat_enqueue_iteration(FlatPlan &F, cudaStream_t st, LoopHandle loop) {
-  F.nlaunch += 3;
-  k_flat_cols<<<flat_ncols(F), FLAT_THREADS, F.smem_cols, st>>>(
-      F.n, F.logn, F.omega, F.ck, F.T1, F.S, F.T2, F.tw, F.state, F.partials, FLAT_ITER);
-  k_flat_rows<<<F.n, FLAT_THREADS, F.smem_rows, st>>>(F.n, F.logn, F.T2, F.T1, nullptr, F.d,
-                                                      F.nvar, nullptr, F.tw, F.state,
-                                                      FLAT_ITER);
+  flat_cols(F, st, F.state);
+  flat_rows(F, st, nullptr, nullptr, F.state, FLAT_ITER);
+  ++F.nlaunch;
   k_control<<<1, CONTROL_THREADS, 0, st>>>(F.state, F.partials, flat_ncols(F) - 1, nullptr,
                                            F.trace, loop);
   WF_CUDA(cudaGetLastError());
@@ -266,10 +423,7 @@ static wf_status flat_solve(FlatPlan &F, const double *d, double *s_out, wf_stat
   WF_CUDA(cudaMemcpyAsync(F.state, F.state_h, sizeof(SolverState), cudaMemcpyHostToDevice,
                           F.stream));
   // t_0 = d: its row transforms
-  ++F.nlaunch;
-  k_flat_rows<<<F.n, FLAT_THREADS, F.smem_rows, F.stream>>>(F.n, F.logn, nullptr, F.T1, F.d,
-                                                            nullptr, nullptr, nullptr, F.tw,
-                                                            nullptr, FLAT_FWD);
+  flat_rows(F, F.stream, F.d, nullptr, nullptr, FLAT_FWD);
   WF_CUDA(cudaGetLastError());
   WF_TRY(flat_capture(F));
   WF_CUDA(cudaGraphLaunch(F.graph, F.stream));
@@ -278,12 +432,8 @@ static wf_status flat_solve(FlatPlan &F, const double *d, double *s_out, wf_stat
   WF_CUDA(cudaStreamSynchronize(F.stream));
   F.nlaunch += 3L * ((F.state_h->iter + F.chunk - 1) / F.chunk) * F.chunk;
   // s of the last iteration: the inverse transforms of its filtered spectrum
-  F.nlaunch += 2;
-  k_flat_cols<<<flat_ncols(F), FLAT_THREADS, F.smem_cols, F.stream>>>(
-      F.n, F.logn, F.omega, F.ck, F.T1, F.S, F.T2, F.tw, nullptr, nullptr, FLAT_FINAL);
-  k_flat_rows<<<F.n, FLAT_THREADS, F.smem_rows, F.stream>>>(F.n, F.logn, F.T2, F.T1, nullptr,
-                                                            nullptr, nullptr, s_out, F.tw,
-                                                            nullptr, FLAT_FINAL);
+  flat_cols(F, F.stream, nullptr);
+  flat_rows(F, F.stream, nullptr, s_out, nullptr, FLAT_FINAL);
   WF_CUDA(cudaGetLastError());
   WF_CUDA(cudaEventRecord(F.ev1, F.stream));
   WF_CUDA(cudaStreamSynchronize(F.stream));
@@ -369,7 +519,21 @@ wf_status wf_flat_plan(wf_flat_t *out, int n, double pixel_area, const double *c
   F->ck_max = cmax;
   F->stream = static_cast<cudaStream_t>(stream);
   F->trace_cap = 1 << 20;
-  F->smem_cols = sizeof(double2) * FLAT_CB * n;
+  F->herm = true;
+  for (int y = 0; y < n && F->herm; ++y)
+    for (int x = 0; x <= n / 2 && F->herm; ++x)
+      F->herm = ck[(long)y * n + x] == ck[(long)((n - y) & (n - 1)) * n + ((n - x) & (n - 1))];
+  if (F->herm) {  // [kx][ky bit-reversed]
+    std::vector<double> h(n2, 0.0);
+    for (int x = 0; x <= n / 2; ++x)
+      for (int y = 0; y < n; ++y) {
+        int q = 0;
+        for (int b = 0; b < logn; ++b) q |= ((y >> b) & 1) << (logn - 1 - b);
+        h[(long)x * n + q] = ck[(long)y * n + x];
+      }
+    ck.swap(h);
+  }
+  F->smem_cols = sizeof(double2) * flat_cb(*F) * n;
   F->smem_rows = sizeof(double2) * n;
   auto fail = [&](const char *what, cudaError_t e) {
     set_error(std::string("wf_flat_plan: ") + what + ": " + cudaGetErrorString(e));
@@ -382,7 +546,7 @@ wf_status wf_flat_plan(wf_flat_t *out, int n, double pixel_area, const double *c
   for (double2 **b : {&F->T1, &F->T2, &F->S})
     if ((e = cudaMalloc(b, sizeof(double2) * n2)) != cudaSuccess) return fail("cudaMalloc", e);
   if ((e = cudaMalloc(&F->tw, sizeof(double2) * (n / 2))) != cudaSuccess ||
-      (e = cudaMalloc(&F->partials, sizeof(double) * 2 * (n / FLAT_CB))) != cudaSuccess ||
+      (e = cudaMalloc(&F->partials, sizeof(double) * 3 * (n / 2 + 1))) != cudaSuccess ||
       (e = cudaMalloc(&F->state, sizeof(SolverState))) != cudaSuccess ||
       (e = cudaMallocHost(&F->state_h, sizeof(SolverState))) != cudaSuccess ||
       (e = cudaMalloc(&F->trace, sizeof(TraceEntry) * F->trace_cap)) != cudaSuccess ||
@@ -390,8 +554,12 @@ wf_status wf_flat_plan(wf_flat_t *out, int n, double pixel_area, const double *c
       (e = cudaEventCreate(&F->ev1)) != cudaSuccess)
     return fail("allocation", e);
   if (F->smem_cols > 48 * 1024 &&
-      (e = cudaFuncSetAttribute(k_flat_cols, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)F->smem_cols)) != cudaSuccess)
+      (e = F->herm ? cudaFuncSetAttribute(k_flat_hcols,
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)F->smem_cols)
+                   : cudaFuncSetAttribute(k_flat_cols,
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)F->smem_cols)) != cudaSuccess)
     return fail("shared memory attribute", e);
   // twiddles e^{-2 pi i k / n}: sin and cos of pi (2k / n), exact argument
   std::vector<double2> tw(n / 2);

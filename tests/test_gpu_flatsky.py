@@ -94,3 +94,18 @@ def test_plan_rejects_bad_arguments(torch_cuda):
     nv[5] = 0.0
     with pytest.raises(wf.WFError):
         wf.FlatPlan(8, 1e-6, np.ones(64), nv)            # zero variance
+
+
+@pytest.mark.parametrize("n", [8, 16, 512])
+@pytest.mark.parametrize("symmetric", [True, False])
+def test_both_kernel_forms_closed_form(torch_cuda, ofs, n, symmetric):
+    """Uniform noise: the last stage has t = d, so s = Re ifft2(f fft2(d)).  A spectrum
+    with C_k = C_-k runs the half-spectrum kernels (the smallest grid, an odd number of
+    column CTAs, two columns per CTA), any other one the general kernels."""
+    d, nv, ck, om = setup(ofs, n, n + 7, side_deg=n * 10.0 / 256, uniform=True)
+    if not symmetric:
+        ck = ck * (1.0 + 0.5 * np.random.default_rng(1).random((n, n)))
+    s, st, _ = gpu(torch_cuda, n, om, ck, nv, d, eps_final=1e-12)
+    want = np.real(np.fft.ifft2(ck / (ck + 64.0 * om) * np.fft.fft2(d)))
+    assert st["converged"] == 1
+    assert rel(s, want) < 1e-12
