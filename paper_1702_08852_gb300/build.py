@@ -14,7 +14,7 @@ CSRC = os.path.join(PKG, "csrc")
 OUT = os.path.join(PKG, "_lib")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(OUT, "libwf.so")
-SOURCES = ["plan.cu", "legendre.cu", "legpair.cu", "ringfft.cu", "solve.cu", "capi.cu", "noalloc.cu", "autotune.cu", "batch.cu", "nn.cu", "peak.cu", "pcg.cu", "flatsky.cu", "group.cu"]
+SOURCES = ["plan.cu", "legpair.cu", "ringfft.cu", "solve.cu", "capi.cu", "noalloc.cu", "autotune.cu", "batch.cu", "nn.cu", "peak.cu", "pcg.cu", "flatsky.cu", "group.cu"]
 HEADERS = ["wf_internal.cuh", "tc05.cuh", "fft.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC",

@@ -31,15 +31,13 @@ static void free_plan(wf_plan_s *P) {
   free_pair_tables(*P);
   for (int i = 0; i < 3; ++i)
     if (P->graph[i]) cudaGraphExecDestroy(P->graph[i]);
-  void *bufs[] = {P->pairs, P->cl_d,   P->rc,      P->rg,     P->seed_l,
-                  P->seed_u, P->tw64,  P->tw32,    P->chirp64, P->chirp32, P->bhat64,
+  void *bufs[] = {P->pairs, P->cl_d,   P->tw64,  P->tw32,    P->chirp64, P->chirp32, P->bhat64,
                   P->bhat32, P->nvar,  P->F64,     P->G64,    P->F32,    P->G32,
                   P->x,      P->xtmp,  P->dmap,    P->mtmp,   P->partials, P->red,
                   P->state,  P->trace, P->xacc,  P->src, P->xs64, P->xs32,
-                  P->nvar32, P->dmap32, P->ana_scratch, P->ana_lstart,
-                  P->ana_counter, P->uacc[0], P->uacc[1],
+                  P->nvar32, P->dmap32, P->uacc[0], P->uacc[1],
                   P->cl32, P->twdd, P->chirpdd, P->bhatdd,
-                  P->phasedd, P->rcdd, P->nvardd, P->dmapdd};
+                  P->phasedd, P->nvardd, P->dmapdd};
   for (void *b : bufs)
     if (b) cudaFree(b);
   if (P->state_h) cudaFreeHost(P->state_h);
@@ -73,18 +71,6 @@ static wf_status alloc_work(Plan &P) {
   WF_CUDA(cudaMalloc(&P.dmap, sizeof(double) * P.npix));
   WF_CUDA(cudaMalloc(&P.dmap32, sizeof(float) * P.npix));
   WF_CUDA(cudaMalloc(&P.dmapdd, sizeof(float2) * P.npix));
-  {
-    // queue-scheduled FP32 analysis: partial sums of tiles of 128 ring pairs
-    // (the smallest tile of its variants)
-    const long tiles = (P.npairs + 127) / 128;
-    // 16 bytes per entry: FP32 complex for the FP32 kernels, FP64 complex
-    // for the double-float anchor analysis
-    // (and the packed analysis' global accumulators: 4 warps x FP32 complex)
-    WF_CUDA(cudaMalloc(&P.ana_scratch, sizeof(double2) * std::max(tiles, 2L) * P.nalm));
-    WF_CUDA(cudaMalloc(&P.ana_lstart, sizeof(int) * tiles * (P.lmax + 1)));
-    WF_CUDA(cudaMalloc(&P.ana_counter, sizeof(int)));
-    WF_CUDA(cudaMemsetAsync(P.ana_counter, 0, sizeof(int), P.stream));
-  }
   WF_CUDA(cudaMalloc(&P.mtmp, sizeof(double) * P.npix));
   // per m: ||x_new - x_old||^2, ||x_new||^2, then (anchored stages) ||x_a + delta||^2
   WF_CUDA(cudaMalloc(&P.partials, sizeof(double) * 3 * (P.lmax + 1)));

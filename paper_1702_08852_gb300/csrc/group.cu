@@ -3,7 +3,7 @@
 //
 // For one m the Legendre step of every map of the group is one dense
 // product (Sect. 2.2's Y and Omega Y^T, split by the parity of l - m as in
-// legendre.cu):
+// legpair.cu):
 //   analysis   a_lm[b] = Omega sum_k lam_lm(z_k) P^p_m[k][b],
 //              P^p_m = G_N[m] + (-1)^p G_S[m]                 (p = (l-m) & 1)
 //              -> (rows l) x (K = ring pairs) times (K x N),
@@ -110,54 +110,58 @@ struct GroupState {
 };
 
 // ------------------------------------------------------------- table build
-// lam_lm(z_k) from the FP64 recurrence of the plan's tables (u from the
-// seeds at seed_l, lam = g u; lam = 0 below the seed, |lam| < 2^-100 there),
-// split and scattered into both tables.  One thread per (m, pair).
-__global__ void k_group_tables(const RingPair *__restrict__ pairs, int npairs, int lmax,
-                               const double *__restrict__ rc, const double *__restrict__ rg,
-                               const int *__restrict__ seed_l,
-                               const double2 *__restrict__ seed_u,
+// lam_lm(z_k) in FP64 from the plan's parity-pair tables (two l per step, from the
+// seeds; 0 below them, where |lam| < 2^-100), split and scattered into both tables.  One
+// thread per (m, pair).
+__global__ void k_group_tables(const PairTab<double> t, int npairs, int lmax,
                                const GItem *__restrict__ ana, const int *__restrict__ ana_first,
                                const GItem *__restrict__ syn, const int *__restrict__ syn_first,
                                int k8, float *ta_hi, float *ta_lo, float *ts_hi, float *ts_lo) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   if (k >= npairs) return;
-  const long mk = (long)m * npairs + k;
-  const int ls = seed_l[mk];
-  if (ls > lmax) return;
-  const double2 su = seed_u[mk];
-  const double z = pairs[k].z;
+  const int J = (lmax - m) / 2 + 1, js = t.js[(long)m * t.stride + k];
+  if (js >= J) return;
+  const long q0 = pair_base(lmax, m);
+  const double2 sd = t.seed[(long)m * t.stride + k];
+  const double z = t.z[k];
+  const int form = t.form(k);
+  const double w = t.w[form * t.stride + k];
+  const double2 *rec = t.rec[form] + q0;
   // analysis: column k % GKC of chunk k / GKC
   const int ca = k / GKC, ja = k % GKC, kca = min(GKC, k8 - GKC * ca);
   // synthesis: row k % 128 of pair tile k / 128
   const int ts = k / GT, is = k % GT;
-  double u1 = 0.0, u2 = 0.0;
-  for (int l = ls; l <= lmax; ++l) {
-    const long i = glm_index(lmax, l, m);
-    double u;
-    if (l == ls) u = su.x;
-    else if (l == ls + 1) u = su.y;
-    else u = fma(rc[i] * z, u1, -u2);
-    u2 = u1;
-    u1 = u;
-    const double lam = rg[i] * u;
-    const float hi = tf32_trunc((float)lam);
-    const float lo = tf32_trunc((float)(lam - (double)hi));
-    const int p = (l - m) & 1, j = (l - m - p) >> 1;
-    {
-      const GItem &it = ana[ana_first[m] + j / GT];
-      const long o = it.a_off[p] + (long)ca * it.r8[p] * GKC + core_off(j % GT, ja, kca);
-      ta_hi[o] = hi;
-      ta_lo[o] = lo;
-    }
-    {
-      const GItem &it = syn[syn_first[m] + ts];
-      const int kp = it.k[p];
-      const int c = j / GKC, kc = min(GKC, kp - GKC * c);
-      const long o = it.a_off[p] + (long)c * it.r8[p] * GKC + core_off(is, j % GKC, kc);
-      ts_hi[o] = hi;
-      ts_lo[o] = lo;
+  double s1 = 0.0, s2 = 0.0;
+  for (int j = js; j < J; ++j) {
+    double s;
+    if (j == js) s = sd.x;
+    else if (j == js + 1) s = sd.y;
+    else s = fma(fma(rec[j].x, w, rec[j].y), s1, s2);
+    const double even = j > js ? fma(t.sn[q0 + j - 1], s1, t.se[q0 + j] * s) : t.se[q0 + j] * s;
+    const double odd = z * (t.so[q0 + j] * s);
+    s2 = s1;
+    s1 = s;
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      if (m + 2 * j + p > lmax) break;
+      const double lam = p ? odd : even;
+      const float hi = tf32_trunc((float)lam);
+      const float lo = tf32_trunc((float)(lam - (double)hi));
+      {
+        const GItem &it = ana[ana_first[m] + j / GT];
+        const long o = it.a_off[p] + (long)ca * it.r8[p] * GKC + core_off(j % GT, ja, kca);
+        ta_hi[o] = hi;
+        ta_lo[o] = lo;
+      }
+      {
+        const GItem &it = syn[syn_first[m] + ts];
+        const int kp = it.k[p];
+        const int c = j / GKC, kc = min(GKC, kp - GKC * c);
+        const long o = it.a_off[p] + (long)c * it.r8[p] * GKC + core_off(is, j % GKC, kc);
+        ts_hi[o] = hi;
+        ts_lo[o] = lo;
+      }
     }
   }
 }
@@ -534,8 +538,7 @@ static wf_status build_group(Plan &P) {
                                (int)smem_bytes(2 * G_MAX_MAPS)));
   dim3 grid((P.npairs + 127) / 128, L + 1);
   ++P.nlaunch;
-  k_group_tables<<<grid, 128, 0, P.stream>>>(P.pairs, P.npairs, L, P.rc, P.rg, P.seed_l,
-                                             P.seed_u, g->ana, g->ana_first, g->syn,
+  k_group_tables<<<grid, 128, 0, P.stream>>>(P.pt64, P.npairs, L, g->ana, g->ana_first, g->syn,
                                              g->syn_first, g->k8, g->ta_hi, g->ta_lo,
                                              g->ts_hi, g->ts_lo);
   WF_CUDA(cudaGetLastError());

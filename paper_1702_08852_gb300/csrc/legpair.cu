@@ -46,6 +46,9 @@
 // at Nside 1024; measured 0.435 ms (synthesis, from 0.645) and 0.597 ms (analysis,
 // from 0.891), at Nside 256 17.7 and 23 us (from 23 and 38): what is left is the
 // reductions, the loads between the blocks and, on small maps, the largest m's chain.
+// Double-float (84 FP32 operations per step against 116 for two l of the one-step
+// recurrence): Nside 512 synthesis 0.63 ms (0.76), analysis 0.92 ms (0.97 and a combine
+// pass of 0.04), bound by the FP32 pipe's dependent chains at 16 warps per SM.
 //
 // Checkpoints: ck[(block b of 16 j of m)][pair] holds (s_{16b-1}, s_{16b-2}), so any 16
 // j can be computed on their own: a warp of the analysis owns 16 j of one m, keeps
@@ -70,12 +73,7 @@ namespace wf {
 namespace {
 
 // ------------------------------------------------------------- indexing
-// j of one m: J = (L - m) / 2 + 1; first table entry of m: sum of J over the
-// smaller m.  Blocks of 16 j of one m: (L - m) / 32 + 1.
-__host__ __device__ __forceinline__ long tri_j(long n) { return n + 1 + (n * n) / 4; }
-__host__ __device__ __forceinline__ long pair_base(int lmax, int m) {
-  return tri_j(lmax) - tri_j(lmax - m);
-}
+// blocks of 16 j of one m: (L - m) / 32 + 1
 __host__ __device__ __forceinline__ long tri_b(long n) {
   const long q = (n + 1) / 32, r = (n + 1) % 32;  // t = 0 .. n: sum of t / 32 + 1
   return n + 1 + 16 * q * (q - 1) + q * r;
@@ -91,6 +89,7 @@ __device__ __forceinline__ long alm_base(int lmax, int m) {  // index of (m, m)
 template <typename V> struct Cx;  // complex element of F, G and the alm input
 template <> struct Cx<double> { typedef double2 type; };
 template <> struct Cx<float> { typedef float2 type; };
+template <> struct Cx<dd> { typedef PairVec<dd>::type type; };
 template <typename V> struct alignas(16) Quad { V a, b, c, d; };
 template <typename V> struct alignas(2 * sizeof(V)) Pair { V a, b; };
 
@@ -109,6 +108,79 @@ __device__ __forceinline__ void fma2(float &dx, float &dy, float ax, float ay, f
       : "f"(ax), "f"(ay), "f"(bx), "f"(by), "f"(cx), "f"(cy));
 }
 
+// ------------------------------------------------------------- double-float
+// dd: an unevaluated sum hi + lo of two floats (~48-bit significand), products by the
+// FMA two-product, sums by two-sum (Dekker, Knuth); explicit _rn intrinsics, so nothing
+// is contracted or reassociated.  The anchors of the mixed solver need the FP64
+// iteration map to ~1e-10, not to FP64's last bit, and this part's FP64 unit runs at
+// ~1/64 of its FP32 rate.
+__device__ __forceinline__ dd dd_of(double x) {
+  const float h = (float)x;
+  return {h, (float)(x - (double)h)};
+}
+__device__ __forceinline__ double dd_val(dd a) { return (double)a.hi + (double)a.lo; }
+// (s, e) with |s| >= |e| -> normalised pair
+__device__ __forceinline__ dd dd_quick(float s, float e) {
+  const float h = __fadd_rn(s, e);
+  return {h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+// a b and the rounding error of the float product
+__device__ __forceinline__ void dd_prod(dd a, dd b, float &p, float &e) {
+  p = __fmul_rn(a.hi, b.hi);
+  e = fmaf(a.hi, b.hi, -p);
+  e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
+}
+__device__ __forceinline__ float two_sum(float a, float b, float &err) {
+  const float s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  return s;
+}
+__device__ __forceinline__ dd operator+(dd a, dd b) {
+  float err;
+  const float s = two_sum(a.hi, b.hi, err);
+  return dd_quick(s, __fadd_rn(err, __fadd_rn(a.lo, b.lo)));
+}
+__device__ __forceinline__ dd operator-(dd a, dd b) { return a + dd{-b.hi, -b.lo}; }
+__device__ __forceinline__ dd operator*(dd a, dd b) {
+  float p, e;
+  dd_prod(a, b, p, e);
+  return dd_quick(p, e);
+}
+__device__ __forceinline__ dd fmav(dd a, dd b, dd c) {
+  float p, e, err;
+  dd_prod(a, b, p, e);
+  const float s = two_sum(p, c.hi, err);
+  return dd_quick(s, __fadd_rn(__fadd_rn(e, c.lo), err));
+}
+// a b + c without the last normalisation: the factor of the next product
+__device__ __forceinline__ dd coefv(dd a, dd b, dd c) {
+  float p, e, err;
+  dd_prod(a, b, p, e);
+  const float s = two_sum(p, c.hi, err);
+  return {s, __fadd_rn(__fadd_rn(e, c.lo), err)};
+}
+// acc += s x, acc kept unnormalised (hi the running sum, lo the rounding errors)
+__device__ __forceinline__ void accv(dd &acc, dd s, dd x) {
+  float p, e, err;
+  dd_prod(s, x, p, e);
+  acc.hi = two_sum(acc.hi, p, err);
+  acc.lo = __fadd_rn(acc.lo, __fadd_rn(err, e));
+}
+__device__ __forceinline__ double coefv(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float coefv(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double shfx(double v, int s) { return __shfl_xor_sync(0xffffffffu, v, s); }
+__device__ __forceinline__ float shfx(float v, int s) { return __shfl_xor_sync(0xffffffffu, v, s); }
+__device__ __forceinline__ dd shfx(dd v, int s) { return {shfx(v.hi, s), shfx(v.lo, s)}; }
+// a checkpoint in the kernel's arithmetic (the dd kernels read the FP64 ones)
+template <typename V, typename W>
+__device__ __forceinline__ typename Cx<V>::type state_as(W v) {
+  if constexpr (std::is_same<V, dd>::value)
+    return {dd_of(v.x), dd_of(v.y)};
+  else
+    return v;
+}
+
 __device__ __forceinline__ int wmin(int v) { return __reduce_min_sync(0xffffffffu, v); }
 __device__ __forceinline__ int wmax(int v) { return __reduce_max_sync(0xffffffffu, v); }
 
@@ -122,7 +194,7 @@ __device__ __forceinline__ V lane_sums(V *v, int lane) {
     for (int j = 0; j < s; ++j) {
       const V send = upper ? v[j] : v[j + s];
       const V keep = upper ? v[j + s] : v[j];
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+      v[j] = keep + shfx(send, s);
     }
   }
   return v[0];
@@ -176,7 +248,7 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
 #pragma unroll
   for (int i = 0; i < NP; ++i) {  // in flight while the coefficients are staged
     const int k = pair0 + lane + 32 * i;
-    w[i] = (V)0;
+    w[i] = V(0);
     js[i] = INT_MAX / 2;
     if (k < npairs) {
       w[i] = wt[k];
@@ -226,7 +298,7 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
       const int k = pair0 + lane + 32 * i;
-      u[i] = o[i] = er[i] = ei[i] = orr[i] = oi[i] = z[i] = (V)0;
+      u[i] = o[i] = er[i] = ei[i] = orr[i] = oi[i] = z[i] = V(0);
       if (k < npairs) {
         z[i] = t.z[k];
         u[i] = t.lmm[(long)m * npairs + k];  // lam_mm
@@ -260,9 +332,9 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
     const int k = pair0 + lane + 32 * i;
-    s1[i] = s2[i] = d0[i] = d1[i] = er[i] = ei[i] = orr[i] = oi[i] = (V)0;
+    s1[i] = s2[i] = d0[i] = d1[i] = er[i] = ei[i] = orr[i] = oi[i] = V(0);
     if (js[i] < J) {
-      const C s = t.seed[(long)m * t.stride + k];
+      const C s = state_as<V>(t.seed[(long)m * t.stride + k]);
       d0[i] = s.x;
       d1[i] = s.y;
       jmin = min(jmin, js[i]);
@@ -306,7 +378,7 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
       const Quad<V> q = sx[jj];
 #pragma unroll
       for (int i = 0; i < NP; ++i) {
-        V s = fmav(fmav(r.a, w[i], r.b), s1[i], s2[i]);
+        V s = fmav(coefv(r.a, w[i], r.b), s1[i], s2[i]);
         if (inj) {
           s = jj == js[i] ? d0[i] : s;
           s = jj == js[i] + 1 ? d1[i] : s;
@@ -348,31 +420,33 @@ constexpr int CKJ = 16;
 // FP32 the real and the imaginary sum of one parity are one packed accumulator.
 // INJ: a pair's seeds c may enter, at step `rel` and the next (else c is the state
 // before the block), and the pairs may differ in their form (table sr[i]).
-template <typename V, int R, bool INJ>
-__device__ __forceinline__ void pair_block(V (&v)[4 * CKJ], const Pair<V> *const (&sr)[R],
+// SKIP: the sums start there (NJ of them).
+template <typename V, int R, bool INJ, int NJ, int SKIP>
+__device__ __forceinline__ void pair_block(V (&v)[4 * NJ], const Pair<V> *const (&sr)[R],
                                            const V (&w)[R], const typename Cx<V>::type (&c)[R],
                                            const Quad<V> (&p)[R], const int (&rel)[R]) {
   V s1[R], s2[R];
 #pragma unroll
   for (int i = 0; i < R; ++i) {
     const bool inj = INJ && (unsigned)rel[i] < (unsigned)CKJ;
-    s1[i] = inj ? (V)0 : c[i].x;
-    s2[i] = inj ? (V)0 : c[i].y;
+    s1[i] = inj ? V(0) : c[i].x;
+    s2[i] = inj ? V(0) : c[i].y;
   }
 #pragma unroll
-  for (int jj = 0; jj < CKJ; ++jj) {
+  for (int jj = 0; jj < NJ + SKIP; ++jj) {
     Pair<V> r = sr[0][jj];
 #pragma unroll
     for (int i = 0; i < R; ++i) {
       if (INJ && i > 0) r = sr[i][jj];
-      V s = fmav(fmav(r.a, w[i], r.b), s1[i], s2[i]);
+      V s = fmav(coefv(r.a, w[i], r.b), s1[i], s2[i]);
       if (INJ) {
         s = jj == rel[i] ? c[i].x : s;
         if (jj > 0) s = jj == rel[i] + 1 ? c[i].y : s;
       }
       s2[i] = s1[i];
       s1[i] = s;
-      V *x = v + 4 * jj;
+      if (jj < SKIP) continue;
+      V *x = v + 4 * (jj - SKIP);
       if constexpr (std::is_same<V, float>::value) {
         fma2(x[0], x[1], s, s, p[i].a, p[i].b, x[0], x[1]);
         fma2(x[2], x[3], s, s, p[i].c, p[i].d, x[2], x[3]);
@@ -486,16 +560,33 @@ __device__ __forceinline__ void pair_partials(double num, double den, double dx,
   }
 }
 
+// the epilogue's tables and sums: the kernel's own arithmetic, or (dd) FP64
+template <typename E>
+__device__ __forceinline__ const E *epi(const E *own, const double *) { return own; }
+template <typename E>
+__device__ __forceinline__ const E *epi(const dd *, const double *f64) { return f64; }
+template <typename E> __device__ __forceinline__ E epi_val(E v) { return v; }
+template <typename E> __device__ __forceinline__ double epi_val(dd v) { return dd_val(v); }
+
 template <typename V>
-__global__ void __launch_bounds__(32 * PANA_MAXWARPS, sizeof(V) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(32 * PANA_MAXWARPS, std::is_same<V, double>::value ? 1 : 2)
     k_pair_anal(const PairTab<V> t, int npairs, int lmax,
                 const double *__restrict__ cl, double omega,
                 const typename Cx<V>::type *__restrict__ G, double2 *__restrict__ x,
                 double *__restrict__ partials, const double2 *__restrict__ src,
                 typename Cx<V>::type *__restrict__ xs, const float *__restrict__ cl32,
-                const SolverState *__restrict__ st, int mode, int lstatic) {
+                const double *__restrict__ se64, const double *__restrict__ sn64,
+                const double *__restrict__ so64, const SolverState *__restrict__ st, int mode, int lstatic) {
   typedef typename Cx<V>::type C;
+  typedef typename CkVec<V>::type Ck;
   constexpr int R = std::is_same<V, float>::value ? 2 : 1;  // pairs in flight per lane
+  // where seeds may enter: FP32 the blocks in jin; dd the block of js, from the seed
+  // table (the FP64 state before it may be below FP32's range); FP64 none
+  constexpr bool DD = std::is_same<V, dd>::value, SEEDS = R == 2 || DD;
+  // j per warp item: dd halves a block (32 double-float sums leave room for 16 warps
+  // per SM, 64 for 8: 1.01 ms at Nside 512), the second half repeating the first's
+  // recurrence
+  constexpr int NJ = DD ? CKJ / 2 : CKJ, HALVES = CKJ / NJ;
   const int m = blockIdx.x;
   int L = lstatic;
   double xi = 0.0, mu = 0.0;
@@ -520,43 +611,48 @@ __global__ void __launch_bounds__(32 * PANA_MAXWARPS, sizeof(V) == 4 ? 2 : 1)
     Quad<V> *sd = sp + tile;                                          // [J16]
     Pair<V> *srec = reinterpret_cast<Pair<V> *>(sd + J16);            // [3][J16]
     const long q0 = pair_base(lmax, m), cb = block_base(lmax, m);
-    for (int j = tid; j < J16; j += blockDim.x) sd[j] = {(V)0, (V)0, (V)0, (V)0};
+    for (int j = tid; j < J16; j += blockDim.x) sd[j] = {V(0), V(0), V(0), V(0)};
     for (int f = 0; f < 3; ++f)
       for (int j = tid; j < J16; j += blockDim.x) {
-        const Pair<V> zero = {(V)0, (V)0};
+        const Pair<V> zero = {V(0), V(0)};
         srec[f * J16 + j] = j < J ? reinterpret_cast<const Pair<V> *>(t.rec[f])[q0 + j] : zero;
       }
     for (int t0 = 0; t0 < npairs; t0 += PANA_TILE) {
       const int nt = min(PANA_TILE, npairs - t0);
       __syncthreads();  // the previous tile's reads are done
       for (int k = tid; k < (nt + 63) / 64 * 64; k += blockDim.x) {
-        Quad<V> q = {(V)0, (V)0, (V)0, (V)0};
+        Quad<V> q = {V(0), V(0), V(0), V(0)};
         if (k < nt) q = reinterpret_cast<const Quad<V> *>(G)[(long)m * npairs + t0 + k];
-        if (t0 + k == npairs - 1) q.c = q.d = (V)0;  // the equator
+        if (t0 + k == npairs - 1) q.c = q.d = V(0);  // the equator
         const V z = t.z[t0 + k];
         sp[k] = {q.a + q.c, q.b + q.d, z * (q.a - q.c), z * (q.b - q.d)};
       }
       __syncthreads();
       // js, the checkpoints and w are loaded one step (32 R pairs) ahead
-      const int *jrow = t.jin + (long)m * t.stride + t0 + lane;
-      for (int b = warp; b < nb; b += nwarps) {
-        const int j0 = b * CKJ;
-        const C *crow = t.ck + (cb + b) * t.stride + t0 + lane;
+      const int *jrow = (DD ? t.js : t.jin) + (long)m * t.stride + t0 + lane;
+      const Ck *srow = t.seed + (long)m * t.stride + t0 + lane;
+      for (int bh = warp; bh < HALVES * nb; bh += nwarps) {
+        const int b = bh / HALVES, j0 = b * CKJ;
+        const Ck *crow = t.ck + (cb + b) * t.stride + t0 + lane;
         int rel[R], form[R];
-        C c[R];
+        Ck c[R];
         V w[R];
         auto load = [&](int g) {
 #pragma unroll
           for (int i = 0; i < R; ++i) {
             form[i] = t.form(t0 + g + 32 * i);
-            rel[i] = R == 2 ? jrow[g + 32 * i] - j0 : -1;  // FP64: no seeds enter
+            rel[i] = SEEDS ? jrow[g + 32 * i] - j0 : -1;
             c[i] = crow[g + 32 * i];
+            if constexpr (DD) {
+              const Ck sd0 = srow[g + 32 * i];
+              if ((unsigned)rel[i] < (unsigned)CKJ) c[i] = sd0;
+            }
             w[i] = t.w[form[i] * t.stride + t0 + lane + g + 32 * i];
           }
         };
-        V v[4 * CKJ];
+        V v[4 * NJ];
 #pragma unroll
-        for (int i = 0; i < 4 * CKJ; ++i) v[i] = (V)0;
+        for (int i = 0; i < 4 * NJ; ++i) v[i] = V(0);
         // below its first warp of pairs a block is zero
         int g = max(0, t.gfirst[cb + b] - t0) / (32 * R) * (32 * R);
         if (g < nt) load(g);
@@ -571,39 +667,52 @@ __global__ void __launch_bounds__(32 * PANA_MAXWARPS, sizeof(V) == 4 ? 2 : 1)
           for (int i = 0; i < R; ++i) {
             sr[i] = srec + form[i] * J16 + j0;
             wc[i] = w[i];
-            d[i] = c[i];
+            d[i] = state_as<V>(c[i]);
             rl[i] = rel[i];
             p[i] = sp[g + 32 * i + lane];
             slow |= (unsigned)rel[i] < (unsigned)CKJ;
           }
           if (g + 32 * R < nt) load(g + 32 * R);
-          if (R == 2 && __any_sync(0xffffffffu, slow))
-            pair_block<V, R, true>(v, sr, wc, d, p, rl);
-          else
-            pair_block<V, R, false>(v, sr, wc, d, p, rl);
+          if constexpr (DD) {
+            if (bh & 1)
+              pair_block<V, R, true, NJ, NJ>(v, sr, wc, d, p, rl);
+            else
+              pair_block<V, R, true, NJ, 0>(v, sr, wc, d, p, rl);
+          } else {
+            if (R == 2 && __any_sync(0xffffffffu, slow))
+              pair_block<V, R, true, NJ, 0>(v, sr, wc, d, p, rl);
+            else
+              pair_block<V, R, false, NJ, 0>(v, sr, wc, d, p, rl);
+          }
         }
-        V *dd = reinterpret_cast<V *>(sd) + 4 * j0 + lane;
-        const V lo = lane_sums(v, lane), hi = lane_sums(v + 32, lane);
-        dd[0] += lo;
-        dd[32] += hi;
+        V *out = reinterpret_cast<V *>(sd) + 4 * (j0 + (bh % HALVES) * NJ) + lane;
+        const V lo = lane_sums(v, lane);
+        out[0] = out[0] + lo;
+        if constexpr (!DD) {
+          const V hi = lane_sums(v + 32, lane);
+          out[32] = out[32] + hi;
+        }
       }
     }
     __syncthreads();
     for (int i = tid; i <= L - m; i += blockDim.x) {
       const int j = i >> 1;
-      V sr, si;
+      // dd: back to l in FP64
+      typedef typename std::conditional<DD, double, V>::type E;
+      const E *fo = epi<E>(t.so, so64), *fe = epi<E>(t.se, se64), *fn = epi<E>(t.sn, sn64);
+      E sr, si;
       if (i & 1) {
-        const V f = t.so[q0 + j];
-        sr = f * sd[j].c;
-        si = f * sd[j].d;
+        const E f = fo[q0 + j];
+        sr = f * epi_val<E>(sd[j].c);
+        si = f * epi_val<E>(sd[j].d);
       } else {
-        const V f = t.se[q0 + j];
-        sr = f * sd[j].a;
-        si = f * sd[j].b;
+        const E f = fe[q0 + j];
+        sr = f * epi_val<E>(sd[j].a);
+        si = f * epi_val<E>(sd[j].b);
         if (j > 0) {
-          const V g = t.sn[q0 + j - 1];
-          sr = fmav(g, sd[j - 1].a, sr);
-          si = fmav(g, sd[j - 1].b, si);
+          const E g = fn[q0 + j - 1];
+          sr = fmav(g, epi_val<E>(sd[j - 1].a), sr);
+          si = fmav(g, epi_val<E>(sd[j - 1].b), si);
         }
       }
       if constexpr (std::is_same<V, float>::value)
@@ -675,8 +784,8 @@ wf_status launch_legendre_anal<double2>(const Plan &P, const double2 *G, double2
   ++P.nlaunch;
   const int warps = std::max(2, std::min(PANA_MAXWARPS, P.lmax / 32 + 1));
   k_pair_anal<double><<<P.lmax + 1, 32 * warps, anal_smem(8, P.npairs, P.lmax), P.stream>>>(
-      P.pt64, P.npairs, P.lmax, P.cl_d, P.omega, G, x, P.partials, src, nullptr, nullptr, st,
-      mode, lstatic);
+      P.pt64, P.npairs, P.lmax, P.cl_d, P.omega, G, x, P.partials, src, nullptr, nullptr,
+      nullptr, nullptr, nullptr, st, mode, lstatic);
   WF_CUDA(cudaGetLastError());
   return WF_OK;
 }
@@ -711,8 +820,75 @@ wf_status launch_legendre_anal<float2>(const Plan &P, const float2 *G, double2 *
   ++P.nlaunch;
   const int warps = std::max(2, std::min(PANA_MAXWARPS, P.lmax / 32 + 1));
   k_pair_anal<float><<<P.lmax + 1, 32 * warps, anal_smem(4, P.npairs, P.lmax), P.stream>>>(
-      P.pt32, P.npairs, P.lmax, P.cl_d, P.omega, G, x, P.partials, src, xs_out, P.cl32, st, mode,
+      P.pt32, P.npairs, P.lmax, P.cl_d, P.omega, G, x, P.partials, src, xs_out, P.cl32, nullptr,
+      nullptr, nullptr, st, mode, lstatic);
+  WF_CUDA(cudaGetLastError());
+  return WF_OK;
+}
+
+template <int NP>
+static void synth_dd(const Plan &P, const float4 *x, float4 *F, const SolverState *st,
+                     int lstatic) {
+  const int tile = PSYN_THREADS * NP;
+  const dim3 grid((P.npairs + tile - 1) / tile, P.lmax + 1);
+  typedef Cx<dd>::type C;
+  k_pair_synth<dd, NP><<<grid, PSYN_THREADS, synth_smem(8, P.lmax), P.stream>>>(
+      P.ptdd, P.npairs, P.lmax, reinterpret_cast<const C *>(x), reinterpret_cast<C *>(F), st,
       lstatic);
+}
+
+wf_status launch_legendre_synth_dd(const Plan &P, const float4 *xs, float4 *F,
+                                   const SolverState *st, int lstatic) {
+  ++P.nlaunch;
+  if (P.npairs >= 1024)
+    synth_dd<2>(P, xs, F, st, lstatic);
+  else
+    synth_dd<1>(P, xs, F, st, lstatic);
+  WF_CUDA(cudaGetLastError());
+  return WF_OK;
+}
+
+wf_status launch_legendre_anal_dd(const Plan &P, const float4 *G, double2 *x,
+                                  const SolverState *st, int mode, int lstatic,
+                                  const double2 *src) {
+  ++P.nlaunch;
+  typedef Cx<dd>::type C;
+  const int warps = std::max(2, std::min(PANA_MAXWARPS, P.lmax / 32 + 1));
+  k_pair_anal<dd><<<P.lmax + 1, 32 * warps, anal_smem(8, P.npairs, P.lmax), P.stream>>>(
+      P.ptdd, P.npairs, P.lmax, P.cl_d, P.omega, reinterpret_cast<const C *>(G), x, P.partials,
+      src, nullptr, nullptr, P.pt64.se, P.pt64.sn, P.pt64.so, st, mode, lstatic);
+  WF_CUDA(cudaGetLastError());
+  return WF_OK;
+}
+
+// FP64 coefficients in the synthesis' FP32
+__global__ void k_to_f32(const double2 *__restrict__ x, long n, float2 *__restrict__ xs) {
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long)gridDim.x * blockDim.x)
+    xs[i] = make_float2((float)x[i].x, (float)x[i].y);
+}
+
+wf_status launch_to_f32(const Plan &P, const double2 *x, float2 *xs) {
+  ++P.nlaunch;
+  const unsigned grid = (unsigned)std::min((P.nalm + 255) / 256, 8L * P.num_sms);
+  k_to_f32<<<grid, 256, 0, P.stream>>>(x, P.nalm, xs);
+  WF_CUDA(cudaGetLastError());
+  return WF_OK;
+}
+
+// FP64 coefficients in double-float, the dd synthesis' input
+__global__ void k_alm_to_dd(const double2 *__restrict__ x, long n, float4 *__restrict__ xs) {
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long)gridDim.x * blockDim.x) {
+    const dd re = dd_of(x[i].x), im = dd_of(x[i].y);
+    xs[i] = make_float4(re.hi, re.lo, im.hi, im.lo);
+  }
+}
+
+wf_status launch_prescale_dd(const Plan &P, const double2 *x, float4 *xs) {
+  ++P.nlaunch;
+  const unsigned grid = (unsigned)std::min((P.nalm + 255) / 256, 8L * P.num_sms);
+  k_alm_to_dd<<<grid, 256, 0, P.stream>>>(x, P.nalm, xs);
   WF_CUDA(cudaGetLastError());
   return WF_OK;
 }
@@ -731,6 +907,12 @@ wf_status init_pair_attributes() {
                                cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   WF_CUDA(cudaFuncSetAttribute(k_pair_synth<float, 4>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  WF_CUDA(cudaFuncSetAttribute(k_pair_synth<dd, 1>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  WF_CUDA(cudaFuncSetAttribute(k_pair_synth<dd, 2>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  WF_CUDA(cudaFuncSetAttribute(k_pair_anal<dd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               big));
   WF_CUDA(cudaFuncSetAttribute(k_pair_anal<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                big));
   WF_CUDA(cudaFuncSetAttribute(k_pair_anal<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -919,6 +1101,7 @@ __global__ void k_pair_lmm(int npairs, int lmax, int keq, const double *__restri
 }
 
 static wf_status build_pair_tables32(Plan &P, long nq);
+static wf_status build_pair_tables_dd(Plan &P, long nq);
 
 // The tables and the checkpoints.  mant, expo: lam_mm of every (m, pair).
 wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
@@ -988,7 +1171,7 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
   k_pair_walk<<<(unsigned)((n + 127) / 128), 128, 0, P.stream>>>(P.npairs, lmax, t, u, mant,
                                                                  expo);
   WF_CUDA(cudaGetLastError());
-  return WF_OK;
+  return build_pair_tables_dd(P, nq);
 }
 
 // FP32 copies of the FP64 tables
@@ -1021,7 +1204,50 @@ static wf_status build_pair_tables32(Plan &P, long nq) {
   return WF_OK;
 }
 
+// the FP64 tables as double-float pairs; js, the seeds and the checkpoints are shared
+__global__ void k_pair_split(const double *__restrict__ in, long n, dd *__restrict__ out) {
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long)gridDim.x * blockDim.x)
+    out[i] = dd_of(in[i]);
+}
+
+static wf_status build_pair_tables_dd(Plan &P, long nq) {
+  const PairTab<double> &t = P.pt64;
+  PairTab<dd> &u = P.ptdd;
+  auto split = [&P](auto **dst, const void *src, long n) {
+    WF_CUDA(cudaMalloc(dst, sizeof(dd) * n));
+    const unsigned grid = (unsigned)std::min((n + 255) / 256, 4096L);
+    k_pair_split<<<grid, 256, 0, P.stream>>>(static_cast<const double *>(src), n,
+                                             reinterpret_cast<dd *>(*dst));
+    WF_CUDA(cudaGetLastError());
+    return WF_OK;
+  };
+  for (int f = 0; f < 3; ++f) WF_TRY(split(&u.rec[f], t.rec[f], 2 * nq));
+  WF_TRY(split(&u.rec_e, t.rec_e, 2 * nq));
+  WF_TRY(split(&u.se, t.se, nq));
+  WF_TRY(split(&u.sn, t.sn, nq));
+  WF_TRY(split(&u.so, t.so, nq));
+  WF_TRY(split(&u.ge, t.ge, nq));
+  WF_TRY(split(&u.go, t.go, nq));
+  WF_TRY(split(&u.w, t.w, 3L * t.stride));
+  WF_TRY(split(&u.z, t.z, t.stride));
+  if (t.lmm) WF_TRY(split(&u.lmm, t.lmm, (long)P.npairs * (P.lmax + 1)));
+  u.stride = t.stride;
+  u.js = t.js;
+  u.seed = t.seed;
+  u.ck = t.ck;
+  u.gfirst = t.gfirst;
+  u.keq = t.keq;
+  for (int f = 0; f < 2; ++f) u.kform[f] = t.kform[f];
+  return WF_OK;
+}
+
 void free_pair_tables(Plan &P) {
+  PairTab<dd> &d = P.ptdd;
+  void *g[] = {d.rec[0], d.rec[1], d.rec[2], d.rec_e, d.se, d.sn, d.so, d.ge, d.go, d.w, d.z,
+               d.lmm};
+  for (void *p : g)
+    if (p) cudaFree(p);
   PairTab<float> &u = P.pt32;
   void *f[] = {u.rec[0], u.rec[1], u.rec[2], u.se, u.sn, u.so, u.w, u.z, u.ck, u.jin, u.seed};
   for (void *p : f)

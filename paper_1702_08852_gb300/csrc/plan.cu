@@ -8,16 +8,9 @@
 // z = 2 (2 nside - i)/(3 nside) starting at phi = 0 when i + nside is odd and
 // at pi/(4 nside) when it is even; the south half mirrors the north.
 //
-// Legendre functions: lam_lm(z) (Y_lm = lam_lm(cos theta) e^{i m phi}) obey
-// lam_l = a_l z lam_{l-1} - (a_l / a_{l-1}) lam_{l-2},
-// a_l = sqrt((4 l^2 - 1) / (l^2 - m^2)).  The kernels run the rescaled
-// variable u_l = lam_l / g_l with g_m = g_{m+1} = 1, g_l = (a_l/a_{l-1}) g_{l-2},
-// which obeys u_l = c_l z u_{l-1} - u_{l-2}, c_l = a_l g_{l-1} / g_l: one
-// multiply and one fused multiply-add per step.  The seed of each (m, ring)
-// is the first l at which |lam_lm| reaches 2^-100, with the two values
-// u_ls, u_ls+1 computed here in FP64 with an explicit power-of-two exponent
-// (lam_mm = (-1)^m sqrt((2m+1)!!/(4 pi (2m)!!)) sin^m theta underflows any
-// floating-point format at high m); terms below 2^-100 are dropped.
+// The Legendre tables are legpair.cu's; here only lam_mm = (-1)^m sqrt((2m+1)!! /
+// (4 pi (2m)!!)) sin^m theta, which underflows any floating-point format at high m, as
+// mantissa and power-of-two exponent.
 #include <math.h>
 
 #include <algorithm>
@@ -226,51 +219,6 @@ static wf_status make_fft_tables(Plan &P) {
 }
 
 // ---------------------------------------------------------------- Legendre
-static wf_status make_recurrence_tables(Plan &P) {
-  const int L = P.lmax;
-  std::vector<double> c(P.nalm, 0.0), g(P.nalm, 1.0);
-  for (int m = 0; m <= L; ++m) {
-    double a_prev = 0.0, g2 = 1.0, g1 = 1.0;  // g_{l-2}, g_{l-1}
-    for (int l = m; l <= L; ++l) {
-      long i = alm_idx(L, l, m);
-      if (l == m) {
-        g[i] = 1.0;
-        c[i] = 0.0;
-        continue;
-      }
-      double a = sqrt((4.0 * l * l - 1.0) / ((double)l * l - (double)m * m));
-      double gl;
-      if (l == m + 1) {
-        gl = 1.0;
-      } else {
-        gl = (a / a_prev) * g2;
-      }
-      g[i] = gl;
-      c[i] = a * g1 / gl;
-      a_prev = a;
-      g2 = g1;
-      g1 = gl;
-    }
-  }
-  WF_CUDA(cudaMalloc(&P.rc, sizeof(double) * P.nalm));
-  WF_CUDA(cudaMalloc(&P.rg, sizeof(double) * P.nalm));
-  {
-    // the double-float Legendre kernels' coefficient table (hi, lo)
-    std::vector<float2> cdd(P.nalm);
-    for (long i = 0; i < P.nalm; ++i) {
-      const float h = (float)c[i];
-      cdd[i] = make_float2(h, (float)(c[i] - (double)h));
-    }
-    WF_CUDA(cudaMalloc(&P.rcdd, sizeof(float2) * P.nalm));
-    WF_CUDA(cudaMemcpy(P.rcdd, cdd.data(), sizeof(float2) * P.nalm, cudaMemcpyHostToDevice));
-  }
-  WF_CUDA(cudaMemcpy(P.rc, c.data(), sizeof(double) * P.nalm,
-                     cudaMemcpyHostToDevice));
-  WF_CUDA(cudaMemcpy(P.rg, g.data(), sizeof(double) * P.nalm,
-                     cudaMemcpyHostToDevice));
-  return WF_OK;
-}
-
 // lam_mm for every m of one ring pair, as mantissa * 2^exponent.
 __global__ void k_seed_diag(const RingPair *pairs, int npairs, int lmax,
                             double *mant, int *expo) {
@@ -292,11 +240,10 @@ __global__ void k_seed_diag(const RingPair *pairs, int npairs, int lmax,
   }
 }
 
-// For each (m, pair): walk the recurrence in scaled FP64 until |lam| >= 2^-100
-// and store the start l and the two rescaled values there.
-__global__ void k_seed_walk(const RingPair *pairs, int npairs, int lmax,
-                            const double *mant, const int *expo,
-                            const double *rg, int *seed_l, double2 *seed_u) {
+// For each (m, pair): the first l with |lam_lm| >= 2^-100 (lmax + 1: none), by the
+// one-step recurrence in scaled FP64.  Only wf_legendre_terms needs it.
+__global__ void k_first_l(const RingPair *pairs, int npairs, int lmax, const double *mant,
+                          const int *expo, int *first) {
   long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long)npairs * (lmax + 1)) return;
   const int m = (int)(t / npairs);
@@ -307,18 +254,10 @@ __global__ void k_seed_walk(const RingPair *pairs, int npairs, int lmax,
   double a_prev = 0.0;
   int l = m;
   int found = lmax + 1;
-  double lam0 = 0.0, lam1 = 0.0;
   for (;;) {
     // actual value v * 2^e; compare exponents against -100
     if (v != 0.0 && ilogb(v) + e >= -100) {
       found = l;
-      lam0 = ldexp(v, e);
-      if (l + 1 <= lmax) {
-        double a = sqrt((4.0 * (l + 1) * (l + 1) - 1.0) /
-                        ((double)(l + 1) * (l + 1) - (double)m * m));
-        double vn = (l == m) ? a * z * v : a * z * v - (a / a_prev) * vp;
-        lam1 = ldexp(vn, e);
-      }
       break;
     }
     if (l == lmax) break;
@@ -335,13 +274,34 @@ __global__ void k_seed_walk(const RingPair *pairs, int npairs, int lmax,
       e += 200;
     }
   }
-  seed_l[t] = found;
-  double2 u = make_double2(0.0, 0.0);
-  if (found <= lmax) {
-    u.x = lam0 / rg[alm_idx_d(lmax, found, m)];
-    if (found + 1 <= lmax) u.y = lam1 / rg[alm_idx_d(lmax, found + 1, m)];
+  first[t] = found;
+}
+
+// lam_mm of every (m, pair) as mantissa and exponent, for f(mant, expo); waits for the
+// stream and frees them
+template <typename Fn>
+static wf_status with_diag(Plan &P, Fn f) {
+  const long n = (long)P.npairs * (P.lmax + 1);
+  double *mant = nullptr;
+  int *expo = nullptr;
+  WF_CUDA(cudaMalloc(&mant, sizeof(double) * n));
+  wf_status st = WF_OK;
+  cudaError_t e = cudaMalloc(&expo, sizeof(int) * n);
+  if (e == cudaSuccess) {
+    k_seed_diag<<<(P.npairs + 127) / 128, 128, 0, P.stream>>>(P.pairs, P.npairs, P.lmax, mant,
+                                                              expo);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) st = f(mant, expo);
+    const cudaError_t w = cudaStreamSynchronize(P.stream);
+    if (e == cudaSuccess) e = w;
   }
-  seed_u[t] = u;
+  cudaFree(mant);
+  cudaFree(expo);
+  if (st == WF_OK && e != cudaSuccess) {
+    set_error(std::string("Legendre tables: ") + cudaGetErrorString(e));
+    return WF_ERR_CUDA;
+  }
+  return st;
 }
 
 static wf_status make_seeds(Plan &P) {
@@ -350,32 +310,35 @@ static wf_status make_seeds(Plan &P) {
   P.device = dev;
   WF_CUDA(cudaDeviceGetAttribute(&P.num_sms, cudaDevAttrMultiProcessorCount, dev));
   // FP32 synthesis: one pair per thread on small maps (Nside 90: 6.4 us, 7.5 with two),
-  // two in the middle (Nside 256: 17.7 us, 19.3 with one, 20.3 with four; Nside 512:
-  // 69, 85, 72), four on large ones (Nside 1024: 435 us, 529 with two); FP64 is bound
+  // two in the middle (Nside 256: 17.0 us, 18.8 with one, 18.7 with four; Nside 512:
+  // 69, 85, 71), four on large ones (Nside 1024: 436 us, 531 with two); FP64 is bound
   // by its unit and takes one
   P.syn_np[1] = P.npairs >= 1536 ? 4 : P.npairs >= 384 ? 2 : 1;
+  return with_diag(P, [&](const double *mant, const int *expo) {
+    return build_pair_tables(P, mant, expo);
+  });
+}
+
+wf_status first_l_table(Plan &P, std::vector<int> &out) {
   const long n = (long)P.npairs * (P.lmax + 1);
-  double *mant = nullptr;
-  int *expo = nullptr;
-  WF_CUDA(cudaMalloc(&mant, sizeof(double) * n));
-  WF_CUDA(cudaMalloc(&expo, sizeof(int) * n));
-  WF_CUDA(cudaMalloc(&P.seed_l, sizeof(int) * n));
-  WF_CUDA(cudaMalloc(&P.seed_u, sizeof(double2) * n));
-  k_seed_diag<<<(P.npairs + 127) / 128, 128, 0, P.stream>>>(P.pairs, P.npairs,
-                                                            P.lmax, mant, expo);
-  WF_CUDA(cudaGetLastError());
-  k_seed_walk<<<(unsigned)((n + 255) / 256), 256, 0, P.stream>>>(
-      P.pairs, P.npairs, P.lmax, mant, expo, P.rg, P.seed_l, P.seed_u);
-  WF_CUDA(cudaGetLastError());
-  WF_TRY(build_pair_tables(P, mant, expo));
-  WF_CUDA(cudaStreamSynchronize(P.stream));
-  WF_CUDA(cudaFree(mant));
-  WF_CUDA(cudaFree(expo));
-  return WF_OK;
+  return with_diag(P, [&](const double *mant, const int *expo) {
+    int *first = nullptr;
+    WF_CUDA(cudaMalloc(&first, sizeof(int) * n));
+    k_first_l<<<(unsigned)((n + 255) / 256), 256, 0, P.stream>>>(P.pairs, P.npairs, P.lmax,
+                                                                 mant, expo, first);
+    std::vector<int> h(n);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(h.data(), first, sizeof(int) * n, cudaMemcpyDeviceToHost, P.stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(P.stream);
+    cudaFree(first);
+    WF_CUDA(e);
+    out.swap(h);
+    return WF_OK;
+  });
 }
 
 wf_status build_tables(Plan &P) {
-  WF_TRY(init_legendre_attributes());
   WF_TRY(init_pair_attributes());
   WF_TRY(init_ring_attributes());
   make_pairs(P);
@@ -392,7 +355,6 @@ wf_status build_tables(Plan &P) {
     WF_CUDA(cudaMemcpy(P.cl32, cl32.data(), sizeof(float) * (P.lmax + 1),
                        cudaMemcpyHostToDevice));
   }
-  WF_TRY(make_recurrence_tables(P));
   WF_TRY(make_seeds(P));
   return WF_OK;
 }

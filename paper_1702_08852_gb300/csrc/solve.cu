@@ -757,9 +757,7 @@ static wf_status fp64_step(Plan &P, const double2 *x, double2 *gx, double *num) 
 // reduced term count of one Legendre transform at band L (cached per L)
 wf_status legendre_terms(Plan &P, int L, double *terms) {
   if (P.seed_l_h.empty()) {
-    P.seed_l_h.resize((size_t)P.npairs * (P.lmax + 1));
-    WF_CUDA(cudaMemcpy(P.seed_l_h.data(), P.seed_l, sizeof(int) * P.seed_l_h.size(),
-                       cudaMemcpyDeviceToHost));
+    WF_TRY(first_l_table(P, P.seed_l_h));
     P.work_cache.assign(P.lmax + 1, -1.0);
   }
   if (P.work_cache[L] < 0.0) {

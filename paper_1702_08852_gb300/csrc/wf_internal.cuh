@@ -38,6 +38,16 @@ void set_error_static(const char *msg);
 template <typename V> struct PairVec;
 template <> struct PairVec<double> { typedef double2 type; };
 template <> struct PairVec<float> { typedef float2 type; };
+struct dd {  // double-float: the unevaluated sum hi + lo (legpair.cu)
+  float hi, lo;
+  dd() = default;
+  __host__ __device__ dd(float h, float l) : hi(h), lo(l) {}
+  __host__ __device__ explicit dd(int v) : hi((float)v), lo(0.f) {}
+};
+template <> struct PairVec<dd> { struct type { dd x, y; }; };
+// the checkpoints' type: the double-float kernels read the FP64 ones
+template <typename V> struct CkVec { typedef typename PairVec<V>::type type; };
+template <> struct CkVec<dd> { typedef double2 type; };
 template <typename V>
 struct PairTab {
   typename PairVec<V>::type *rec[3] = {};  // (A, B) of the three forms
@@ -46,8 +56,8 @@ struct PairTab {
   V *w = nullptr;                  // [3][stride]: z^2 - 1, z^2 - 1/2, z^2
   V *z = nullptr;                  // [stride]
   int *js = nullptr;               // [lmax+1][stride] first j with |Q_j| >= 2^-100
-  typename PairVec<V>::type *ck = nullptr;  // [block of 16 j of m][stride]
-  typename PairVec<V>::type *seed = nullptr;  // [lmax+1][stride] (s_js, s_js+1)
+  typename CkVec<V>::type *ck = nullptr;  // [block of 16 j of m][stride]
+  typename CkVec<V>::type *seed = nullptr;  // [lmax+1][stride] (s_js, s_js+1)
   int *jin = nullptr;              // [lmax+1][stride] FP32: j where ck holds the seeds
   int *gfirst = nullptr;           // [block]: first warp of pairs with a term in it
   int kform[2] = {0, 0};           // pairs below kform[f]: form f (multiples of 32)
@@ -58,6 +68,13 @@ struct PairTab {
   typename PairVec<V>::type *rec_e = nullptr;
   V *ge = nullptr, *go = nullptr, *lmm = nullptr;
 };
+
+// j of one m: J = (L - m) / 2 + 1; the first (m, j) table entry of m is the sum of J
+// over the smaller m
+__host__ __device__ __forceinline__ long tri_j(long n) { return n + 1 + (n * n) / 4; }
+__host__ __device__ __forceinline__ long pair_base(int lmax, int m) {
+  return tri_j(lmax) - tri_j(lmax - m);
+}
 
 // One iso-latitude ring pair: the north ring and its mirror image in the
 // south (the equator ring is a "pair" with no south ring).  Both rings share
@@ -170,11 +187,7 @@ struct Plan {
   double *cl_d = nullptr;        // [lmax+1]
   PairTab<double> pt64;          // parity-pair basis, FP64
   PairTab<float> pt32;           // and FP32
-  double *rc = nullptr;          // [nalm] recurrence coefficient c_lm
-  double *rg = nullptr;          // [nalm] scale g_lm (lambda = g u)
-  float2 *rcdd = nullptr;        // [nalm] rc as double-float pairs (hi, lo)
-  int *seed_l = nullptr;         // [lmax+1][npairs] first l with |lambda| >= 2^-100
-  double2 *seed_u = nullptr;     // [lmax+1][npairs] (u_ls, u_ls+1)
+  PairTab<dd> ptdd;              // and double-float
   float *cl32 = nullptr;         // [lmax+1] C_l in FP32 (the FP32 analysis' filter)
 
   // ring pairs per thread of the synthesis, [0] = FP64, [1] = FP32 (make_seeds, or the
@@ -183,10 +196,6 @@ struct Plan {
   int syn_np[2] = {1, 1};
   int ana_np[2] = {4, 8};
   int ana_queue = 0, syn_x2 = 0, ana_x2 = 0, ana_gacc = 0;
-  // double-float analysis: per-tile sums, first l of each item, the queue's next item
-  float *ana_scratch = nullptr;  // [tiles of 128 pairs][nalm] double2
-  int *ana_lstart = nullptr;     // [lmax+1][tiles] first l written per item
-  int *ana_counter = nullptr;    // the queue's next item (reset by the combine)
   int num_sms = 0;
   float tune_syn_ms[2][6] = {{-1, -1, -1, -1, -1, -1}, {-1, -1, -1, -1, -1, -1}};
   float tune_ana_ms[2][15] = {{-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1},
@@ -220,7 +229,7 @@ struct Plan {
   double2 *x = nullptr;          // [nalm] current iterate
   double2 *xtmp = nullptr;       // [nalm]
   double2 *xacc = nullptr;       // [nalm] refined solution (mixed precision)
-  double2 *xs64 = nullptr;       // [nalm] g_lm x_lm as double-float pairs, synthesis input
+  double2 *xs64 = nullptr;       // [nalm] x_lm as double-float pairs, synthesis input
   float2 *xs32 = nullptr;        // [nalm] x_lm, synthesis input (FP32)
   double2 *src = nullptr;        // [nalm] harmonic source of a correction solve
   // mixed solver, stage boundaries between anchored stages: the unfiltered
@@ -273,11 +282,11 @@ struct Plan {
   struct GroupState *group = nullptr;
   double group_ms = 0.0, group_flop = 0.0, group_bytes = 0.0;
   long group_launches = 0;
-  std::vector<int> seed_l_h;         // host copy of seed_l
+  std::vector<int> seed_l_h;         // first l with |lambda_lm| >= 2^-100, [m][pair]
 };
 
 // ---------------------------------------------------------------- kernels
-// Legendre transforms (legendre.cu).  Modes of the analysis:
+// Legendre transforms (legpair.cu).  Modes of the analysis:
 enum AnalysisMode { ANA_PLAIN = 0, ANA_FILTER = 1 };
 
 // The synthesis reads the coefficients in its own precision: the FP32 ones are written
@@ -300,7 +309,7 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo);
 void free_pair_tables(Plan &P);
 
 // Double-float (pairs of FP32) Legendre transforms with FP64 inputs and
-// outputs, for the anchor steps of the mixed solver (legendre.cu): the same
+// outputs, for the anchor steps of the mixed solver (legpair.cu): the same
 // contracts as launch_legendre_synth<double2> / launch_legendre_anal<double2>.
 // Their ring coefficients F, G and the synthesis input are double-float
 // pairs (re hi, re lo, im hi, im lo), 16 bytes like an FP64 complex (the
@@ -341,7 +350,6 @@ wf_status launch_ring_batch32(const Plan &P, int mode, const float2 *F, float2 *
 wf_status launch_to_dd(const Plan &P, const double *in, float2 *out, long n);
 
 // once per plan (kernel attributes; allowed outside stream capture only)
-wf_status init_legendre_attributes();
 wf_status init_ring_attributes();
 
 // autotune.cu: time the Legendre launch variants once per geometry
@@ -353,6 +361,7 @@ wf_status solve_batch(Plan **plans, int n, const double *const *d, double *const
 
 // plan.cu
 wf_status build_tables(Plan &P);
+wf_status first_l_table(Plan &P, std::vector<int> &out);
 wf_status upload_noise(Plan &P, const double *nvar_dev, const uint8_t *mask_dev);
 
 // solve.cu
