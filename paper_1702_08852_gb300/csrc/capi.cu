@@ -31,7 +31,7 @@ static void free_plan(wf_plan_s *P) {
   free_pair_tables(*P);
   for (int i = 0; i < 3; ++i)
     if (P->graph[i]) cudaGraphExecDestroy(P->graph[i]);
-  void *bufs[] = {P->pairs, P->cl_d,   P->tw64,  P->tw32,    P->chirp64, P->chirp32, P->bhat64,
+  void *bufs[] = {P->pairs, P->cl_d,   P->tp64, P->tp32, P->tpdd, P->tw64,  P->tw32,    P->chirp64, P->chirp32, P->bhat64,
                   P->bhat32, P->nvar,  P->F64,     P->G64,    P->F32,    P->G32,
                   P->x,      P->xtmp,  P->dmap,    P->mtmp,   P->partials, P->red,
                   P->state,  P->trace, P->xacc,  P->src, P->xs64, P->xs32,

@@ -5,6 +5,10 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
+
+#include <algorithm>
+#include <vector>
 
 namespace wf {
 
@@ -40,6 +44,9 @@ template <> struct CT<float2> {
     sincospif((float)r / (float)den, s, c);
   }
 };
+
+// one entry of the twiddle table (TwPass)
+template <typename T2> struct alignas(16) TwPair { typename CT<T2>::W a, b; };
 
 template <typename T2>
 __device__ __forceinline__ T2 cmul(T2 a, T2 b) {
@@ -80,31 +87,19 @@ __device__ __forceinline__ int sw(int i) {
   return i ^ ((b ^ (b << 2)) & 15);
 }
 
-// Twiddles of one pass: pair(j) gives W_2h^j = e^{-i pi j / h} and
-// W_h^j = (W_2h^j)^2 (h a power of two, 0 <= j < h).  FP32 computes them:
-// sincospi of the exact argument j / h (1/h is exact) and one complex square
-// -- no memory access on the FFT's critical path.  FP64 reads the plan's
-// table tw[i] = e^{-2 pi i i / Mmax} (FP64 sincospi would cost more than the
-// butterfly on this part's FP64 pipe).
-template <typename T2> struct TwPass;
-template <> struct TwPass<float2> {
-  float inv;
-  __device__ __forceinline__ TwPass(int h, const float2 *, int) : inv(1.0f / (float)h) {}
-  __device__ __forceinline__ void pair(int j, float2 &w2h, float2 &wh) const {
-    float s, c;
-    sincospif((float)j * inv, &s, &c);
-    w2h = make_float2(c, -s);
-    wh = make_float2(c * c - s * s, -2.0f * c * s);
-  }
-};
-template <> struct TwPass<double2> {
-  const double2 *tw;
-  int ts;
-  __device__ __forceinline__ TwPass(int h, const double2 *t, int Mmax)
-      : tw(t), ts(Mmax / (2 * h)) {}
-  __device__ __forceinline__ void pair(int j, double2 &w2h, double2 &wh) const {
-    w2h = tw[j * ts];
-    wh = tw[2 * j * ts];
+// Twiddles of one pass of span h: pair(j), j < h / 2, gives W_2h^j = e^{-i pi j / h}
+// and W_h^j = (W_2h^j)^2, side by side in a table that holds every span's entries at
+// h / 2 - 1 (twiddle_table: Mmax / 2 - 1 entries for lengths up to Mmax).  The table
+// (16 KB in FP32 for 2048 points) stays in L1; computing the pair in FP32 by sincospi
+// took 40 of a butterfly's ~100 instructions.
+template <typename T2>
+struct TwPass {
+  const TwPair<T2> *t;
+  __device__ __forceinline__ TwPass(int h, const TwPair<T2> *tw) : t(tw + (h / 2 - 1)) {}
+  __device__ __forceinline__ void pair(int j, T2 &w2h, T2 &wh) const {
+    const TwPair<T2> v = t[j];
+    w2h = CT<T2>::ldw(&v.a);
+    wh = CT<T2>::ldw(&v.b);
   }
 };
 
@@ -192,29 +187,18 @@ template <> struct CT<ddc> {
     *c = ddr(cd);
   }
 };
-template <> struct TwPass<ddc> {
-  const float4 *tw;
-  int ts;
-  __device__ __forceinline__ TwPass(int h, const float4 *t, int Mmax)
-      : tw(t), ts(Mmax / (2 * h)) {}
-  __device__ __forceinline__ void pair(int j, ddc &w2h, ddc &wh) const {
-    w2h = CT<ddc>::ldw(tw + j * ts);
-    wh = CT<ddc>::ldw(tw + 2 * j * ts);
-  }
-};
-
 // natural -> bit-reversed; INV uses e^{+2 pi i jk/M}.  Two radix-2 stages
 // (spans h and h/2) per pass over shared memory ("radix-2^2"): the output
 // order stays bit-reversed, and the barriers and shared-memory round trips
 // halve.  An odd number of stages ends with one radix-2 pass of span 1.
 // Where the twiddle index j = b mod q is the same for all of a thread's
-// butterflies (q <= blockDim), the twiddles are computed once per pass.
+// butterflies (q <= blockDim), the twiddles are loaded once per pass.
 template <typename T2, bool INV>
-__device__ void fft_dif(T2 *buf, int M, const typename CT<T2>::W *__restrict__ tw, int Mmax) {
+__device__ void fft_dif(T2 *buf, int M, const TwPair<T2> *__restrict__ tw) {
   int h = M >> 1;
   for (; h >= 2; h >>= 2) {
     const int q = h >> 1;
-    const TwPass<T2> tp(h, tw, Mmax);
+    const TwPass<T2> tp(h, tw);
     const bool fixed = q <= (int)blockDim.x;
     T2 w1f, w2f;
     if (fixed) tp.pair((int)threadIdx.x & (q - 1), w1f, w2f);
@@ -248,7 +232,7 @@ __device__ void fft_dif(T2 *buf, int M, const typename CT<T2>::W *__restrict__ t
 // bit-reversed -> natural; an odd number of stages starts with one radix-2
 // pass of span 1, then pairs of stages (spans h and 2h) per pass
 template <typename T2, bool INV>
-__device__ void fft_dit(T2 *buf, int M, const typename CT<T2>::W *__restrict__ tw, int Mmax) {
+__device__ void fft_dit(T2 *buf, int M, const TwPair<T2> *__restrict__ tw) {
   int h = 1;
   int bits = 0;
   while ((1 << bits) < M) ++bits;
@@ -262,7 +246,7 @@ __device__ void fft_dit(T2 *buf, int M, const typename CT<T2>::W *__restrict__ t
     h = 2;
   }
   for (; h < M; h <<= 2) {
-    const TwPass<T2> tp(2 * h, tw, Mmax);  // pair(j) = (W_4h^j, W_2h^j)
+    const TwPass<T2> tp(2 * h, tw);  // pair(j) = (W_4h^j, W_2h^j)
     const bool fixed = h <= (int)blockDim.x;
     T2 waf, wbf;
     if (fixed) tp.pair((int)threadIdx.x & (h - 1), wbf, waf);
@@ -290,6 +274,17 @@ __device__ void fft_dit(T2 *buf, int M, const typename CT<T2>::W *__restrict__ t
 
 __device__ __forceinline__ int bitrev_n(int x, int bits) {
   return (int)(__brev((unsigned)x) >> (32 - bits));
+}
+
+// the host table of TwPass in FP64: a = e^{-i pi j / h}, b = e^{-2 i pi j / h}
+inline std::vector<TwPair<double2>> twiddle_table(int Mmax) {
+  std::vector<TwPair<double2>> t(std::max(1, Mmax / 2 - 1));
+  for (int h = 2; h <= Mmax / 2; h <<= 1)
+    for (int j = 0; j < h / 2; ++j) {
+      const double x = M_PI * (double)j / (double)h;
+      t[h / 2 - 1 + j] = {make_double2(cos(x), -sin(x)), make_double2(cos(2.0 * x), -sin(2.0 * x))};
+    }
+  return t;
 }
 
 }  // namespace wf

@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(FLAT_THREADS)
 __global__ void __launch_bounds__(FLAT_THREADS)
     k_flat_hcols(int n, int cb, double omega, const double *__restrict__ ck,
                  const double2 *__restrict__ T1, double2 *__restrict__ S,
-                 double2 *__restrict__ T2, const double2 *__restrict__ tw,
+                 double2 *__restrict__ T2, const TwPair<double2> *__restrict__ tw,
                  const SolverState *__restrict__ st, double *__restrict__ partials, int mode) {
   extern __shared__ __align__(16) unsigned char flat_smem[];
   double2 *buf = reinterpret_cast<double2 *>(flat_smem);  // [cb][n]
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(FLAT_THREADS)
       buf[c * n + sw(y)] = T1[((long)(y >> 1) * nk + kx0 + c) * 2 + (y & 1)];
     }
     __syncthreads();
-    for (int c = 0; c < nc; ++c) fft_dif<double2, false>(buf + c * n, n, tw, n);
+    for (int c = 0; c < nc; ++c) fft_dif<double2, false>(buf + c * n, n, tw);
     double num = 0.0, den = 0.0;
     const double mo = st->mu * omega, xo = st->xi * omega;
     for (int e = tid; e < nc * n; e += nt) {
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(FLAT_THREADS)
     }
     __syncthreads();
   }
-  for (int c = 0; c < nc; ++c) fft_dit<double2, true>(buf + c * n, n, tw, n);
+  for (int c = 0; c < nc; ++c) fft_dit<double2, true>(buf + c * n, n, tw);
   for (int e = tid; e < nc * n; e += nt) {
     const int c = (e >> 1) % nc, y = (e >> 1) / nc * 2 + (e & 1);
     T2[((long)(y >> 1) * nk + kx0 + c) * 2 + (y & 1)] = buf[c * n + sw(y)];
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(FLAT_THREADS)
     k_flat_hrows(int n, int logn, const double2 *__restrict__ T2, double2 *__restrict__ T1,
                  const double *__restrict__ in, const double *__restrict__ d,
                  const double *__restrict__ nvar, double *__restrict__ out,
-                 const double2 *__restrict__ tw, const SolverState *__restrict__ st, int mode) {
+                 const TwPair<double2> *__restrict__ tw, const SolverState *__restrict__ st, int mode) {
   extern __shared__ __align__(16) unsigned char flat_smem[];
   double2 *buf = reinterpret_cast<double2 *>(flat_smem);  // [n]
   if (mode == FLAT_ITER && st->done) return;
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(FLAT_THREADS)
         buf[sw(bitrev_n(n - k, logn))] = make_double2(a.x + b.y, b.x - a.y);
     }
     __syncthreads();
-    fft_dit<double2, true>(buf, n, tw, n);
+    fft_dit<double2, true>(buf, n, tw);
     const double scale = 1.0 / ((double)n * (double)n);
     if (mode == FLAT_FINAL) {
       for (int x = tid; x < n; x += nt) {
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(FLAT_THREADS)
     }
     __syncthreads();
   }
-  fft_dif<double2, false>(buf, n, tw, n);
+  fft_dif<double2, false>(buf, n, tw);
   for (int k = tid; k < nk; k += nt) {
     const double2 z = buf[sw(bitrev_n(k, logn))], m = buf[sw(bitrev_n((n - k) & (n - 1), logn))];
     T1[trow + 2 * k] = make_double2(0.5 * (z.x + m.x), 0.5 * (z.y - m.y));
@@ -309,6 +309,7 @@ struct FlatPlan {
   cudaStream_t stream = nullptr, capture_stream = nullptr;
   double *ck = nullptr, *nvar = nullptr, *d = nullptr, *partials = nullptr;
   double2 *T1 = nullptr, *T2 = nullptr, *S = nullptr, *tw = nullptr;
+  TwPair<double2> *tp = nullptr;  // the h kernels' twiddles
   SolverState *state = nullptr, *state_h = nullptr;
   TraceEntry *trace = nullptr;
   int trace_cap = 0, trace_len = 0;
@@ -322,7 +323,7 @@ struct FlatPlan {
 static void flat_free(FlatPlan *F) {
   if (!F) return;
   if (F->graph) cudaGraphExecDestroy(F->graph);
-  void *b[] = {F->ck, F->nvar, F->d, F->partials, F->T1, F->T2, F->S, F->tw, F->state,
+  void *b[] = {F->ck, F->nvar, F->d, F->partials, F->T1, F->T2, F->S, F->tw, F->tp, F->state,
                F->trace};
   for (void *x : b)
     if (x) cudaFree(x);
@@ -369,7 +370,7 @@ static void flat_cols(FlatPlan &F, cudaStream_t s, const SolverState *st) {
   ++F.nlaunch;
   if (F.herm)
     k_flat_hcols<<<flat_ncols(F), std::max(32, std::min(FLAT_THREADS, F.n / 4)), F.smem_cols, s>>>(
-        F.n, flat_cb(F), F.omega, F.ck, F.T1, F.S, F.T2, F.tw, st, F.partials, mode);
+        F.n, flat_cb(F), F.omega, F.ck, F.T1, F.S, F.T2, F.tp, st, F.partials, mode);
   else
     k_flat_cols<<<flat_ncols(F), FLAT_THREADS, F.smem_cols, s>>>(
         F.n, F.logn, F.omega, F.ck, F.T1, F.S, F.T2, F.tw, st, F.partials, mode);
@@ -381,7 +382,7 @@ static void flat_rows(FlatPlan &F, cudaStream_t s, const double *in, double *out
   ++F.nlaunch;
   if (F.herm)
     k_flat_hrows<<<F.n / 2, std::max(32, std::min(FLAT_THREADS, F.n / 4)), F.smem_rows, s>>>(
-        F.n, F.logn, F.T2, F.T1, in, F.d, F.nvar, out, F.tw, st, mode);
+        F.n, F.logn, F.T2, F.T1, in, F.d, F.nvar, out, F.tp, st, mode);
   else
     k_flat_rows<<<F.n, FLAT_THREADS, F.smem_rows, s>>>(F.n, F.logn, F.T2, F.T1, in, F.d, F.nvar,
                                                        out, F.tw, st, mode);
@@ -545,7 +546,9 @@ wf_status wf_flat_plan(wf_flat_t *out, int n, double pixel_area, const double *c
     if ((e = cudaMalloc(b, sizeof(double) * n2)) != cudaSuccess) return fail("cudaMalloc", e);
   for (double2 **b : {&F->T1, &F->T2, &F->S})
     if ((e = cudaMalloc(b, sizeof(double2) * n2)) != cudaSuccess) return fail("cudaMalloc", e);
+  const std::vector<TwPair<double2>> tp = twiddle_table(n);
   if ((e = cudaMalloc(&F->tw, sizeof(double2) * (n / 2))) != cudaSuccess ||
+      (e = cudaMalloc(&F->tp, sizeof(tp[0]) * tp.size())) != cudaSuccess ||
       (e = cudaMalloc(&F->partials, sizeof(double) * 3 * (n / 2 + 1))) != cudaSuccess ||
       (e = cudaMalloc(&F->state, sizeof(SolverState))) != cudaSuccess ||
       (e = cudaMallocHost(&F->state_h, sizeof(SolverState))) != cudaSuccess ||
@@ -591,6 +594,8 @@ wf_status wf_flat_plan(wf_flat_t *out, int n, double pixel_area, const double *c
   if ((e = cudaMemcpy(F->nvar, nv.data(), sizeof(double) * n2, cudaMemcpyHostToDevice)) !=
           cudaSuccess ||
       (e = cudaMemcpy(F->ck, ck.data(), sizeof(double) * n2, cudaMemcpyHostToDevice)) !=
+          cudaSuccess ||
+      (e = cudaMemcpy(F->tp, tp.data(), sizeof(tp[0]) * tp.size(), cudaMemcpyHostToDevice)) !=
           cudaSuccess ||
       (e = cudaMemcpy(F->tw, tw.data(), sizeof(double2) * tw.size(), cudaMemcpyHostToDevice)) !=
           cudaSuccess)

@@ -17,6 +17,7 @@
 #include <complex>
 #include <vector>
 
+#include "fft.cuh"
 #include "wf_internal.cuh"
 
 namespace wf {
@@ -153,6 +154,25 @@ static wf_status make_fft_tables(Plan &P) {
   WF_CUDA(cudaMemcpy(P.tw32, tw32.data(), sizeof(float2) * tw.size(),
                      cudaMemcpyHostToDevice));
   WF_TRY(upload_dd(tw, &P.twdd));
+  {
+    const std::vector<TwPair<double2>> t = twiddle_table(Mmax);
+    std::vector<TwPair<float2>> t32(t.size());
+    std::vector<double2> flat(2 * t.size());
+    for (size_t i = 0; i < t.size(); ++i) {
+      t32[i] = {make_float2((float)t[i].a.x, (float)t[i].a.y),
+                make_float2((float)t[i].b.x, (float)t[i].b.y)};
+      flat[2 * i] = t[i].a;
+      flat[2 * i + 1] = t[i].b;
+    }
+    WF_CUDA(cudaMalloc(&P.tp64, sizeof(t[0]) * t.size()));
+    WF_CUDA(cudaMemcpy(P.tp64, t.data(), sizeof(t[0]) * t.size(), cudaMemcpyHostToDevice));
+    WF_CUDA(cudaMalloc(&P.tp32, sizeof(t32[0]) * t32.size()));
+    WF_CUDA(cudaMemcpy(P.tp32, t32.data(), sizeof(t32[0]) * t32.size(), cudaMemcpyHostToDevice));
+    float4 *dd = nullptr;
+    const wf_status st = upload_dd(flat, &dd);
+    P.tpdd = dd;
+    WF_TRY(st);
+  }
   P.chirp_total = chirp_total;
   P.bhat_total = bhat_total;
   if (chirp_total > 0) {

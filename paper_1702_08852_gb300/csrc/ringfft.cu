@@ -35,15 +35,14 @@ namespace wf {
 // In place: buf[0..n) holds a_j = x_j conj(w_j) and buf[n..M) zeros on entry;
 // on exit buf[0..n) holds X = DFT_n(x).
 template <typename T2>
-__device__ void bluestein(T2 *buf, int n, int M, const typename CT<T2>::W *__restrict__ tw,
-                          int Mmax, const typename CT<T2>::W *__restrict__ chirp,
-                          const typename CT<T2>::W *__restrict__ bhat) {
-  fft_dif<T2, false>(buf, M, tw, Mmax);
+__device__ void bluestein(T2 *buf, int n, int M, const TwPair<T2> *__restrict__ twp,
+                          const typename CT<T2>::W *chirp, const typename CT<T2>::W *bhat) {
+  fft_dif<T2, false>(buf, M, twp);
   #pragma unroll 8
   for (int q = threadIdx.x; q < M; q += blockDim.x)
     buf[sw(q)] = cmul(buf[sw(q)], CT<T2>::ldw(bhat + q));
   __syncthreads();
-  fft_dit<T2, true>(buf, M, tw, Mmax);
+  fft_dit<T2, true>(buf, M, twp);
   #pragma unroll 8
   for (int k = threadIdx.x; k < n; k += blockDim.x)
     buf[sw(k)] = cmulc(buf[sw(k)], CT<T2>::ldw(chirp + k));
@@ -118,19 +117,21 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
            const typename CT<T2>::G *__restrict__ F, typename CT<T2>::G *__restrict__ G,
            const double *__restrict__ in_map, double *__restrict__ out_map,
            const double *__restrict__ nvar, const typename CT<T2>::W *__restrict__ tw,
-           int Mmax, const typename CT<T2>::W *__restrict__ chirp_all,
+           int Mmax, const TwPair<T2> *__restrict__ twp,
+           const typename CT<T2>::W *__restrict__ chirp_all,
            const typename CT<T2>::W *__restrict__ bhat_all,
-           const SolverState *__restrict__ st, int lstatic, int reverse,
+           const SolverState *__restrict__ st, int lstatic, int rev,
            const float *__restrict__ in32, const float *__restrict__ nv32, int red_ofs,
+           int tab_ofs,
            const typename CT<T2>::W *__restrict__ phase_all,
            const float2 *__restrict__ in_dd, const float2 *__restrict__ nv_dd,
            long bstride_f, long bstride_m) {
   typedef typename CT<T2>::T T;
   typedef typename CT<T2>::G GT;
   typedef typename CT<T2>::W WT;
-  // reverse: the polar rings grow with the pair index; taking the largest
-  // first keeps the small ones for the tail of the launch
-  const int blk = reverse ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
+  // the first `rev` pairs are the polar ones, which grow with the index: the largest
+  // first keeps the small ones for the end
+  const int blk = (int)blockIdx.x < rev ? rev - 1 - (int)blockIdx.x : (int)blockIdx.x;
   // batched launches (plain transforms of several maps): map blockIdx.y
   if (gridDim.y > 1) {
     const long bm = blockIdx.y;
@@ -178,6 +179,24 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
   while ((1 << bits) < M) ++bits;
   const WT *chirp = blue ? chirp_all + rp.chirp_ofs : nullptr;
   const WT *bhat = blue ? bhat_all + rp.bhat_ofs : nullptr;
+  if (tab_ofs && blue) {
+    // copied while the coefficients are folded: read M + 2 n (fused: 2 M + 4 n) times
+    // off the critical path instead of from L2 in the middle of each transform
+    WT *sb = reinterpret_cast<WT *>(smraw + tab_ofs), *sc = sb + M;
+    auto copy = [](WT *dst, const WT *src, int count) {
+      const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+      constexpr int E = sizeof(WT) >= 16 ? 1 : 2;  // elements per 16 bytes
+      for (int i = threadIdx.x * E; i < count; i += blockDim.x * E)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + i * (int)sizeof(WT)),
+                     "l"(src + i)
+                     : "memory");
+    };
+    copy(sb, bhat, M);
+    copy(sc, chirp, n);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    bhat = sb;
+    chirp = sc;
+  }
   const WT *phs = (blue && phase_all) ? phase_all + rp.chirp_ofs : nullptr;
   const bool south = rp.ringS >= 0;
   // F and G: [m][pair][north, south] with `npairs` pairs, or (0: the grouped
@@ -188,6 +207,11 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
   const T2 zero = CT<T2>::mk((T)0, (T)0);
   const T sgn = rp.phi_num ? (T)-1 : (T)1;  // e^{i n phi0}
   const int tstep = (rp.phi_num && Mmax % (2 * rp.phi_den) == 0) ? Mmax / (2 * rp.phi_den) : 0;
+
+  auto tables_here = []() {  // this thread's copies, then everyone's
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+  };
 
   if (MODE != RING_ANALYSIS) {
     const GT *FN = F + rowN;
@@ -223,7 +247,10 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
         red[threadIdx.x] = pN;
         red[blockDim.x + threadIdx.x] = pS;
       }
-      __syncthreads();
+      if (tab_ofs && blue)
+        tables_here();
+      else
+        __syncthreads();
       if ((int)threadIdx.x < n) {
         T2 cN = zero, cS = zero;
         for (int q = 0; q < P; ++q) {
@@ -237,6 +264,7 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
         buf[sw(k)] = blue ? cmulc(cconj(Zk), CT<T2>::ldw(chirp + k)) : Zk;
       }
     } else {
+      if (tab_ofs && blue) tables_here();
       #pragma unroll 4
       for (int k = threadIdx.x; k < n; k += blockDim.x) {
         T2 cN = zero, cS = zero;
@@ -253,9 +281,9 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
       for (int k = n + threadIdx.x; k < M; k += blockDim.x) buf[sw(k)] = zero;
     __syncthreads();
     if (blue) {
-      bluestein<T2>(buf, n, M, tw, Mmax, chirp, bhat);  // DFT(conj Z)
+      bluestein<T2>(buf, n, M, twp, chirp, bhat);  // DFT(conj Z)
     } else {
-      fft_dif<T2, true>(buf, M, tw, Mmax);  // bit-reversed output
+      fft_dif<T2, true>(buf, M, twp);  // bit-reversed output
     }
     // pixel step; position q holds pixel j
     #pragma unroll 4
@@ -317,6 +345,7 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
       for (int k = n + threadIdx.x; k < M; k += blockDim.x) buf[sw(k)] = zero;
     __syncthreads();
   } else {
+    if (tab_ofs && blue) tables_here();
     #pragma unroll 4
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
       const double tN = in_map[rp.ofsN + j];
@@ -333,9 +362,9 @@ __global__ void __launch_bounds__(RING_THREADS_BIG)
   }
   // forward DFT of t (natural order output)
   if (blue)
-    bluestein<T2>(buf, n, M, tw, Mmax, chirp, bhat);
+    bluestein<T2>(buf, n, M, twp, chirp, bhat);
   else
-    fft_dit<T2, false>(buf, M, tw, Mmax);
+    fft_dit<T2, false>(buf, M, twp);
   // split the two real rings and apply e^{-i m phi0}: for m = k + j n,
   // G[m] = sgn^j e^{-i k phi0} X_k (X^N or X^S)
   GT *GN = G + rowN;
@@ -374,18 +403,21 @@ template <> struct Tables<double2> {
   static const double2 *tw(const Plan &P) { return P.tw64; }
   static const double2 *ch(const Plan &P) { return P.chirp64; }
   static const double2 *bh(const Plan &P) { return P.bhat64; }
+  static const void *tp(const Plan &P) { return P.tp64; }
 };
 template <> struct Tables<float2> {
   static const float2 *ph(const Plan &) { return nullptr; }
   static const float2 *tw(const Plan &P) { return P.tw32; }
   static const float2 *ch(const Plan &P) { return P.chirp32; }
   static const float2 *bh(const Plan &P) { return P.bhat32; }
+  static const void *tp(const Plan &P) { return P.tp32; }
 };
 template <> struct Tables<ddc> {
   static const float4 *ph(const Plan &P) { return P.phasedd; }
   static const float4 *tw(const Plan &P) { return P.twdd; }
   static const float4 *ch(const Plan &P) { return P.chirpdd; }
   static const float4 *bh(const Plan &P) { return P.bhatdd; }
+  static const void *tp(const Plan &P) { return P.tpdd; }
 };
 
 template <typename T2, int MODE>
@@ -396,12 +428,30 @@ static wf_status launch_ring_mode(const Plan &P, const typename CT<T2>::G *F,
                                   int nbatch = 1, long bstride_f = 0, long bstride_m = 0,
                                   bool rows = false) {
   auto kern = k_ring<T2, MODE>;
-  // two launches: the polar rings (pairs 0 .. nside-2, Bluestein unless n is
-  // a power of two) and the equatorial belt (pairs nside-1 .. 2 nside-1);
-  // they touch disjoint rings and run concurrently on two streams
+  // the polar rings (pairs 0 .. nside-2, Bluestein unless n is a power of two) and the
+  // equatorial belt (pairs nside-1 .. 2 nside-1) touch disjoint rings: one launch while
+  // its shared memory (the larger of the two, and the polar rings' chirp tables) lets
+  // four CTAs share an SM, as their registers do; else two, side by side on two streams
   const int npolar = P.nside - 1;
-  const int groups[2][2] = {{0, npolar}, {npolar, P.npairs}};
-  const bool fork = npolar > 0 && P.side_stream;
+  int Mg[2] = {1, 1}, nmin[2] = {INT_MAX, INT_MAX}, tab = 0;
+  for (int k = 0; k < P.npairs; ++k) {
+    const RingPair &rp = P.pairs_h[k];
+    const int g = k >= npolar;
+    Mg[g] = std::max(Mg[g], rp.fftM);
+    nmin[g] = std::min(nmin[g], rp.nphi);
+    if (rp.fftM != rp.nphi) tab = std::max(tab, rp.fftM + rp.nphi);
+  }
+  const int Mall = std::max(Mg[0], Mg[1]), nall = std::min(nmin[0], nmin[1]);
+  // rings with fewer pixels than threads fold through a partial-sum area of 2 x threads
+  // entries placed after the FFT buffer
+  auto bytes = [](int M, int n, int threads) {
+    return sizeof(T2) * (M + (n < threads ? 2 * threads : 0));
+  };
+  constexpr size_t QUARTER = 56 * 1024;
+  const size_t all = bytes(Mall, nall, RING_THREADS);
+  const bool one = all + sizeof(typename CT<T2>::W) * tab <= QUARTER;
+  const int groups[2][2] = {{0, one ? P.npairs : npolar}, {one ? P.npairs : npolar, P.npairs}};
+  const bool fork = !one && npolar > 0 && P.side_stream;
   if (fork) {
     WF_CUDA(cudaEventRecord(P.fork_ev, P.stream));
     WF_CUDA(cudaStreamWaitEvent(P.side_stream, P.fork_ev, 0));
@@ -409,22 +459,19 @@ static wf_status launch_ring_mode(const Plan &P, const typename CT<T2>::G *F,
   for (int g = 0; g < 2; ++g) {
     const int b = groups[g][0], e = groups[g][1];
     if (e <= b) continue;
-    int Mg = 1, nmin = INT_MAX;
-    for (int k = b; k < e; ++k) {
-      Mg = std::max(Mg, P.pairs_h[k].fftM);
-      nmin = std::min(nmin, P.pairs_h[k].nphi);
-    }
-    const int threads = Mg >= 8192 ? RING_THREADS_BIG : RING_THREADS;
-    // rings with fewer pixels than threads fold through a partial-sum area
-    // of 2 x threads entries placed after the FFT buffer
-    const int red_ofs = nmin < threads ? Mg : 0;
-    const size_t smem = sizeof(T2) * (Mg + (nmin < threads ? 2 * threads : 0));
+    const int M = one ? Mall : Mg[g], n = one ? nall : nmin[g];
+    const int threads = M >= 8192 ? RING_THREADS_BIG : RING_THREADS;
+    const int red_ofs = n < threads ? M : 0;
+    size_t smem = bytes(M, n, threads);
+    const int tab_ofs = one && tab ? (int)smem : 0;
+    if (tab_ofs) smem += sizeof(typename CT<T2>::W) * tab;
     cudaStream_t s = (fork && g == 1) ? P.side_stream : P.stream;
     ++P.nlaunch;
     kern<<<dim3(e - b, nbatch), threads, smem, s>>>(
-        P.pairs, b, rows ? 0 : P.npairs, P.lmax, F, G, in_map, out_map, P.nvar, Tables<T2>::tw(P),
-        P.fftMmax, Tables<T2>::ch(P), Tables<T2>::bh(P), st, lstatic, g == 0, in32,
-        P.nvar32, red_ofs, Tables<T2>::ph(P), in_dd, P.nvardd, bstride_f, bstride_m);
+        P.pairs, b, rows ? 0 : P.npairs, P.lmax, F, G, in_map, out_map, P.nvar,
+        Tables<T2>::tw(P), P.fftMmax, static_cast<const TwPair<T2> *>(Tables<T2>::tp(P)),
+        Tables<T2>::ch(P), Tables<T2>::bh(P), st, lstatic, g == 0 ? npolar : 0, in32, P.nvar32,
+        red_ofs, tab_ofs, Tables<T2>::ph(P), in_dd, P.nvardd, bstride_f, bstride_m);
     WF_CUDA(cudaGetLastError());
   }
   if (fork) {

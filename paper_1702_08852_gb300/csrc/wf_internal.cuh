@@ -205,6 +205,7 @@ struct Plan {
   int fftMmax = 1;
   double2 *tw64 = nullptr;       // e^{-2 pi i k / Mmax}, k < Mmax/2
   float2 *tw32 = nullptr;
+  void *tp64 = nullptr, *tp32 = nullptr, *tpdd = nullptr;  // TwPair tables (fft.cuh)
   double2 *chirp64 = nullptr;    // e^{i pi j^2 / n}, per Bluestein ring
   float2 *chirp32 = nullptr;
   double2 *bhat64 = nullptr;     // FFT_M of the chirp kernel, bit-reversed order
