@@ -139,17 +139,14 @@ def measured_peaks():
 
 
 # DRAM bytes (read + write, ncu) of one full-band launch of the FP32 analysis
-# variant the autotuner picks at Nside 1024 / lmax 2048 (an ncu capture of
-# the --kernel-case legendre32 run); scaled to a live launch by its share
-# of the full band's terms.  None once the kernel changes after a capture,
-# and for a plan whose autotuner picked another analysis variant.
-ANALYSIS_DRAM_FULL_BAND = {"nside": 1024, "bytes": 213754624.0,
+# at Nside 1024 / lmax 2048 (an ncu capture of the --kernel-case legendre32
+# run); scaled to a live launch by its share of the full band's terms.  None
+# once the kernel changes after a capture, as the parity-pair analysis has.
+ANALYSIS_DRAM_FULL_BAND = {"nside": 1024, "bytes": None,
                            "terms": 3140761977.0,
                            "variant": {"ana_np": 4, "ana_queue": 0, "ana_packed": 1,
                                        "ana_global_acc": 1},
-                           "source": "ncu --set full, one full-band launch of the kernel "
-                                     "case (dram__bytes_read.sum 137.4 MB + "
-                                     "dram__bytes_write.sum 76.4 MB)"}
+                           "source": "no capture since the kernel changed"}
 
 
 def analysis_variant(tuning):
@@ -182,10 +179,10 @@ def alu_peaks(wf):
             "source": "measured live: wf_alu_peak FMA chains on every SM, best of 5"}
 
 
-# FP32 flops of the double-float formulas per (l, m, ring pair) term: the
-# recurrence step (product c u, product by z, difference: 28 with an FMA
-# counted as 2) and two accumulations of a product (15 each)
-DD_FLOPS_PER_TERM = 58.0
+# FP32 operations of the double-float formulas per (l, m, ring pair) term: 84
+# per step of the parity-pair recurrence (the step and four accumulations of a
+# product), which serves two l
+DD_FLOPS_PER_TERM = 42.0
 KERNEL_NAMES = ["legendre_analysis_f32", "legendre_synthesis_f32", "ring_step_f32",
                 "legendre_synthesis_dd", "legendre_analysis_dd", "ring_step_dd"]
 
@@ -194,7 +191,7 @@ def kernel_rooflines(kern, alu, peaks, peak_src, args, ana_variant):
     """Per-kernel rooflines of the timed solves (wf_kernel_stats, CUDA events
     around every launch) and the dominant kernel's at the top level.
     Legendre kernels: 7 algorithmic flops per term against the measured FP32
-    FMA peak (the double-float ones: the 58 FP32 flops of their formulas per
+    FMA peak (the double-float ones: the 42 FP32 operations of their formulas per
     term against the same peak, and their FP64-equivalent 7 flops per term
     beside the measured FP64 peak); ring steps: DRAM bytes they cannot avoid
     against the measured copy bandwidth."""

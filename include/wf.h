@@ -354,7 +354,7 @@ wf_status wf_trace(wf_plan_t plan, int *count, int *stage, double *xi,
  *            1 = Legendre synthesis, 2 = ring step (fold, inverse ring
  *            FFTs, the t-update of Eq. 14, forward ring FFTs; both launches)
  *            of the captured FP32 / FP64 iterations; 3 = Legendre
- *            synthesis, 4 = Legendre analysis (with its tile combine),
+ *            synthesis, 4 = Legendre analysis,
  *            5 = ring step, all three in double-float, of the mixed solver's
  *            anchor-arithmetic steps (anchors, stage boundaries, tail).
  *  ms        summed CUDA-event time of the timed launches.

@@ -11,9 +11,12 @@
 //      mu = xi - alpha, the band limit of the next stage, trace, stop.
 // The order follows Algorithm 2: s and t of iteration i use the xi of the
 // stage that produced x_i; the cooling happens after the Cauchy test.
-// Iterations are captured in a CUDA graph of `chunk` iterations; every kernel
-// returns at once when the control kernel has set `done`, so the host only
-// polls the state between graph launches.
+// Iterations are captured in a CUDA graph whose WHILE node repeats a few of
+// them until the control kernel clears its condition: one launch per solve
+// loop, no polling (graphs of `chunk` iterations launched until the state
+// reads done ran up to half of their slots empty).  opts.timing keeps those
+// graphs, with events around each kernel.  Every kernel returns at once when
+// the control kernel has set `done`.
 #include <math.h>
 
 #include <algorithm>
