@@ -32,10 +32,13 @@
 // Near the equator Q_j grows like lam / z while neighbouring Q_j cancel in
 // lam_{m+2j}, so rounding in s_j is amplified by up to 1/z there (measured in
 // FP64 at Nside 1024: 1.1e-13 of the map's rms on the rings next to the equator,
-// 1.5e-15 with the one-step recurrence).  The FP64 synthesis therefore gives the
-// ring pairs k >= keq (|z| < ~0.2, where lam_mm itself is the seed for every m)
-// to the one-step recurrence lam_l <- z lam_{l-1}, lam_{l-2}, two l per j, at 8
-// multiply-adds instead of 6.  The analysis, which sums over all rings, does not
+// 1.5e-15 with the one-step recurrence).  The FP64 and double-float syntheses
+// therefore give the ring pairs k >= keq (|z| < 1/6 and what makes whole warps, where
+// lam_mm itself is the seed for every m: equatorial_pair) to the one-step recurrence
+// lam_l <- z lam_{l-1}, lam_{l-2}, two l per j, at 8 multiply-adds instead of 6.  They
+// get warps, and in FP64 CTAs, of their own, so no number of pairs per thread and no
+// Nside mixes the two kinds (Nside 128, ring pairs 254 and 255: 2.8e-14 of the rms
+// without it, 4.3e-15 with it).  The analysis, which sums over all rings, does not
 // need it (2.6e-14 of the rms against 3.0e-14 with the one-step recurrence).
 //
 // Bound: the FP64 unit, 2 multiply-adds per clock and SM.  At Nside 1024, lmax 2048
@@ -167,6 +170,18 @@ __device__ __forceinline__ void accv(dd &acc, dd s, dd x) {
   acc.hi = two_sum(acc.hi, p, err);
   acc.lo = __fadd_rn(acc.lo, __fadd_rn(err, e));
 }
+// c z f + acc, the step of the one-step recurrence (equator)
+__device__ __forceinline__ double eqv(double c, double z, double f, double acc) {
+  return fma(c * z, f, acc);
+}
+__device__ __forceinline__ float eqv(float c, float z, float f, float acc) {
+  return fmaf(c * z, f, acc);
+}
+__device__ __forceinline__ dd eqv(dd c, dd z, dd f, dd acc) {
+  dd x;
+  dd_prod(c, z, x.hi, x.lo);
+  return fmav(x, f, acc);
+}
 __device__ __forceinline__ double coefv(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float coefv(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double shfx(double v, int s) { return __shfl_xor_sync(0xffffffffu, v, s); }
@@ -218,7 +233,7 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
     k_pair_synth(const PairTab<V> t, int npairs, int lmax,
                  const typename Cx<V>::type *__restrict__ x,
                  typename Cx<V>::type *__restrict__ F, const SolverState *__restrict__ st,
-                 int lstatic) {
+                 int lstatic, int nlow, int eq_ofs) {
   typedef typename Cx<V>::type C;
   const int m = blockIdx.y;
   int L = lstatic;
@@ -232,16 +247,24 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
   const int J = (L - m) / 2 + 1;
   // per j a quad (E_re, E_im, O_re, O_im), or, PK, two: (E_re, E_re, E_im, E_im),
   // (O_re, O_re, O_im, O_im); then the forms' (A, B), [NF][J]
+  constexpr int QJ = PK ? 2 : 1;
+  constexpr int NE = PK ? NP : 1;  // equatorial pairs per thread
   Quad<V> *sx = reinterpret_cast<Quad<V> *>(smraw);
-  Pair<V> *srec = reinterpret_cast<Pair<V> *>(smraw + sizeof(Quad<V>) * J * (PK ? 2 : 1));
-  const int pair00 = blockIdx.x * blockDim.x * NP;
+  Pair<V> *srec = reinterpret_cast<Pair<V> *>(sx + QJ * J);
+  // the same for the equatorial warps, where the CTA has both kinds behind the others
+  Quad<V> *sxe = reinterpret_cast<Quad<V> *>(smraw + eq_ofs);
+  Pair<V> *sre = reinterpret_cast<Pair<V> *>(sxe + QJ * J);
+  // the first nlow warps of a row take the pairs below keq, the others the equatorial ones
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int warp0 = blockIdx.x * nw;
+  const bool equator = warp0 + warp >= nlow;
+  const int pair0 = equator ? t.keq + (warp0 + warp - nlow) * 32 * NE
+                            : (warp0 + warp) * 32 * NP;
+  const int kend = equator ? npairs : t.keq;
   // FP32 CTAs span several forms: all three are staged and each warp takes its own;
   // FP64 CTAs (at most 64 pairs) stage one
   constexpr int NF = std::is_same<V, float>::value ? 3 : 1;
-  const bool equator = t.rec_e && pair00 >= t.keq;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int pair0 = pair00 + warp * 32 * NP;
-  const int form = t.form(NF == 1 ? pair00 + (int)blockDim.x / 2 - 1 : pair0 + 16 * NP - 1);
+  const int form = t.form(NF == 1 ? warp0 * 32 * NP + (int)blockDim.x / 2 - 1 : pair0 + 16 * NP - 1);
   const V *wt = t.w + form * t.stride;
   V w[NP];
   int js[NP];
@@ -250,83 +273,83 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
     const int k = pair0 + lane + 32 * i;
     w[i] = V(0);
     js[i] = INT_MAX / 2;
-    if (k < npairs) {
+    if (!equator && k < kend) {
       w[i] = wt[k];
       js[i] = t.js[(long)m * t.stride + k];
     }
   }
   {
     const long q0 = pair_base(lmax, m), a0 = alm_base(lmax, m);
-    const Pair<V> *rec = reinterpret_cast<const Pair<V> *>(equator ? t.rec_e : t.rec[form]);
+    auto put = [](Quad<V> *q, int j, V er, V ei, V orr, V oi) {
+      if constexpr (PK) {
+        q[2 * j] = {er, er, ei, ei};
+        q[2 * j + 1] = {orr, orr, oi, oi};
+      } else {
+        q[j] = {er, ei, orr, oi};
+      }
+    };
     for (int j = threadIdx.x; j < J; j += blockDim.x) {
       const int l = m + 2 * j;
       const C c0 = x[a0 + 2 * j];
       C c1 = {}, c2 = {};
       if (l + 1 <= L) c1 = x[a0 + 2 * j + 1];
       if (l + 2 <= L) c2 = x[a0 + 2 * j + 2];
-      if (equator) {
+      if (t.rec_e && warp0 + nw > nlow) {
         const V ge = t.ge[q0 + j], go = t.go[q0 + j];
-        sx[j] = {ge * c0.x, ge * c0.y, go * c1.x, go * c1.y};
-        srec[j] = rec[q0 + j];
-        continue;
+        put(sxe, j, ge * c0.x, ge * c0.y, go * c1.x, go * c1.y);
+        sre[j] = reinterpret_cast<const Pair<V> *>(t.rec_e)[q0 + j];
       }
-      const V se = t.se[q0 + j], sn = t.sn[q0 + j], so = t.so[q0 + j];
-      const V xr = fmav(se, c0.x, sn * c2.x), xi = fmav(se, c0.y, sn * c2.y);
-      const V yr = so * c1.x, yi = so * c1.y;
-      if constexpr (PK) {
-        sx[2 * j] = {xr, xr, xi, xi};
-        sx[2 * j + 1] = {yr, yr, yi, yi};
-      } else {
-        sx[j] = {xr, xi, yr, yi};
-      }
-      if constexpr (NF == 1) {
-        srec[j] = rec[q0 + j];
-      } else {
+      if (warp0 < nlow) {
+        const V se = t.se[q0 + j], sn = t.sn[q0 + j], so = t.so[q0 + j];
+        put(sx, j, fmav(se, c0.x, sn * c2.x), fmav(se, c0.y, sn * c2.y), so * c1.x, so * c1.y);
+        if constexpr (NF == 1) {
+          srec[j] = reinterpret_cast<const Pair<V> *>(t.rec[form])[q0 + j];
+        } else {
 #pragma unroll
-        for (int f = 0; f < NF; ++f)
-          srec[f * J + j] = reinterpret_cast<const Pair<V> *>(t.rec[f])[q0 + j];
+          for (int f = 0; f < NF; ++f)
+            srec[f * J + j] = reinterpret_cast<const Pair<V> *>(t.rec[f])[q0 + j];
+        }
       }
     }
   }
   __syncthreads();
-  if (pair0 >= npairs) return;
-  const Pair<V> *sr = srec + (NF == 1 ? 0 : form * J);
+  if (pair0 >= kend) return;
 
   Quad<V> *out = reinterpret_cast<Quad<V> *>(F) + (long)m * npairs;
   if (equator) {
-    V z[NP], u[NP], o[NP], er[NP], ei[NP], orr[NP], oi[NP];
+    V z[NE], u[NE], o[NE], er[NE], ei[NE], orr[NE], oi[NE];
 #pragma unroll
-    for (int i = 0; i < NP; ++i) {
+    for (int i = 0; i < NE; ++i) {
       const int k = pair0 + lane + 32 * i;
-      u[i] = o[i] = er[i] = ei[i] = orr[i] = oi[i] = z[i] = V(0);
-      if (k < npairs) {
+      z[i] = u[i] = o[i] = er[i] = ei[i] = orr[i] = oi[i] = V(0);
+      if (k < kend) {
         z[i] = t.z[k];
-        u[i] = t.lmm[(long)m * npairs + k];  // lam_mm
+        u[i] = t.lmm[(long)m * npairs + k];
       }
     }
-#pragma unroll 2
+#pragma unroll 4
     for (int j = 0; j < J; ++j) {
-      const Pair<V> r = sr[j];
-      const Quad<V> q = sx[j];
+      const Pair<V> r = sre[j];
+      const Quad<V> q = sxe[j];
 #pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        u[i] = fmav(r.a * z[i], o[i], u[i]);
+      for (int i = 0; i < NE; ++i) {
+        u[i] = eqv(r.a, z[i], o[i], u[i]);
         accv(er[i], u[i], q.a);
         accv(ei[i], u[i], q.b);
-        o[i] = fmav(r.b * z[i], u[i], o[i]);
+        o[i] = eqv(r.b, z[i], u[i], o[i]);
         accv(orr[i], o[i], q.c);
         accv(oi[i], o[i], q.d);
       }
     }
 #pragma unroll
-    for (int i = 0; i < NP; ++i) {
+    for (int i = 0; i < NE; ++i) {
       const int k = pair0 + lane + 32 * i;
-      if (k >= npairs) continue;
-      out[k] = {er[i] + orr[i], ei[i] + oi[i], er[i] - orr[i], ei[i] - oi[i]};
+      if (k < kend) out[k] = {er[i] + orr[i], ei[i] + oi[i], er[i] - orr[i], ei[i] - oi[i]};
     }
     return;
   }
 
+  const Pair<V> *sr = srec + (NF == 1 ? 0 : form * J);
   V s1[NP], s2[NP], d0[NP], d1[NP], er[NP], ei[NP], orr[NP], oi[NP];
   int jmin = INT_MAX, jinj = -1;
 #pragma unroll
@@ -398,7 +421,7 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
     const int k = pair0 + lane + 32 * i;
-    if (k >= npairs) continue;
+    if (k >= kend) continue;
     const V z = t.z[k], zr = z * orr[i], zi = z * oi[i];
     out[k] = {er[i] + zr, ei[i] + zi, er[i] - zr, ei[i] - zi};
   }
@@ -744,10 +767,25 @@ __global__ void __launch_bounds__(32 * PANA_MAXWARPS, std::is_same<V, double>::v
 }
 
 // ------------------------------------------------------------- launch
-// per j: a quad (packed FP32: two) and one form's pair (FP32: three)
-static size_t synth_smem(size_t v, int lmax, bool packed = false) {
-  return ((packed ? 8 : 4) + (v == 4 ? 6 : 2)) * v * (lmax / 2 + 1);
-}
+// The synthesis' warps: nlow of 32 np pairs each below keq, then the equatorial ones; mix:
+// in the same CTAs, else the equatorial ones in CTAs of their own.  Shared memory per j: a
+// quad (packed FP32: two) and one form's pair (FP32: three), equatorial a quad or two and
+// a pair.
+struct SynthGrid {
+  unsigned ctas;
+  int nlow, eq_ofs;
+  size_t smem;
+  SynthGrid(size_t v, int npairs, int keq, int lmax, int threads, int np, bool packed, bool mix) {
+    const int nw = threads / 32, j = lmax / 2 + 1, ne = packed ? np : 1;
+    const size_t quads = packed ? 8 : 4, low = (quads + (v == 4 ? 6 : 2)) * v * j,
+                 eq = (quads + 2) * v * j;
+    nlow = (keq + 32 * np - 1) / (32 * np);
+    if (!mix) nlow = (nlow + nw - 1) / nw * nw;
+    ctas = (unsigned)((nlow + (npairs - keq + 32 * ne - 1) / (32 * ne) + nw - 1) / nw);
+    eq_ofs = mix ? (int)((low + 15) / 16 * 16) : 0;
+    smem = mix ? eq_ofs + eq : low;
+  }
+};
 static size_t anal_smem(size_t v, int npairs, int lmax) {
   const size_t j16 = (size_t)(lmax / 32 + 1) * CKJ;
   return 4 * v * std::min((npairs + 63) / 64 * 64, PANA_TILE) + 10 * v * j16;
@@ -756,9 +794,9 @@ static size_t anal_smem(size_t v, int npairs, int lmax) {
 template <int NP>
 static void synth64(const Plan &P, const double2 *x, double2 *F, const SolverState *st,
                     int lstatic, int threads) {
-  const dim3 grid((P.npairs + threads * NP - 1) / (threads * NP), P.lmax + 1);
-  k_pair_synth<double, NP><<<grid, threads, synth_smem(8, P.lmax), P.stream>>>(
-      P.pt64, P.npairs, P.lmax, x, F, st, lstatic);
+  const SynthGrid g(8, P.npairs, P.pt64.keq, P.lmax, threads, NP, false, false);
+  k_pair_synth<double, NP><<<dim3(g.ctas, P.lmax + 1), threads, g.smem, P.stream>>>(
+      P.pt64, P.npairs, P.lmax, x, F, st, lstatic, g.nlow, g.eq_ofs);
 }
 
 template <>
@@ -793,11 +831,11 @@ wf_status launch_legendre_anal<double2>(const Plan &P, const double2 *G, double2
 template <int NP>
 static void synth32(const Plan &P, const float2 *x, float2 *F, const SolverState *st,
                     int lstatic) {
-  const int tile = PSYN_THREADS32 * NP;
-  const dim3 grid((P.npairs + tile - 1) / tile, P.lmax + 1);
-  k_pair_synth<float, NP>
-      <<<grid, PSYN_THREADS32, synth_smem(4, P.lmax, NP % 2 == 0), P.stream>>>(
-          P.pt32, P.npairs, P.lmax, x, F, st, lstatic);
+  // small maps: both kinds of pairs in a CTA, so that no part of one idles
+  const SynthGrid g(4, P.npairs, P.pt32.keq, P.lmax, PSYN_THREADS32, NP, NP % 2 == 0,
+                    P.npairs < 1024);
+  k_pair_synth<float, NP><<<dim3(g.ctas, P.lmax + 1), PSYN_THREADS32, g.smem, P.stream>>>(
+      P.pt32, P.npairs, P.lmax, x, F, st, lstatic, g.nlow, g.eq_ofs);
 }
 
 template <>
@@ -829,12 +867,11 @@ wf_status launch_legendre_anal<float2>(const Plan &P, const float2 *G, double2 *
 template <int NP>
 static void synth_dd(const Plan &P, const float4 *x, float4 *F, const SolverState *st,
                      int lstatic) {
-  const int tile = PSYN_THREADS * NP;
-  const dim3 grid((P.npairs + tile - 1) / tile, P.lmax + 1);
+  const SynthGrid g(8, P.npairs, P.ptdd.keq, P.lmax, PSYN_THREADS, NP, false, false);
   typedef Cx<dd>::type C;
-  k_pair_synth<dd, NP><<<grid, PSYN_THREADS, synth_smem(8, P.lmax), P.stream>>>(
+  k_pair_synth<dd, NP><<<dim3(g.ctas, P.lmax + 1), PSYN_THREADS, g.smem, P.stream>>>(
       P.ptdd, P.npairs, P.lmax, reinterpret_cast<const C *>(x), reinterpret_cast<C *>(F), st,
-      lstatic);
+      lstatic, g.nlow, g.eq_ofs);
 }
 
 wf_status launch_legendre_synth_dd(const Plan &P, const float4 *xs, float4 *F,
@@ -1103,6 +1140,22 @@ __global__ void k_pair_lmm(int npairs, int lmax, int keq, const double *__restri
 static wf_status build_pair_tables32(Plan &P, long nq);
 static wf_status build_pair_tables_dd(Plan &P, long nq);
 
+// The first of the pairs that take the one-step recurrence: those with |z| < 1/6 (above,
+// the two recurrences' errors are within a factor of two, and the parity-pair basis is
+// the better one from |z| ~ 1/2 on), as far as lam_mm, where it starts, stays above 2^-90
+// for every m.  From a multiple of 64 or 32 on where lam_mm allows it and |z| stays below
+// 4/9: the kernels take 32 or 64 pairs at a time, and a part of them costs as much as all.
+static int equatorial_pair(const Plan &P) {
+  auto starts = [&P](int k) { return P.lmax * log2(P.pairs_h[k].sth) > -90.0; };
+  int k = P.npairs;
+  while (k > 0 && P.pairs_h[k - 1].z < 1.0 / 6.0 && starts(k - 1)) --k;
+  for (int step = P.npairs < 512 ? 32 : 64; step >= 32; step /= 2) {
+    const int whole = k / step * step;
+    if (3 * whole >= 2 * P.npairs && starts(whole)) return whole;
+  }
+  return k;
+}
+
 // The tables and the checkpoints.  mant, expo: lam_mm of every (m, pair).
 wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
   const int lmax = P.lmax;
@@ -1125,10 +1178,7 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
     WF_CUDA(cudaMemcpy(*dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice));
     return WF_OK;
   };
-  // the equatorial pairs, in whole CTAs of the synthesis
-  int keq = P.npairs;
-  while (keq > 0 && z[keq - 1] < 0.2 && lmax * log2(P.pairs_h[keq - 1].sth) > -90.0) --keq;
-  keq = (keq + PSYN_THREADS - 1) / PSYN_THREADS * PSYN_THREADS;
+  const int keq = equatorial_pair(P);
   PairTab<double> &t = P.pt64;
   for (int f = 0; f < 2; ++f) t.kform[f] = (kform[f] + 16) / 32 * 32;
   t.keq = keq;

@@ -1,0 +1,127 @@
+"""Accuracy on the rings next to the equator, ring by ring.
+
+There Q_j = lam / z of the parity-pair basis amplifies rounding by up to 1/z, so the
+Legendre kernels switch to the one-step recurrence; the norm over a whole map does not
+show whether they do.  Its lmax + 1 steps each leave a rounding of at most u of an O(1)
+value, in a recurrence that neither grows nor shrinks there, and the sums as many again:
+they add like a random walk, so the error is held to 4 u sqrt(lmax + 1) of the rms.  u is
+2^-53 in FP64, 2^-24 in FP32 and 2^-47 in double-float (an operation's bound)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+UNIT = {"f64": 2.0 ** -53, "f32": 2.0 ** -24, "df64": 2.0 ** -47}
+
+
+def tol(prec, lmax):
+    return 4.0 * UNIT[prec] * np.sqrt(lmax + 1.0)
+
+
+@pytest.fixture(scope="module")
+def torch_cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1702_08852_gb300 import build
+    build.build()
+    return torch
+
+
+def rand_alm(lmax, seed):
+    from paper_1702_08852_gb300 import inputs
+    rng = np.random.default_rng(seed)
+    n = inputs.nalm(lmax)
+    a = rng.standard_normal(n) + 1j * rng.standard_normal(n)
+    _, ms = inputs.lm_of_slots(lmax)
+    a[ms == 0] = a[ms == 0].real
+    return a
+
+
+def walk(osht, nside, lmax, i):
+    """(l, lam_lm(z) of m = 0 .. l) for l = 0 .. lmax on ring i, the textbook recurrence in
+    long double, from the oracle's lam_mm (its rounding scales a whole m and is not the
+    recurrence's)."""
+    ld = np.longdouble
+    m = np.arange(lmax + 1, dtype=ld)
+    _, _, z, sth, _ = osht.ring_info(nside, i)
+    z = ld(z)
+    k = np.arange(lmax + 1)
+    mm = osht.lambda_all(lmax, z, sth)[osht.alm_index(lmax, k, k)].astype(ld)
+    prev, cur = np.zeros(lmax + 1, ld), np.zeros(lmax + 1, ld)
+    cur[0] = mm[0]
+    yield 0, cur[:1]
+    for l in range(1, lmax + 1):
+        k = m[:l]
+        a = np.sqrt((4 * ld(l) * l - 1) / (ld(l) * l - k * k))
+        b = np.sqrt(((ld(l) - 1) ** 2 - k * k) / (4 * (ld(l) - 1) ** 2 - 1))
+        nxt = np.zeros(lmax + 1, ld)
+        nxt[:l] = a * (z * cur[:l] - b * prev[:l])
+        nxt[l] = mm[l]
+        prev, cur = cur, nxt
+        yield l, cur[:l + 1]
+
+
+def slots(lmax, l):
+    m = np.arange(l + 1)
+    return m * (2 * lmax + 1 - m) // 2 + l
+
+
+def ring(nside, i):
+    """(first pixel, phase step num: phi_0 = pi num / (4 nside)) of the belt's ring i
+    (nside <= i <= 3 nside), 4 nside pixels."""
+    return 2 * nside * (nside - 1) + (i - nside) * 4 * nside, 0 if (i + nside) & 1 else 1
+
+
+def phase(nside, lmax, num):
+    m = np.arange(lmax + 1)
+    return np.exp(1j * np.pi * ((m * num) % (8 * nside)) / (4.0 * nside))
+
+
+def synth_rings(osht, a, nside, lmax, i):
+    """The belt's rings i and 4 nside - i (i <= 2 nside) of Y a."""
+    _, num = ring(nside, i)
+    f = np.zeros((2, lmax + 1), np.clongdouble)
+    for l, lam in walk(osht, nside, lmax, i):
+        v = lam * a[slots(lmax, l)]
+        s = 1 - 2 * ((np.arange(l + 1) + l) & 1)
+        f[0, :l + 1] += v
+        f[1, :l + 1] += s * v
+    f = f.astype(np.complex128) * phase(nside, lmax, num)
+    n = 4 * nside
+    out = []
+    for row in f:
+        c = np.zeros(n, complex)
+        np.add.at(c, np.arange(lmax + 1) % n, row)
+        np.add.at(c, -np.arange(1, lmax + 1) % n, row[1:].conj())
+        out.append((np.fft.ifft(c) * n).real)
+    return out
+
+
+def check_synthesis(torch, osht, prec, nside, lmax, variant=None):
+    from paper_1702_08852_gb300 import wf
+    a = rand_alm(lmax, nside + lmax)
+    rings = [2 * nside, 2 * nside - 1, 2 * nside - 2, 2 * nside - 4]
+    with wf.Plan(nside, lmax, np.ones(lmax + 1)) as p:
+        if variant:
+            p.set_tuning(**variant)
+        f = {"f64": p.alm2map, "f32": p.alm2map_f32, "df64": p.alm2map_df64}[prec]
+        got = f(torch.from_numpy(a).cuda()).cpu().numpy()
+    for i in rings:
+        for j, ref in zip((i, 4 * nside - i), synth_rings(osht, a, nside, lmax, i)):
+            first = ring(nside, j)[0]
+            err = got[first:first + 4 * nside] - ref
+            assert np.sqrt(np.mean(err ** 2)) <= tol(prec, lmax) * np.sqrt(np.mean(ref ** 2)), j
+
+
+# whole warps of pairs from the equator on (64, 128, 192), a part of one (75), the pairs
+# per thread that a plan may run
+@pytest.mark.parametrize("nside,lmax", [(64, 128), (75, 150), (128, 256), (192, 384), (512, 1024)])
+@pytest.mark.parametrize("np_", [1, 2, 4])
+def test_synthesis_f64(torch_cuda, osht, nside, lmax, np_):
+    check_synthesis(torch_cuda, osht, "f64", nside, lmax, {"syn_np": [np_, 2]})
+
+
+@pytest.mark.parametrize("nside,lmax", [(75, 150), (128, 256), (192, 384)])
+def test_synthesis_df64(torch_cuda, osht, nside, lmax):
+    check_synthesis(torch_cuda, osht, "df64", nside, lmax)
