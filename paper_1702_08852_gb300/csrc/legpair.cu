@@ -32,13 +32,13 @@
 // Near the equator Q_j grows like lam / z while neighbouring Q_j cancel in
 // lam_{m+2j}, so rounding in s_j is amplified by up to 1/z there (measured in
 // FP64 at Nside 1024: 1.1e-13 of the map's rms on the rings next to the equator,
-// 1.5e-15 with the one-step recurrence).  The FP64 and double-float syntheses
-// therefore give the ring pairs k >= keq (|z| < 1/6 and what makes whole warps, where
-// lam_mm itself is the seed for every m: equatorial_pair) to the one-step recurrence
-// lam_l <- z lam_{l-1}, lam_{l-2}, two l per j, at 8 multiply-adds instead of 6.  They
-// get warps, and in FP64 CTAs, of their own, so no number of pairs per thread and no
-// Nside mixes the two kinds (Nside 128, ring pairs 254 and 255: 2.8e-14 of the rms
-// without it, 4.3e-15 with it).  The analysis, which sums over all rings, does not
+// 1.5e-15 with the one-step recurrence; in FP32 7e-5 at Nside 256 and 4e-4 at
+// Nside 1024, 4e-7 and 1e-6 with it).  The synthesis therefore gives the ring pairs k >= keq
+// (|z| < 1/6 and what makes whole warps, where lam_mm itself is the seed for every m:
+// equatorial_pair) to the one-step recurrence lam_l <- z lam_{l-1}, lam_{l-2}, two l per
+// j, at 8 multiply-adds instead of 6 (FP32: 10, z in two parts).  They get warps, and in
+// FP64 CTAs, of their own, so no number of pairs per thread and no Nside mixes the two
+// kinds.  The analysis, which sums over all rings, does not
 // need it (2.6e-14 of the rms against 3.0e-14 with the one-step recurrence).
 //
 // Bound: the FP64 unit, 2 multiply-adds per clock and SM.  At Nside 1024, lmax 2048
@@ -170,17 +170,27 @@ __device__ __forceinline__ void accv(dd &acc, dd s, dd x) {
   acc.hi = two_sum(acc.hi, p, err);
   acc.lo = __fadd_rn(acc.lo, __fadd_rn(err, e));
 }
-// c z f + acc, the step of the one-step recurrence (equator)
-__device__ __forceinline__ double eqv(double c, double z, double f, double acc) {
+// c z f + acc, the step of the one-step recurrence (equator); FP32 carries z in two
+// parts and rounds c f: c nears 2 along l, and a rounded c z would add up its error
+__device__ __forceinline__ double eqv(double c, double z, double, double f, double acc) {
   return fma(c * z, f, acc);
 }
-__device__ __forceinline__ float eqv(float c, float z, float f, float acc) {
-  return fmaf(c * z, f, acc);
+__device__ __forceinline__ float eqv(float c, float z, float zl, float f, float acc) {
+  const float x = c * f;
+  return fmaf(x, z, fmaf(x, zl, acc));
 }
-__device__ __forceinline__ dd eqv(dd c, dd z, dd f, dd acc) {
+__device__ __forceinline__ dd eqv(dd c, dd z, dd, dd f, dd acc) {
   dd x;
   dd_prod(c, z, x.hi, x.lo);
   return fmav(x, f, acc);
+}
+// the same for two pairs, each half rounded as the scalar one
+__device__ __forceinline__ void eqv2(float c, float z0, float z1, float l0, float l1, float f0,
+                                     float f1, float &a0, float &a1) {
+  float t0, t1;
+  const float x0 = c * f0, x1 = c * f1;
+  fma2(t0, t1, x0, x1, l0, l1, a0, a1);
+  fma2(a0, a1, x0, x1, z0, z1, t0, t1);
 }
 __device__ __forceinline__ double coefv(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float coefv(float a, float b, float c) { return fmaf(a, b, c); }
@@ -294,7 +304,7 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
       C c1 = {}, c2 = {};
       if (l + 1 <= L) c1 = x[a0 + 2 * j + 1];
       if (l + 2 <= L) c2 = x[a0 + 2 * j + 2];
-      if (t.rec_e && warp0 + nw > nlow) {
+      if (warp0 + nw > nlow) {
         const V ge = t.ge[q0 + j], go = t.go[q0 + j];
         put(sxe, j, ge * c0.x, ge * c0.y, go * c1.x, go * c1.y);
         sre[j] = reinterpret_cast<const Pair<V> *>(t.rec_e)[q0 + j];
@@ -317,28 +327,42 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
 
   Quad<V> *out = reinterpret_cast<Quad<V> *>(F) + (long)m * npairs;
   if (equator) {
-    V z[NE], u[NE], o[NE], er[NE], ei[NE], orr[NE], oi[NE];
+    V z[NE], zl[NE], u[NE], o[NE], er[NE], ei[NE], orr[NE], oi[NE];
 #pragma unroll
     for (int i = 0; i < NE; ++i) {
       const int k = pair0 + lane + 32 * i;
-      z[i] = u[i] = o[i] = er[i] = ei[i] = orr[i] = oi[i] = V(0);
+      z[i] = zl[i] = u[i] = o[i] = er[i] = ei[i] = orr[i] = oi[i] = V(0);
       if (k < kend) {
         z[i] = t.z[k];
+        if constexpr (std::is_same<V, float>::value) zl[i] = t.zl[k];
         u[i] = t.lmm[(long)m * npairs + k];
       }
     }
 #pragma unroll 4
     for (int j = 0; j < J; ++j) {
       const Pair<V> r = sre[j];
-      const Quad<V> q = sxe[j];
+      if constexpr (PK) {
+        const Quad<V> xe = sxe[2 * j], xo = sxe[2 * j + 1];
 #pragma unroll
-      for (int i = 0; i < NE; ++i) {
-        u[i] = eqv(r.a, z[i], o[i], u[i]);
-        accv(er[i], u[i], q.a);
-        accv(ei[i], u[i], q.b);
-        o[i] = eqv(r.b, z[i], u[i], o[i]);
-        accv(orr[i], o[i], q.c);
-        accv(oi[i], o[i], q.d);
+        for (int i = 0; i < NE; i += 2) {
+          eqv2(r.a, z[i], z[i + 1], zl[i], zl[i + 1], o[i], o[i + 1], u[i], u[i + 1]);
+          fma2(er[i], er[i + 1], u[i], u[i + 1], xe.a, xe.b, er[i], er[i + 1]);
+          fma2(ei[i], ei[i + 1], u[i], u[i + 1], xe.c, xe.d, ei[i], ei[i + 1]);
+          eqv2(r.b, z[i], z[i + 1], zl[i], zl[i + 1], u[i], u[i + 1], o[i], o[i + 1]);
+          fma2(orr[i], orr[i + 1], o[i], o[i + 1], xo.a, xo.b, orr[i], orr[i + 1]);
+          fma2(oi[i], oi[i + 1], o[i], o[i + 1], xo.c, xo.d, oi[i], oi[i + 1]);
+        }
+      } else {
+        const Quad<V> q = sxe[j];
+#pragma unroll
+        for (int i = 0; i < NE; ++i) {
+          u[i] = eqv(r.a, z[i], zl[i], o[i], u[i]);
+          accv(er[i], u[i], q.a);
+          accv(ei[i], u[i], q.b);
+          o[i] = eqv(r.b, z[i], zl[i], u[i], o[i]);
+          accv(orr[i], o[i], q.c);
+          accv(oi[i], o[i], q.d);
+        }
       }
     }
 #pragma unroll
@@ -1163,10 +1187,12 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
   const long nb = block_base(lmax, lmax) + 1;
   const int stride = (P.npairs + 63) / 64 * 64;  // rows padded to whole steps
   std::vector<double> w(3 * (size_t)stride, 0.0), z(stride, 0.0);
+  std::vector<float> zl(stride, 0.f);
   // the forms' limits z^2 = 3/4 and 1/4, in whole warps of pairs
   int kform[2] = {0, 0};
   for (int k = 0; k < P.npairs; ++k) {
     z[k] = P.pairs_h[k].z;
+    zl[k] = (float)(z[k] - (double)(float)z[k]);
     for (int f = 0; f < 2; ++f)
       if (z[k] * z[k] > (f ? 0.25 : 0.75)) kform[f] = k + 1;
     w[k] = -(1.0 - z[k]) * (1.0 + z[k]);
@@ -1185,6 +1211,7 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
   t.stride = stride;
   WF_TRY(up(&t.w, w));
   WF_TRY(up(&t.z, z));
+  WF_TRY(up(&P.pt32.zl, zl));
   for (double2 **a : {&t.rec[0], &t.rec[1], &t.rec[2], &t.rec_e})
     WF_CUDA(cudaMalloc(a, sizeof(double2) * nq));
   for (double **a : {&t.se, &t.sn, &t.so, &t.ge, &t.go})
@@ -1248,9 +1275,13 @@ static wf_status build_pair_tables32(Plan &P, long nq) {
   WF_TRY(round(&u.so, t.so, nq));
   WF_TRY(round(&u.w, t.w, 3L * t.stride));
   WF_TRY(round(&u.z, t.z, t.stride));
+  WF_TRY(round(&u.rec_e, t.rec_e, 2 * nq));
+  WF_TRY(round(&u.ge, t.ge, nq));
+  WF_TRY(round(&u.go, t.go, nq));
+  if (t.lmm) WF_TRY(round(&u.lmm, t.lmm, (long)P.npairs * (P.lmax + 1)));
   u.stride = t.stride;
   for (int f = 0; f < 2; ++f) u.kform[f] = t.kform[f];
-  u.keq = P.npairs;
+  u.keq = t.keq;
   return WF_OK;
 }
 
@@ -1299,7 +1330,8 @@ void free_pair_tables(Plan &P) {
   for (void *p : g)
     if (p) cudaFree(p);
   PairTab<float> &u = P.pt32;
-  void *f[] = {u.rec[0], u.rec[1], u.rec[2], u.se, u.sn, u.so, u.w, u.z, u.ck, u.jin, u.seed};
+  void *f[] = {u.rec[0], u.rec[1], u.rec[2], u.se, u.sn, u.so, u.w, u.z, u.ck, u.jin, u.seed,
+               u.rec_e, u.ge, u.go, u.zl, u.lmm};
   for (void *p : f)
     if (p) cudaFree(p);
   PairTab<double> &t = P.pt64;

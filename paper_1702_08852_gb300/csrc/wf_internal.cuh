@@ -54,7 +54,7 @@ struct PairTab {
   V *se = nullptr, *sn = nullptr, *so = nullptr;  // basis change, scales and signs included
   int stride = 0;                  // row length: npairs rounded up to 64
   V *w = nullptr;                  // [3][stride]: z^2 - 1, z^2 - 1/2, z^2
-  V *z = nullptr;                  // [stride]
+  V *z = nullptr, *zl = nullptr;   // [stride]; FP32: z = z + zl
   int *js = nullptr;               // [lmax+1][stride] first j with |Q_j| >= 2^-100
   typename CkVec<V>::type *ck = nullptr;  // [block of 16 j of m][stride]
   typename CkVec<V>::type *seed = nullptr;  // [lmax+1][stride] (s_js, s_js+1)

@@ -125,3 +125,9 @@ def test_synthesis_f64(torch_cuda, osht, nside, lmax, np_):
 @pytest.mark.parametrize("nside,lmax", [(75, 150), (128, 256), (192, 384)])
 def test_synthesis_df64(torch_cuda, osht, nside, lmax):
     check_synthesis(torch_cuda, osht, "df64", nside, lmax)
+
+
+@pytest.mark.parametrize("nside,lmax", [(64, 128), (75, 150), (128, 256), (256, 512), (512, 1024)])
+@pytest.mark.parametrize("np_", [1, 2, 4])
+def test_synthesis_f32(torch_cuda, osht, nside, lmax, np_):
+    check_synthesis(torch_cuda, osht, "f32", nside, lmax, {"syn_np": [1, np_]})
