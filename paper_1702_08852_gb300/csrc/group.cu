@@ -120,7 +120,8 @@ __global__ void k_group_tables(const PairTab<double> t, int npairs, int lmax,
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   if (k >= npairs) return;
-  const int J = (lmax - m) / 2 + 1, js = t.js[(long)m * t.stride + k];
+  // the equatorial pairs start at lam_mm
+  const int J = (lmax - m) / 2 + 1, js = k < t.keq ? t.js[(long)m * t.stride + k] : 0;
   if (js >= J) return;
   const long q0 = pair_base(lmax, m);
   const double2 sd = t.seed[(long)m * t.stride + k];

@@ -33,13 +33,14 @@
 // lam_{m+2j}, so rounding in s_j is amplified by up to 1/z there (measured in
 // FP64 at Nside 1024: 1.1e-13 of the map's rms on the rings next to the equator,
 // 1.5e-15 with the one-step recurrence; in FP32 7e-5 at Nside 256 and 4e-4 at
-// Nside 1024, 4e-7 and 1e-6 with it).  The synthesis therefore gives the ring pairs k >= keq
-// (|z| < 1/6 and what makes whole warps, where lam_mm itself is the seed for every m:
-// equatorial_pair) to the one-step recurrence lam_l <- z lam_{l-1}, lam_{l-2}, two l per
-// j, at 8 multiply-adds instead of 6 (FP32: 10, z in two parts).  They get warps, and in
-// FP64 CTAs, of their own, so no number of pairs per thread and no Nside mixes the two
-// kinds.  The analysis, which sums over all rings, does not
-// need it (2.6e-14 of the rms against 3.0e-14 with the one-step recurrence).
+// Nside 1024, 4e-7 and 1e-6 with it).  The ring pairs k >= keq (|z| < 1/6 and what makes
+// whole warps, where lam_mm itself is the seed for every m: equatorial_pair) therefore
+// take the one-step recurrence lam_l <- z lam_{l-1}, lam_{l-2}, two l per j, at 8
+// multiply-adds instead of 6 (FP32: 10, z in two parts).  In the synthesis they get warps,
+// and in FP64 CTAs, of their own, so no number of pairs per thread and no Nside mixes the
+// two kinds.  In the analysis a block's sums over them are separate ones, of even and odd
+// l instead of E and O: a map that is zero but on nine rings around the equator comes out
+// to 1.6e-7 in FP32 at Nside 512 (1.3e-4 without it) and to 2e-14 in FP64 (1.9e-13).
 //
 // Bound: the FP64 unit, 2 multiply-adds per clock and SM.  At Nside 1024, lmax 2048
 // (3.14e9 terms) the synthesis takes 16.6 ms (21.4 ms with the one-step recurrence)
@@ -335,7 +336,7 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
       if (k < kend) {
         z[i] = t.z[k];
         if constexpr (std::is_same<V, float>::value) zl[i] = t.zl[k];
-        u[i] = t.lmm[(long)m * npairs + k];
+        u[i] = state_as<V>(t.ck_e[block_base(lmax, m) * t.estride + k - t.keq / 64 * 64]).x;
       }
     }
 #pragma unroll 4
@@ -460,6 +461,7 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
 //   a_{m+2j} = Omega (se_j De_j + sn_{j-1} De_{j-1}),  a_{m+2j+1} = Omega so_j Do_j,
 // with the solver's filter, source term and Cauchy sums fused.
 constexpr int PANA_TILE = 2048;
+constexpr int PAIR_SMEM = 220 * 1024;  // dynamic shared memory limit of these kernels
 constexpr int PANA_MAXWARPS = 8;
 constexpr int CKJ = 16;
 
@@ -467,33 +469,50 @@ constexpr int CKJ = 16;
 // FP32 the real and the imaginary sum of one parity are one packed accumulator.
 // INJ: a pair's seeds c may enter, at step `rel` and the next (else c is the state
 // before the block), and the pairs may differ in their form (table sr[i]).
-// SKIP: the sums start there (NJ of them).
-template <typename V, int R, bool INJ, int NJ, int SKIP>
+// NJ steps from step `skip` on (dd's second halves: the steps before it run in a loop, one
+// copy of the unrolled ones serves both halves -- with a copy for each, this kernel's
+// warps wait for instructions).
+template <typename V, int R, bool INJ, int NJ>
 __device__ __forceinline__ void pair_block(V (&v)[4 * NJ], const Pair<V> *const (&sr)[R],
                                            const V (&w)[R], const typename Cx<V>::type (&c)[R],
-                                           const Quad<V> (&p)[R], const int (&rel)[R]) {
+                                           const Quad<V> (&p)[R], const int (&rel)[R], int skip) {
   V s1[R], s2[R];
+  int at[R];  // the seeds' step, counted on from the current one
 #pragma unroll
   for (int i = 0; i < R; ++i) {
     const bool inj = INJ && (unsigned)rel[i] < (unsigned)CKJ;
     s1[i] = inj ? V(0) : c[i].x;
     s2[i] = inj ? V(0) : c[i].y;
+    at[i] = inj ? rel[i] : -100;
+  }
+  const Pair<V> *r0 = sr[0];
+  if constexpr (NJ < CKJ) {
+    static_assert(R == 1 && INJ, "halves: one pair per lane");
+#pragma unroll 4
+    for (int jj = 0; jj < skip; ++jj) {
+      const Pair<V> r = *r0++;
+      V s = fmav(coefv(r.a, w[0], r.b), s1[0], s2[0]);
+      s = at[0] == 0 ? c[0].x : s;
+      s = at[0] == -1 ? c[0].y : s;
+      s2[0] = s1[0];
+      s1[0] = s;
+      --at[0];
+    }
   }
 #pragma unroll
-  for (int jj = 0; jj < NJ + SKIP; ++jj) {
-    Pair<V> r = sr[0][jj];
+  for (int jj = 0; jj < NJ; ++jj) {
+    Pair<V> r = r0[jj];
 #pragma unroll
     for (int i = 0; i < R; ++i) {
       if (INJ && i > 0) r = sr[i][jj];
       V s = fmav(coefv(r.a, w[i], r.b), s1[i], s2[i]);
       if (INJ) {
-        s = jj == rel[i] ? c[i].x : s;
-        if (jj > 0) s = jj == rel[i] + 1 ? c[i].y : s;
+        s = jj == at[i] ? c[i].x : s;
+        if (jj > 0 || NJ < CKJ) s = jj == at[i] + 1 ? c[i].y : s;
       }
       s2[i] = s1[i];
       s1[i] = s;
-      if (jj < SKIP) continue;
-      V *x = v + 4 * (jj - SKIP);
+      V *x = v + 4 * jj;
       if constexpr (std::is_same<V, float>::value) {
         fma2(x[0], x[1], s, s, p[i].a, p[i].b, x[0], x[1]);
         fma2(x[2], x[3], s, s, p[i].c, p[i].d, x[2], x[3]);
@@ -503,6 +522,48 @@ __device__ __forceinline__ void pair_block(V (&v)[4 * NJ], const Pair<V> *const 
         accv(x[2], s, p[i].c);
         accv(x[3], s, p[i].d);
       }
+    }
+  }
+}
+
+// The same for equatorial pairs: c is (lam_{m+2j-2}, lam_{m+2j-1}), scaled and folded,
+// before the block; the sums are those of even and of odd l - m, from step `skip` on
+// (dd's second halves).  FP32 steps its two pairs packed.
+template <typename V, int R, int NJ>
+__device__ __forceinline__ void eq_block(V (&v)[4 * NJ], const Pair<V> *sr, const V (&z)[R],
+                                         const V (&zl)[R], const typename Cx<V>::type (&c)[R],
+                                         const Quad<V> (&p)[R], int skip) {
+  V u[R], o[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    u[i] = c[i].x;
+    o[i] = c[i].y;
+  }
+  auto next = [&](Pair<V> r) {
+    if constexpr (R == 2) {
+      eqv2(r.a, z[0], z[1], zl[0], zl[1], o[0], o[1], u[0], u[1]);
+      eqv2(r.b, z[0], z[1], zl[0], zl[1], u[0], u[1], o[0], o[1]);
+    } else {
+      u[0] = eqv(r.a, z[0], zl[0], o[0], u[0]);
+      o[0] = eqv(r.b, z[0], zl[0], u[0], o[0]);
+    }
+  };
+  if constexpr (NJ < CKJ) {
+#pragma unroll 1
+    for (int jj = 0; jj < skip; ++jj) next(sr[jj]);
+    sr += skip;
+  }
+#pragma unroll
+  for (int jj = 0; jj < NJ; ++jj) {
+    next(sr[jj]);
+    asm volatile("" ::: "memory");  // keeps later table loads, and their registers, below
+    V *x = v + 4 * jj;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      accv(x[0], u[i], p[i].a);
+      accv(x[1], u[i], p[i].b);
+      accv(x[2], o[i], p[i].c);
+      accv(x[3], o[i], p[i].d);
     }
   }
 }
@@ -623,13 +684,19 @@ __global__ void __launch_bounds__(32 * PANA_MAXWARPS, std::is_same<V, double>::v
                 double *__restrict__ partials, const double2 *__restrict__ src,
                 typename Cx<V>::type *__restrict__ xs, const float *__restrict__ cl32,
                 const double *__restrict__ se64, const double *__restrict__ sn64,
-                const double *__restrict__ so64, const SolverState *__restrict__ st, int mode, int lstatic) {
+                const double *__restrict__ so64, const double *__restrict__ ge64,
+                const double *__restrict__ go64, const SolverState *__restrict__ st, int mode,
+                int lstatic, int tile_max) {
   typedef typename Cx<V>::type C;
   typedef typename CkVec<V>::type Ck;
   constexpr int R = std::is_same<V, float>::value ? 2 : 1;  // pairs in flight per lane
   // where seeds may enter: FP32 the blocks in jin; dd the block of js, from the seed
   // table (the FP64 state before it may be below FP32's range); FP64 none
   constexpr bool DD = std::is_same<V, dd>::value, SEEDS = R == 2 || DD;
+  // FP32: one item does both kinds of pairs, its pair-basis sums brought to those of
+  // even and odd l before the equatorial ones are added, which saves a lane reduction
+  // (FP64 and dd: the arithmetic of that costs as much as the reduction)
+  constexpr bool ONE = R == 2;
   // j per warp item: dd halves a block (32 double-float sums leave room for 16 warps
   // per SM, 64 for 8: 1.01 ms at Nside 512), the second half repeating the first's
   // recurrence
@@ -653,86 +720,147 @@ __global__ void __launch_bounds__(32 * PANA_MAXWARPS, std::is_same<V, double>::v
   if (m <= L) {
     extern __shared__ __align__(16) unsigned char smraw[];
     const int J = (L - m) / 2 + 1, nb = (J + CKJ - 1) / CKJ, J16 = nb * CKJ;
-    const int tile = min((npairs + 63) / 64 * 64, PANA_TILE);
+    const int tile = min((npairs + 63) / 64 * 64, tile_max);
     Quad<V> *sp = reinterpret_cast<Quad<V> *>(smraw);                 // [tile]
     Quad<V> *sd = sp + tile;                                          // [J16]
-    Pair<V> *srec = reinterpret_cast<Pair<V> *>(sd + J16);            // [3][J16]
+    Quad<V> *se = sd + J16;  // [J16]: equatorial sums; ONE: the change of basis
+    Pair<V> *srec = reinterpret_cast<Pair<V> *>(se + J16);            // [4][J16]
+    Pair<V> *scar = srec + 4 * J16;  // ONE, [nb + 1]: even sum of the last j of a block
     const long q0 = pair_base(lmax, m), cb = block_base(lmax, m);
-    for (int j = tid; j < J16; j += blockDim.x) sd[j] = {V(0), V(0), V(0), V(0)};
-    for (int f = 0; f < 3; ++f)
+    for (int j = tid; j < J16; j += blockDim.x) {
+      sd[j] = se[j] = {V(0), V(0), V(0), V(0)};
+      if constexpr (ONE) {
+        if (j <= nb) scar[j] = {V(0), V(0)};
+        if (j < J) {
+          const V ge = V(1) / t.ge[q0 + j];
+          se[j] = {t.se[q0 + j] * ge, j % CKJ ? t.sn[q0 + j - 1] * ge : V(0),
+                   t.so[q0 + j] / t.go[q0 + j], V(0)};
+        }
+      }
+    }
+    for (int f = 0; f < 4; ++f) {
+      const Pair<V> *rec = reinterpret_cast<const Pair<V> *>(f < 3 ? t.rec[f] : t.rec_e);
       for (int j = tid; j < J16; j += blockDim.x) {
         const Pair<V> zero = {V(0), V(0)};
-        srec[f * J16 + j] = j < J ? reinterpret_cast<const Pair<V> *>(t.rec[f])[q0 + j] : zero;
+        srec[f * J16 + j] = j < J ? rec[q0 + j] : zero;
       }
-    for (int t0 = 0; t0 < npairs; t0 += PANA_TILE) {
-      const int nt = min(PANA_TILE, npairs - t0);
+    }
+    for (int t0 = 0; t0 < npairs; t0 += tile_max) {
+      const int nt = min(tile_max, npairs - t0);
       __syncthreads();  // the previous tile's reads are done
       for (int k = tid; k < (nt + 63) / 64 * 64; k += blockDim.x) {
         Quad<V> q = {V(0), V(0), V(0), V(0)};
         if (k < nt) q = reinterpret_cast<const Quad<V> *>(G)[(long)m * npairs + t0 + k];
         if (t0 + k == npairs - 1) q.c = q.d = V(0);  // the equator
-        const V z = t.z[t0 + k];
+        const V z = t0 + k < t.keq ? t.z[t0 + k] : V(1);
         sp[k] = {q.a + q.c, q.b + q.d, z * (q.a - q.c), z * (q.b - q.d)};
       }
       __syncthreads();
-      // js, the checkpoints and w are loaded one step (32 R pairs) ahead
+      // the tile's pairs below keq are nlow; a block's sums over those and over the
+      // equatorial ones are items of their own
+      const int nlow = max(0, min(nt, t.keq - t0));
+      const int items_low = nlow > 0 || ONE ? HALVES * nb : 0;
+      const int items = items_low + (nlow < nt && !ONE ? HALVES * nb : 0);
+      // js, the checkpoints, w and z are loaded one step (32 R pairs) ahead
       const int *jrow = (DD ? t.js : t.jin) + (long)m * t.stride + t0 + lane;
       const Ck *srow = t.seed + (long)m * t.stride + t0 + lane;
-      for (int bh = warp; bh < HALVES * nb; bh += nwarps) {
+      for (int item = warp; item < items; item += nwarps) {
+        const bool eq = item >= items_low;
+        const int bh = eq ? item - items_low : item;
         const int b = bh / HALVES, j0 = b * CKJ;
-        const Ck *crow = t.ck + (cb + b) * t.stride + t0 + lane;
-        int rel[R], form[R];
-        Ck c[R];
-        V w[R];
-        auto load = [&](int g) {
-#pragma unroll
-          for (int i = 0; i < R; ++i) {
-            form[i] = t.form(t0 + g + 32 * i);
-            rel[i] = SEEDS ? jrow[g + 32 * i] - j0 : -1;
-            c[i] = crow[g + 32 * i];
-            if constexpr (DD) {
-              const Ck sd0 = srow[g + 32 * i];
-              if ((unsigned)rel[i] < (unsigned)CKJ) c[i] = sd0;
-            }
-            w[i] = t.w[form[i] * t.stride + t0 + lane + g + 32 * i];
-          }
-        };
         V v[4 * NJ];
 #pragma unroll
         for (int i = 0; i < 4 * NJ; ++i) v[i] = V(0);
-        // below its first warp of pairs a block is zero
-        int g = max(0, t.gfirst[cb + b] - t0) / (32 * R) * (32 * R);
-        if (g < nt) load(g);
-        for (; g < nt; g += 32 * R) {
-          const Pair<V> *sr[R];
-          V wc[R];
-          C d[R];
-          Quad<V> p[R];
-          int rl[R];
-          bool slow = R == 2 && form[0] != form[R - 1];
+        if (ONE || !eq) {
+          const Ck *crow = t.ck + (cb + b) * t.cstride + t0 + lane;
+          int rel[R], form[R];
+          Ck c[R];
+          V w[R];
+          auto load = [&](int g) {
 #pragma unroll
-          for (int i = 0; i < R; ++i) {
-            sr[i] = srec + form[i] * J16 + j0;
-            wc[i] = w[i];
-            d[i] = state_as<V>(c[i]);
-            rl[i] = rel[i];
-            p[i] = sp[g + 32 * i + lane];
-            slow |= (unsigned)rel[i] < (unsigned)CKJ;
-          }
-          if (g + 32 * R < nt) load(g + 32 * R);
-          if constexpr (DD) {
-            if (bh & 1)
-              pair_block<V, R, true, NJ, NJ>(v, sr, wc, d, p, rl);
-            else
-              pair_block<V, R, true, NJ, 0>(v, sr, wc, d, p, rl);
-          } else {
-            if (R == 2 && __any_sync(0xffffffffu, slow))
-              pair_block<V, R, true, NJ, 0>(v, sr, wc, d, p, rl);
-            else
-              pair_block<V, R, false, NJ, 0>(v, sr, wc, d, p, rl);
+            for (int i = 0; i < R; ++i) {
+              const int k = g + 32 * i;
+              form[i] = t.form(t0 + k);
+              rel[i] = SEEDS ? jrow[k] - j0 : -1;
+              c[i] = crow[k];
+              if constexpr (DD) {
+                const Ck sd0 = srow[k];
+                if ((unsigned)rel[i] < (unsigned)CKJ) c[i] = sd0;
+              }
+              w[i] = t.w[form[i] * t.stride + t0 + lane + k];
+            }
+          };
+          // below its first warp of pairs a block is zero
+          int g = max(0, t.gfirst[cb + b] - t0) / (32 * R) * (32 * R);
+          if (g < nlow) load(g);
+          for (; g < nlow; g += 32 * R) {
+            const Pair<V> *sr[R];
+            V wc[R];
+            C d[R];
+            Quad<V> p[R];
+            int rl[R];
+            bool slow = R == 2 && form[0] != form[R - 1];
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+              sr[i] = srec + form[i] * J16 + j0;
+              wc[i] = w[i];
+              d[i] = state_as<V>(c[i]);
+              rl[i] = rel[i];
+              p[i] = sp[g + 32 * i + lane];
+              slow |= (unsigned)rel[i] < (unsigned)CKJ;
+            }
+            if (g + 32 * R < nlow) load(g + 32 * R);
+            if (DD || (R == 2 && __any_sync(0xffffffffu, slow)))
+              pair_block<V, R, SEEDS, NJ>(v, sr, wc, d, p, rl, DD ? (bh & 1) * NJ : 0);
+            else if constexpr (!DD)
+              pair_block<V, R, false, NJ>(v, sr, wc, d, p, rl, 0);
           }
         }
-        V *out = reinterpret_cast<V *>(sd) + 4 * (j0 + (bh % HALVES) * NJ) + lane;
+        if constexpr (ONE) {
+          // even: De_j and De_{j-1} make up l = m + 2 j; the block's last De_j also
+          // belongs to the first l of the next block
+          if (nlow > 0) {
+            V ca = v[4 * NJ - 4], cc = v[4 * NJ - 3];
+            for (int o = 16; o > 0; o >>= 1) {
+              ca = ca + shfx(ca, o);
+              cc = cc + shfx(cc, o);
+            }
+            if (lane == 0) scar[b + 1] = {scar[b + 1].a + ca, scar[b + 1].b + cc};
+#pragma unroll
+            for (int jj = NJ - 1; jj >= 0; --jj) {
+              const Quad<V> f = se[j0 + jj];
+              V *x = v + 4 * jj;
+              x[0] = f.a * x[0];
+              x[1] = f.a * x[1];
+              if (jj > 0) {
+                x[0] = fmav(f.b, x[-4], x[0]);
+                x[1] = fmav(f.b, x[-3], x[1]);
+              }
+              x[2] = f.c * x[2];
+              x[3] = f.c * x[3];
+            }
+          }
+        }
+        if (ONE || eq) {
+          // the rows start at a multiple of 64, zero below keq
+          const Ck *crow = t.ck_e + (cb + b) * t.estride + (t0 - t.keq / 64 * 64) + lane;
+          for (int g = nlow / (32 * R) * (32 * R); g < nt; g += 32 * R) {
+            V z[R], zl[R];
+            C c[R];
+            Quad<V> p[R];
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+              const int k = g + 32 * i;
+              c[i] = state_as<V>(crow[k]);
+              z[i] = t.z[t0 + lane + k];
+              zl[i] = V(0);
+              if constexpr (std::is_same<V, float>::value) zl[i] = t.zl[t0 + lane + k];
+              p[i] = sp[k + lane];
+            }
+            eq_block<V, R, NJ>(v, srec + 3 * J16 + j0, z, zl, c, p, DD ? (bh & 1) * NJ : 0);
+          }
+        }
+        V *out = reinterpret_cast<V *>(eq ? se : sd) + 4 * (j0 + (bh % HALVES) * NJ) + lane;
         const V lo = lane_sums(v, lane);
         out[0] = out[0] + lo;
         if constexpr (!DD) {
@@ -748,14 +876,26 @@ __global__ void __launch_bounds__(32 * PANA_MAXWARPS, std::is_same<V, double>::v
       typedef typename std::conditional<DD, double, V>::type E;
       const E *fo = epi<E>(t.so, so64), *fe = epi<E>(t.se, se64), *fn = epi<E>(t.sn, sn64);
       E sr, si;
-      if (i & 1) {
-        const E f = fo[q0 + j];
-        sr = f * epi_val<E>(sd[j].c);
-        si = f * epi_val<E>(sd[j].d);
+      if constexpr (ONE) {
+        const E g = (i & 1 ? t.go : t.ge)[q0 + j];
+        const Quad<V> q = sd[j];
+        sr = g * (i & 1 ? q.c : q.a);
+        si = g * (i & 1 ? q.d : q.b);
+        if (j > 0 && i % (2 * CKJ) == 0) {
+          const Pair<V> c = scar[j / CKJ];
+          sr = fmav(t.sn[q0 + j - 1], c.a, sr);
+          si = fmav(t.sn[q0 + j - 1], c.b, si);
+        }
+      } else if (i & 1) {
+        const Quad<V> qe = se[j];
+        const E f = fo[q0 + j], g = epi<E>(t.go, go64)[q0 + j];
+        sr = fmav(g, epi_val<E>(qe.c), f * epi_val<E>(sd[j].c));
+        si = fmav(g, epi_val<E>(qe.d), f * epi_val<E>(sd[j].d));
       } else {
-        const E f = fe[q0 + j];
-        sr = f * epi_val<E>(sd[j].a);
-        si = f * epi_val<E>(sd[j].b);
+        const Quad<V> qe = se[j];
+        const E f = fe[q0 + j], ge = epi<E>(t.ge, ge64)[q0 + j];
+        sr = fmav(ge, epi_val<E>(qe.a), f * epi_val<E>(sd[j].a));
+        si = fmav(ge, epi_val<E>(qe.b), f * epi_val<E>(sd[j].b));
         if (j > 0) {
           const E g = fn[q0 + j - 1];
           sr = fmav(g, epi_val<E>(sd[j - 1].a), sr);
@@ -810,9 +950,19 @@ struct SynthGrid {
     smem = mix ? eq_ofs + eq : low;
   }
 };
-static size_t anal_smem(size_t v, int npairs, int lmax) {
+static size_t anal_smem(size_t v, int npairs, int lmax, int tile) {
   const size_t j16 = (size_t)(lmax / 32 + 1) * CKJ;
-  return 4 * v * std::min((npairs + 63) / 64 * 64, PANA_TILE) + 10 * v * j16;
+  return 4 * v * std::min((npairs + 63) / 64 * 64, tile) + 16 * v * j16 +
+         2 * v * (j16 / CKJ + 1);
+}
+// half a tile where a whole one leaves too little shared memory (FP64 above lmax ~ 2500)
+static int anal_tile(size_t v, int npairs, int lmax) {
+  return anal_smem(v, npairs, lmax, PANA_TILE) <= PAIR_SMEM ? PANA_TILE : PANA_TILE / 2;
+}
+// a warp per item of the CTA of m = 0 (FP64, dd: twice its blocks)
+static int anal_threads(size_t v, int lmax) {
+  const int nb = lmax / 32 + 1;
+  return 32 * std::max(2, std::min(PANA_MAXWARPS, v == 4 ? nb : 2 * nb));
 }
 
 template <int NP>
@@ -844,10 +994,11 @@ wf_status launch_legendre_anal<double2>(const Plan &P, const double2 *G, double2
                                         const SolverState *st, int mode, int lstatic,
                                         const double2 *src, double2 *) {
   ++P.nlaunch;
-  const int warps = std::max(2, std::min(PANA_MAXWARPS, P.lmax / 32 + 1));
-  k_pair_anal<double><<<P.lmax + 1, 32 * warps, anal_smem(8, P.npairs, P.lmax), P.stream>>>(
+  const int tile = anal_tile(8, P.npairs, P.lmax);
+  k_pair_anal<double><<<P.lmax + 1, anal_threads(8, P.lmax), anal_smem(8, P.npairs, P.lmax, tile),
+                     P.stream>>>(
       P.pt64, P.npairs, P.lmax, P.cl_d, P.omega, G, x, P.partials, src, nullptr, nullptr,
-      nullptr, nullptr, nullptr, st, mode, lstatic);
+      nullptr, nullptr, nullptr, nullptr, nullptr, st, mode, lstatic, tile);
   WF_CUDA(cudaGetLastError());
   return WF_OK;
 }
@@ -880,10 +1031,11 @@ wf_status launch_legendre_anal<float2>(const Plan &P, const float2 *G, double2 *
                                        const SolverState *st, int mode, int lstatic,
                                        const double2 *src, float2 *xs_out) {
   ++P.nlaunch;
-  const int warps = std::max(2, std::min(PANA_MAXWARPS, P.lmax / 32 + 1));
-  k_pair_anal<float><<<P.lmax + 1, 32 * warps, anal_smem(4, P.npairs, P.lmax), P.stream>>>(
+  const int tile = anal_tile(4, P.npairs, P.lmax);
+  k_pair_anal<float><<<P.lmax + 1, anal_threads(4, P.lmax), anal_smem(4, P.npairs, P.lmax, tile),
+                     P.stream>>>(
       P.pt32, P.npairs, P.lmax, P.cl_d, P.omega, G, x, P.partials, src, xs_out, P.cl32, nullptr,
-      nullptr, nullptr, st, mode, lstatic);
+      nullptr, nullptr, nullptr, nullptr, st, mode, lstatic, tile);
   WF_CUDA(cudaGetLastError());
   return WF_OK;
 }
@@ -914,10 +1066,12 @@ wf_status launch_legendre_anal_dd(const Plan &P, const float4 *G, double2 *x,
                                   const double2 *src) {
   ++P.nlaunch;
   typedef Cx<dd>::type C;
-  const int warps = std::max(2, std::min(PANA_MAXWARPS, P.lmax / 32 + 1));
-  k_pair_anal<dd><<<P.lmax + 1, 32 * warps, anal_smem(8, P.npairs, P.lmax), P.stream>>>(
+  const int tile = anal_tile(8, P.npairs, P.lmax);
+  k_pair_anal<dd><<<P.lmax + 1, anal_threads(8, P.lmax), anal_smem(8, P.npairs, P.lmax, tile),
+                     P.stream>>>(
       P.ptdd, P.npairs, P.lmax, P.cl_d, P.omega, reinterpret_cast<const C *>(G), x, P.partials,
-      src, nullptr, nullptr, P.pt64.se, P.pt64.sn, P.pt64.so, st, mode, lstatic);
+      src, nullptr, nullptr, P.pt64.se, P.pt64.sn, P.pt64.so, P.pt64.ge, P.pt64.go, st, mode,
+      lstatic, tile);
   WF_CUDA(cudaGetLastError());
   return WF_OK;
 }
@@ -955,7 +1109,7 @@ wf_status launch_prescale_dd(const Plan &P, const double2 *x, float4 *xs) {
 }
 
 wf_status init_pair_attributes() {
-  const int big = 220 * 1024;
+  const int big = PAIR_SMEM;
   WF_CUDA(cudaFuncSetAttribute(k_pair_synth<double, 1>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   WF_CUDA(cudaFuncSetAttribute(k_pair_synth<double, 2>,
@@ -991,13 +1145,18 @@ __global__ void k_pair_walk(int npairs, int lmax, const PairTab<double> t_,
   const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long)npairs * (lmax + 1)) return;
   const int m = (int)(t / npairs), k = (int)(t % npairs);
-  const int J = (lmax - m) / 2 + 1, stride = t_.stride;
-  const long q0 = pair_base(lmax, m), cb = block_base(lmax, m), mk = (long)m * stride + k;
+  const int J = (lmax - m) / 2 + 1, stride = t_.cstride;
+  const long q0 = pair_base(lmax, m), cb = block_base(lmax, m), mk = (long)m * t_.stride + k;
   const int form = t_.form(k);
   const double2 *rec = t_.rec[form] + q0;
-  const double w = t_.w[form * stride + k];
+  const double w = t_.w[form * t_.stride + k];
   double v = mant[t] * sqrt(2.0 * m + 3.0), vp = 0.0;  // Q_0 = lam_mm / eps_{m+1}
   int e = expo[t], j = 0;                              // value v 2^e
+  if (k >= t_.keq) {  // the grouped tables' start; nothing else reads them
+    v = ldexp(v, e);
+    t_.seed[mk] = make_double2(v, J > 1 ? fma(rec[1].x, w, rec[1].y) * v : 0.0);
+    return;
+  }
   // the state before the block of j: rec[0] = (0, 0), so (0, s_0) yields s_0 at j = 0
   double b1 = 0.0, b2 = v;
   int be = e;
@@ -1058,6 +1217,32 @@ __global__ void k_pair_walk(int npairs, int lmax, const PairTab<double> t_,
     const double s = fma(fma(r.x, w, r.y), s1, s2);
     s2 = s1;
     s1 = s;
+  }
+}
+
+// The equatorial pairs' checkpoints: the one-step recurrence from lam_mm, (even, odd)
+// before each block.
+__global__ void k_eq_walk(int npairs, int lmax, const PairTab<double> t_, const PairTab<float> u,
+                          const double *__restrict__ mant, const int *__restrict__ expo) {
+  const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int n = npairs - t_.keq;
+  if (t >= (long)n * (lmax + 1)) return;
+  const int m = (int)(t / n), k = t_.keq + (int)(t % n);
+  const int J = (lmax - m) / 2 + 1;
+  const double2 *rec = t_.rec_e + pair_base(lmax, m);
+  const double z = t_.z[k];
+  const long i = (long)m * npairs + k;
+  long at = block_base(lmax, m) * t_.estride + k - t_.keq / 64 * 64;
+  double even = ldexp(mant[i], expo[i]), odd = 0.0;  // rec[0].x = 0 leaves lam_mm
+  for (int j = 0; j < J; ++j) {
+    if ((j & 15) == 0) {
+      t_.ck_e[at] = make_double2(even, odd);
+      u.ck_e[at] = make_float2((float)even, (float)odd);
+      at += t_.estride;
+    }
+    const double2 r = rec[j];
+    even = fma(r.x * z, odd, even);
+    odd = fma(r.y * z, even, odd);
   }
 }
 
@@ -1151,16 +1336,6 @@ __global__ void k_pair_coefs(int lmax, PairTab<double> t) {
   }
 }
 
-// lam_mm of the pairs from keq on (mantissa and exponent 0 there)
-__global__ void k_pair_lmm(int npairs, int lmax, int keq, const double *__restrict__ mant,
-                           const int *__restrict__ expo, double *__restrict__ lmm) {
-  const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int n = npairs - keq;
-  if (t >= (long)n * (lmax + 1)) return;
-  const long i = t / n * npairs + keq + t % n;
-  lmm[i] = ldexp(mant[i], expo[i]);
-}
-
 static wf_status build_pair_tables32(Plan &P, long nq);
 static wf_status build_pair_tables_dd(Plan &P, long nq);
 
@@ -1208,6 +1383,8 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
   PairTab<double> &t = P.pt64;
   for (int f = 0; f < 2; ++f) t.kform[f] = (kform[f] + 16) / 32 * 32;
   t.keq = keq;
+  t.cstride = (keq + 63) / 64 * 64;
+  t.estride = stride - keq / 64 * 64;
   t.stride = stride;
   WF_TRY(up(&t.w, w));
   WF_TRY(up(&t.z, z));
@@ -1218,29 +1395,27 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
     WF_CUDA(cudaMalloc(a, sizeof(double) * nq));
   k_pair_coefs<<<(lmax + 32) / 32, 32, 0, P.stream>>>(lmax, t);
   WF_CUDA(cudaGetLastError());
-  if (keq < P.npairs) {
-    const long ne = (long)(P.npairs - keq) * (lmax + 1);
-    WF_CUDA(cudaMalloc(&t.lmm, sizeof(double) * (size_t)P.npairs * (lmax + 1)));
-    k_pair_lmm<<<(unsigned)((ne + 255) / 256), 256, 0, P.stream>>>(P.npairs, lmax, keq, mant,
-                                                                   expo, t.lmm);
-    WF_CUDA(cudaGetLastError());
-  }
   WF_TRY(build_pair_tables32(P, nq));
   PairTab<float> &u = P.pt32;
   // no seed: js and jin beyond every block; no checkpoint: zero (also the rows'
   // padding)
-  const size_t mk = (size_t)stride * (lmax + 1), ck = (size_t)nb * stride;
+  const size_t mk = (size_t)stride * (lmax + 1), ck = (size_t)nb * std::max(t.cstride, 1),
+               ce = (size_t)nb * t.estride;
   WF_CUDA(cudaMalloc(&t.js, sizeof(int) * mk));
   WF_CUDA(cudaMalloc(&u.jin, sizeof(int) * mk));
   WF_CUDA(cudaMalloc(&t.seed, sizeof(double2) * mk));
   WF_CUDA(cudaMalloc(&u.seed, sizeof(float2) * mk));
   WF_CUDA(cudaMalloc(&t.ck, sizeof(double2) * ck));
   WF_CUDA(cudaMalloc(&u.ck, sizeof(float2) * ck));
+  WF_CUDA(cudaMalloc(&t.ck_e, sizeof(double2) * ce));
+  WF_CUDA(cudaMalloc(&u.ck_e, sizeof(float2) * ce));
   WF_CUDA(cudaMalloc(&t.gfirst, sizeof(int) * nb));
   WF_CUDA(cudaMemsetAsync(t.js, 0x3f, sizeof(int) * mk, P.stream));
   WF_CUDA(cudaMemsetAsync(u.jin, 0x3f, sizeof(int) * mk, P.stream));
   WF_CUDA(cudaMemsetAsync(t.ck, 0, sizeof(double2) * ck, P.stream));
   WF_CUDA(cudaMemsetAsync(u.ck, 0, sizeof(float2) * ck, P.stream));
+  WF_CUDA(cudaMemsetAsync(t.ck_e, 0, sizeof(double2) * ce, P.stream));
+  WF_CUDA(cudaMemsetAsync(u.ck_e, 0, sizeof(float2) * ce, P.stream));
   WF_CUDA(cudaMemsetAsync(t.gfirst, 0x7f, sizeof(int) * nb, P.stream));  // none
   u.js = t.js;
   u.gfirst = t.gfirst;
@@ -1248,6 +1423,11 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
   k_pair_walk<<<(unsigned)((n + 127) / 128), 128, 0, P.stream>>>(P.npairs, lmax, t, u, mant,
                                                                  expo);
   WF_CUDA(cudaGetLastError());
+  if (keq < P.npairs) {
+    const long ne = (long)(P.npairs - keq) * (lmax + 1);
+    k_eq_walk<<<(unsigned)((ne + 127) / 128), 128, 0, P.stream>>>(P.npairs, lmax, t, u, mant, expo);
+    WF_CUDA(cudaGetLastError());
+  }
   return build_pair_tables_dd(P, nq);
 }
 
@@ -1278,10 +1458,11 @@ static wf_status build_pair_tables32(Plan &P, long nq) {
   WF_TRY(round(&u.rec_e, t.rec_e, 2 * nq));
   WF_TRY(round(&u.ge, t.ge, nq));
   WF_TRY(round(&u.go, t.go, nq));
-  if (t.lmm) WF_TRY(round(&u.lmm, t.lmm, (long)P.npairs * (P.lmax + 1)));
   u.stride = t.stride;
   for (int f = 0; f < 2; ++f) u.kform[f] = t.kform[f];
   u.keq = t.keq;
+  u.cstride = t.cstride;
+  u.estride = t.estride;
   return WF_OK;
 }
 
@@ -1312,31 +1493,32 @@ static wf_status build_pair_tables_dd(Plan &P, long nq) {
   WF_TRY(split(&u.go, t.go, nq));
   WF_TRY(split(&u.w, t.w, 3L * t.stride));
   WF_TRY(split(&u.z, t.z, t.stride));
-  if (t.lmm) WF_TRY(split(&u.lmm, t.lmm, (long)P.npairs * (P.lmax + 1)));
   u.stride = t.stride;
   u.js = t.js;
   u.seed = t.seed;
   u.ck = t.ck;
+  u.ck_e = t.ck_e;
   u.gfirst = t.gfirst;
   u.keq = t.keq;
+  u.cstride = t.cstride;
+  u.estride = t.estride;
   for (int f = 0; f < 2; ++f) u.kform[f] = t.kform[f];
   return WF_OK;
 }
 
 void free_pair_tables(Plan &P) {
   PairTab<dd> &d = P.ptdd;
-  void *g[] = {d.rec[0], d.rec[1], d.rec[2], d.rec_e, d.se, d.sn, d.so, d.ge, d.go, d.w, d.z,
-               d.lmm};
+  void *g[] = {d.rec[0], d.rec[1], d.rec[2], d.rec_e, d.se, d.sn, d.so, d.ge, d.go, d.w, d.z};
   for (void *p : g)
     if (p) cudaFree(p);
   PairTab<float> &u = P.pt32;
   void *f[] = {u.rec[0], u.rec[1], u.rec[2], u.se, u.sn, u.so, u.w, u.z, u.ck, u.jin, u.seed,
-               u.rec_e, u.ge, u.go, u.zl, u.lmm};
+               u.rec_e, u.ge, u.go, u.zl, u.ck_e};
   for (void *p : f)
     if (p) cudaFree(p);
   PairTab<double> &t = P.pt64;
   void *b[] = {t.rec[0], t.rec[1], t.rec[2], t.rec_e, t.se, t.sn, t.so, t.ge, t.go, t.w, t.z,
-               t.lmm, t.js, t.seed, t.ck, t.gfirst};
+               t.js, t.seed, t.ck, t.ck_e, t.gfirst};
   for (void *p : b)
     if (p) cudaFree(p);
 }

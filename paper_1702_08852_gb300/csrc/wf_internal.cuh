@@ -55,18 +55,20 @@ struct PairTab {
   int stride = 0;                  // row length: npairs rounded up to 64
   V *w = nullptr;                  // [3][stride]: z^2 - 1, z^2 - 1/2, z^2
   V *z = nullptr, *zl = nullptr;   // [stride]; FP32: z = z + zl
-  int *js = nullptr;               // [lmax+1][stride] first j with |Q_j| >= 2^-100
-  typename CkVec<V>::type *ck = nullptr;  // [block of 16 j of m][stride]
+  int *js = nullptr;               // [lmax+1][stride] first j with |Q_j| >= 2^-100, k < keq
+  typename CkVec<V>::type *ck = nullptr;  // [block of 16 j of m][cstride]: k < keq
+  int cstride = 0, estride = 0;    // keq rounded up to 64; stride less keq rounded down
   typename CkVec<V>::type *seed = nullptr;  // [lmax+1][stride] (s_js, s_js+1)
   int *jin = nullptr;              // [lmax+1][stride] FP32: j where ck holds the seeds
   int *gfirst = nullptr;           // [block]: first warp of pairs with a term in it
   int kform[2] = {0, 0};           // pairs below kform[f]: form f (multiples of 32)
   __host__ __device__ int form(int k) const { return k < kform[0] ? 0 : k < kform[1] ? 1 : 2; }
-  // the pairs k >= keq in the synthesis: the one-step recurrence's coefficients
-  // (l - m even, odd), its scales, and lam_mm [lmax+1][npairs]
+  // the pairs k >= keq: the one-step recurrence's coefficients (l - m even, odd), its
+  // scales and its checkpoints, (even, odd) before the block, lam_mm before the first
   int keq = 0;
   typename PairVec<V>::type *rec_e = nullptr;
-  V *ge = nullptr, *go = nullptr, *lmm = nullptr;
+  V *ge = nullptr, *go = nullptr;
+  typename CkVec<V>::type *ck_e = nullptr;  // [block][estride], from keq / 64 * 64 on
 };
 
 // j of one m: J = (L - m) / 2 + 1; the first (m, j) table entry of m is the sum of J

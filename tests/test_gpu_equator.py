@@ -131,3 +131,43 @@ def test_synthesis_df64(torch_cuda, osht, nside, lmax):
 @pytest.mark.parametrize("np_", [1, 2, 4])
 def test_synthesis_f32(torch_cuda, osht, nside, lmax, np_):
     check_synthesis(torch_cuda, osht, "f32", nside, lmax, {"syn_np": [1, np_]})
+
+
+def strip(nside, seed):
+    """A map that is zero but on the equator and the four rings on each side of it."""
+    m = np.zeros(12 * nside * nside)
+    a, b = ring(nside, 2 * nside - 4)[0], ring(nside, 2 * nside + 5)[0]
+    m[a:b] = np.random.default_rng(seed).standard_normal(b - a)
+    return m
+
+
+def analyse_strip(osht, m, nside, lmax):
+    from paper_1702_08852_gb300 import inputs
+    out = np.zeros(inputs.nalm(lmax), np.clongdouble)
+    n = 4 * nside
+    for i in range(2 * nside - 4, 2 * nside + 1):
+        g = []
+        for j in sorted({i, 4 * nside - i}):
+            first, num = ring(nside, j)
+            x = np.fft.fft(m[first:first + n])
+            g.append(x[np.arange(lmax + 1) % n] * phase(nside, lmax, num).conj())
+        for l, lam in walk(osht, nside, lmax, i):
+            s = 1 - 2 * ((np.arange(l + 1) + l) & 1)
+            v = g[0][:l + 1] + (s * g[1][:l + 1] if len(g) > 1 else 0)
+            out[slots(lmax, l)] += lam * v
+    return (4 * np.pi / m.size * out).astype(np.complex128)
+
+
+# (64, 128) .. (256, 512): whole warps of equatorial pairs; 75: a part of one; 16: a
+# few pairs; 4: every pair
+@pytest.mark.parametrize("nside,lmax", [(4, 9), (16, 33), (64, 128), (75, 150), (256, 512)])
+@pytest.mark.parametrize("prec", ["f64", "f32", "df64"])
+def test_analysis(torch_cuda, osht, prec, nside, lmax):
+    torch = torch_cuda
+    from paper_1702_08852_gb300 import wf
+    m = strip(nside, nside + lmax)
+    with wf.Plan(nside, lmax, np.ones(lmax + 1)) as p:
+        f = {"f64": p.map2alm, "f32": p.map2alm_f32, "df64": p.map2alm_df64}[prec]
+        got = f(torch.from_numpy(m).cuda()).cpu().numpy()
+    ref = analyse_strip(osht, m, nside, lmax)
+    assert np.linalg.norm(got - ref) <= tol(prec, lmax) * np.linalg.norm(ref)
