@@ -21,8 +21,7 @@
 // three equal forms, w0 = 1, 1/2 and 0, for the pairs below kform[0] (near the
 // pole, where -sin^2 theta keeps the small angle that z^2 rounds away), below
 // kform[1], and the others.  Each keeps |B| at or below the size of the sum, so
-// that rounding B does not add to the phase; a CTA or warp takes the form of the
-// pairs it holds.
+// that rounding B does not add to the phase; 32 pairs take the form of their middle one.
 //
 // Per (m, ring pair) and j this costs 2 multiply-adds for the recurrence and 4
 // for the two complex sums, 3 per (l, m, pair) term; the one-step recurrence in
@@ -239,6 +238,10 @@ __device__ __forceinline__ V lane_sums(V *v, int lane) {
 constexpr int PSYN_THREADS = 64;     // FP64
 constexpr int PSYN_THREADS32 = 128;  // FP32
 
+template <typename V>
+__host__ __device__ constexpr int synth_forms(int np) {  // forms staged by a CTA
+  return std::is_same<V, float>::value || (std::is_same<V, double>::value && np > 1) ? 3 : 1;
+}
 template <typename V, int NP>
 __global__ void __launch_bounds__(PSYN_THREADS32)
     k_pair_synth(const PairTab<V> t, int npairs, int lmax,
@@ -272,20 +275,22 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
   const int pair0 = equator ? t.keq + (warp0 + warp - nlow) * 32 * NE
                             : (warp0 + warp) * 32 * NP;
   const int kend = equator ? npairs : t.keq;
-  // FP32 CTAs span several forms: all three are staged and each warp takes its own;
-  // FP64 CTAs (at most 64 pairs) stage one
-  constexpr int NF = std::is_same<V, float>::value ? 3 : 1;
-  const int form = t.form(NF == 1 ? warp0 * 32 * NP + (int)blockDim.x / 2 - 1 : pair0 + 16 * NP - 1);
-  const V *wt = t.w + form * t.stride;
+  // where a CTA spans several forms all three are staged and every 32 pairs take their
+  // own (one form of the CTA's or the warp's for all of them: FP64 with four pairs per
+  // thread, Nside 512, 2.8e-14 of the rms at z = 2/3 instead of 3e-15).  FP64 CTAs with a
+  // pair per thread hold 64 pairs, double-float ones 64, or 128 of 1024 and more: one
+  constexpr int NF = synth_forms<V>(NP);
+  int form[NP];
   V w[NP];
   int js[NP];
 #pragma unroll
   for (int i = 0; i < NP; ++i) {  // in flight while the coefficients are staged
     const int k = pair0 + lane + 32 * i;
+    form[i] = t.form(NF == 1 ? warp0 * 32 * NP + (int)blockDim.x * NP / 2 - 1 : pair0 + 32 * i + 15);
     w[i] = V(0);
     js[i] = INT_MAX / 2;
     if (!equator && k < kend) {
-      w[i] = wt[k];
+      w[i] = t.w[form[i] * t.stride + k];
       js[i] = t.js[(long)m * t.stride + k];
     }
   }
@@ -314,7 +319,7 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
         const V se = t.se[q0 + j], sn = t.sn[q0 + j], so = t.so[q0 + j];
         put(sx, j, fmav(se, c0.x, sn * c2.x), fmav(se, c0.y, sn * c2.y), so * c1.x, so * c1.y);
         if constexpr (NF == 1) {
-          srec[j] = reinterpret_cast<const Pair<V> *>(t.rec[form])[q0 + j];
+          srec[j] = reinterpret_cast<const Pair<V> *>(t.rec[form[0]])[q0 + j];
         } else {
 #pragma unroll
           for (int f = 0; f < NF; ++f)
@@ -374,7 +379,13 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
     return;
   }
 
-  const Pair<V> *sr = srec + (NF == 1 ? 0 : form * J);
+  const Pair<V> *sr[NP];
+  bool mixed = false;
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    sr[i] = srec + (NF == 1 ? 0 : form[i] * J);
+    mixed |= NF > 1 && form[i] != form[0];
+  }
   V s1[NP], s2[NP], d0[NP], d1[NP], er[NP], ei[NP], orr[NP], oi[NP];
   int jmin = INT_MAX, jinj = -1;
 #pragma unroll
@@ -391,57 +402,63 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
   }
   jmin = wmin(jmin);
   jinj = min(wmax(jinj), J - 1);
-  int j = jmin;
-  if constexpr (PK) {
-    auto step = [&](int jj, bool inj) {
-      const Pair<V> r = sr[jj];
+  // INJ: seeds may still enter; MIXED: the pairs' forms differ
+  auto step = [&](int jj, auto INJ, auto MIXED) {
+    Pair<V> r[NP];
+    r[0] = sr[0][jj];
+#pragma unroll
+    for (int i = 1; i < NP; ++i) r[i] = MIXED ? sr[i][jj] : r[0];
+    V s[NP];
+#pragma unroll
+    for (int i = 0; i < NP; i += PK ? 2 : 1) {
+      if constexpr (PK) {
+        V c0, c1;
+        fma2(c0, c1, r[i].a, r[i + 1].a, w[i], w[i + 1], r[i].b, r[i + 1].b);
+        fma2(s[i], s[i + 1], c0, c1, s1[i], s1[i + 1], s2[i], s2[i + 1]);
+      } else {
+        s[i] = fmav(coefv(r[i].a, w[i], r[i].b), s1[i], s2[i]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      if (INJ) {
+        s[i] = jj == js[i] ? d0[i] : s[i];
+        s[i] = jj == js[i] + 1 ? d1[i] : s[i];
+      }
+      s2[i] = s1[i];
+      s1[i] = s[i];
+    }
+    if constexpr (PK) {
       const Quad<V> xe = sx[2 * jj], xo = sx[2 * jj + 1];
 #pragma unroll
       for (int i = 0; i < NP; i += 2) {
-        V c0, c1, a0, a1;
-        fma2(c0, c1, r.a, r.a, w[i], w[i + 1], r.b, r.b);
-        fma2(a0, a1, c0, c1, s1[i], s1[i + 1], s2[i], s2[i + 1]);
-        if (inj) {
-          a0 = jj == js[i] ? d0[i] : a0;
-          a0 = jj == js[i] + 1 ? d1[i] : a0;
-          a1 = jj == js[i + 1] ? d0[i + 1] : a1;
-          a1 = jj == js[i + 1] + 1 ? d1[i + 1] : a1;
-        }
-        s2[i] = s1[i];
-        s2[i + 1] = s1[i + 1];
-        s1[i] = a0;
-        s1[i + 1] = a1;
-        fma2(er[i], er[i + 1], a0, a1, xe.a, xe.b, er[i], er[i + 1]);
-        fma2(ei[i], ei[i + 1], a0, a1, xe.c, xe.d, ei[i], ei[i + 1]);
-        fma2(orr[i], orr[i + 1], a0, a1, xo.a, xo.b, orr[i], orr[i + 1]);
-        fma2(oi[i], oi[i + 1], a0, a1, xo.c, xo.d, oi[i], oi[i + 1]);
+        fma2(er[i], er[i + 1], s[i], s[i + 1], xe.a, xe.b, er[i], er[i + 1]);
+        fma2(ei[i], ei[i + 1], s[i], s[i + 1], xe.c, xe.d, ei[i], ei[i + 1]);
+        fma2(orr[i], orr[i + 1], s[i], s[i + 1], xo.a, xo.b, orr[i], orr[i + 1]);
+        fma2(oi[i], oi[i + 1], s[i], s[i + 1], xo.c, xo.d, oi[i], oi[i + 1]);
       }
-    };
-    for (; j <= jinj; ++j) step(j, true);  // seeds may still enter
-#pragma unroll 4
-    for (; j < J; ++j) step(j, false);
-  } else {
-    auto step = [&](int jj, bool inj) {
-      const Pair<V> r = sr[jj];
+    } else {
       const Quad<V> q = sx[jj];
 #pragma unroll
       for (int i = 0; i < NP; ++i) {
-        V s = fmav(coefv(r.a, w[i], r.b), s1[i], s2[i]);
-        if (inj) {
-          s = jj == js[i] ? d0[i] : s;
-          s = jj == js[i] + 1 ? d1[i] : s;
-        }
-        s2[i] = s1[i];
-        s1[i] = s;
-        accv(er[i], s, q.a);
-        accv(ei[i], s, q.b);
-        accv(orr[i], s, q.c);
-        accv(oi[i], s, q.d);
+        accv(er[i], s[i], q.a);
+        accv(ei[i], s[i], q.b);
+        accv(orr[i], s[i], q.c);
+        accv(oi[i], s[i], q.d);
       }
-    };
-    for (; j <= jinj; ++j) step(j, true);  // seeds may still enter
+    }
+  };
+  const std::true_type yes;
+  const std::false_type no;
+  int j = jmin;
+  if (NF > 1 && NP > 1 && mixed) {
+    for (; j <= jinj; ++j) step(j, yes, yes);
 #pragma unroll 4
-    for (; j < J; ++j) step(j, false);
+    for (; j < J; ++j) step(j, no, yes);
+  } else {
+    for (; j <= jinj; ++j) step(j, yes, no);
+#pragma unroll 4
+    for (; j < J; ++j) step(j, no, no);
   }
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
@@ -933,15 +950,15 @@ __global__ void __launch_bounds__(32 * PANA_MAXWARPS, std::is_same<V, double>::v
 // ------------------------------------------------------------- launch
 // The synthesis' warps: nlow of 32 np pairs each below keq, then the equatorial ones; mix:
 // in the same CTAs, else the equatorial ones in CTAs of their own.  Shared memory per j: a
-// quad (packed FP32: two) and one form's pair (FP32: three), equatorial a quad or two and
-// a pair.
+// quad (packed FP32: two) and the pairs of nf forms, equatorial a quad or two and a pair.
 struct SynthGrid {
   unsigned ctas;
   int nlow, eq_ofs;
   size_t smem;
-  SynthGrid(size_t v, int npairs, int keq, int lmax, int threads, int np, bool packed, bool mix) {
+  SynthGrid(size_t v, int npairs, int keq, int lmax, int threads, int np, int nf, bool packed,
+            bool mix) {
     const int nw = threads / 32, j = lmax / 2 + 1, ne = packed ? np : 1;
-    const size_t quads = packed ? 8 : 4, low = (quads + (v == 4 ? 6 : 2)) * v * j,
+    const size_t quads = packed ? 8 : 4, low = (quads + 2 * nf) * v * j,
                  eq = (quads + 2) * v * j;
     nlow = (keq + 32 * np - 1) / (32 * np);
     if (!mix) nlow = (nlow + nw - 1) / nw * nw;
@@ -968,7 +985,8 @@ static int anal_threads(size_t v, int lmax) {
 template <int NP>
 static void synth64(const Plan &P, const double2 *x, double2 *F, const SolverState *st,
                     int lstatic, int threads) {
-  const SynthGrid g(8, P.npairs, P.pt64.keq, P.lmax, threads, NP, false, false);
+  const SynthGrid g(8, P.npairs, P.pt64.keq, P.lmax, threads, NP, synth_forms<double>(NP), false,
+                    false);
   k_pair_synth<double, NP><<<dim3(g.ctas, P.lmax + 1), threads, g.smem, P.stream>>>(
       P.pt64, P.npairs, P.lmax, x, F, st, lstatic, g.nlow, g.eq_ofs);
 }
@@ -1007,8 +1025,8 @@ template <int NP>
 static void synth32(const Plan &P, const float2 *x, float2 *F, const SolverState *st,
                     int lstatic) {
   // small maps: both kinds of pairs in a CTA, so that no part of one idles
-  const SynthGrid g(4, P.npairs, P.pt32.keq, P.lmax, PSYN_THREADS32, NP, NP % 2 == 0,
-                    P.npairs < 1024);
+  const SynthGrid g(4, P.npairs, P.pt32.keq, P.lmax, PSYN_THREADS32, NP,
+                    synth_forms<float>(NP), NP % 2 == 0, P.npairs < 1024);
   k_pair_synth<float, NP><<<dim3(g.ctas, P.lmax + 1), PSYN_THREADS32, g.smem, P.stream>>>(
       P.pt32, P.npairs, P.lmax, x, F, st, lstatic, g.nlow, g.eq_ofs);
 }
@@ -1043,7 +1061,8 @@ wf_status launch_legendre_anal<float2>(const Plan &P, const float2 *G, double2 *
 template <int NP>
 static void synth_dd(const Plan &P, const float4 *x, float4 *F, const SolverState *st,
                      int lstatic) {
-  const SynthGrid g(8, P.npairs, P.ptdd.keq, P.lmax, PSYN_THREADS, NP, false, false);
+  const SynthGrid g(8, P.npairs, P.ptdd.keq, P.lmax, PSYN_THREADS, NP, synth_forms<dd>(NP), false,
+                    false);
   typedef Cx<dd>::type C;
   k_pair_synth<dd, NP><<<dim3(g.ctas, P.lmax + 1), PSYN_THREADS, g.smem, P.stream>>>(
       P.ptdd, P.npairs, P.lmax, reinterpret_cast<const C *>(x), reinterpret_cast<C *>(F), st,

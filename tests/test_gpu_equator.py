@@ -98,10 +98,10 @@ def synth_rings(osht, a, nside, lmax, i):
     return out
 
 
-def check_synthesis(torch, osht, prec, nside, lmax, variant=None):
+def check_synthesis(torch, osht, prec, nside, lmax, variant=None, rings=None):
     from paper_1702_08852_gb300 import wf
     a = rand_alm(lmax, nside + lmax)
-    rings = [2 * nside, 2 * nside - 1, 2 * nside - 2, 2 * nside - 4]
+    rings = rings or [2 * nside, 2 * nside - 1, 2 * nside - 2, 2 * nside - 4]
     with wf.Plan(nside, lmax, np.ones(lmax + 1)) as p:
         if variant:
             p.set_tuning(**variant)
@@ -171,3 +171,32 @@ def test_analysis(torch_cuda, osht, prec, nside, lmax):
         got = f(torch.from_numpy(m).cuda()).cpu().numpy()
     ref = analyse_strip(osht, m, nside, lmax)
     assert np.linalg.norm(got - ref) <= tol(prec, lmax) * np.linalg.norm(ref)
+
+
+# the first rings of the belt (z = 2/3): the recurrence's form for their z^2, whatever
+# other pairs their thread, warp or CTA holds
+FORMS = [(p, n, l, k) for p, n, l in [("f64", 128, 256), ("f64", 512, 1024), ("f32", 128, 256)]
+         for k in (1, 2, 4)] + [("df64", 512, 1024, 1)]
+
+
+@pytest.mark.parametrize("prec,nside,lmax,np_", FORMS)
+def test_form_of_each_pair(torch_cuda, osht, prec, nside, lmax, np_):
+    check_synthesis(torch_cuda, osht, prec, nside, lmax, {"syn_np": [np_, np_]},
+                    [nside, nside + 1, nside + nside // 8])
+
+
+def test_half_tiles(torch_cuda):
+    """Nside 1024, lmax 2600: the FP64 and double-float analysis take the ring pairs in two
+    halves; the coefficients that a plan of lmax 2048 has (one tile) are the same but for
+    the order of the sums, 2048 pairs' roundings at random."""
+    torch = torch_cuda
+    from paper_1702_08852_gb300 import wf
+    nside, l0, l1 = 1024, 2048, 2600
+    m = torch.from_numpy(np.random.default_rng(3).standard_normal(12 * nside * nside)).cuda()
+    out = []
+    for lmax in (l0, l1):
+        with wf.Plan(nside, lmax, np.ones(lmax + 1)) as p:
+            out.append([f(m).cpu().numpy() for f in (p.map2alm, p.map2alm_df64)])
+    i, j = (np.concatenate([slots(lmax, l) for l in range(l0 + 1)]) for lmax in (l0, l1))
+    for a, b, u in zip(out[0], out[1], (UNIT["f64"], UNIT["df64"])):
+        assert np.linalg.norm(a[i] - b[j]) <= 4 * u * np.sqrt(2048) * np.linalg.norm(a)
