@@ -59,9 +59,7 @@
 // lanes once.  The terms start at the first |Q_j| >= 2^-100 (j = js); in the block that
 // holds js the checkpoint is, where the state before the block is out of the
 // arithmetic's range, the seeds (s_js, s_js+1) instead, which enter at j = js (jin).
-// FP64 always has that state; FP32 where it is above 2^-120, and a block that ends
-// below 2^-80 without it is left out (an FP32 sum does not see such terms beside the
-// O(1) ones).
+// FP64 always has that state; FP32 where it is above 2^-120.
 #include <limits.h>
 #include <math.h>
 
@@ -1222,7 +1220,7 @@ __global__ void k_pair_walk(int npairs, int lmax, const PairTab<double> t_,
   const double seed0 = s1;
   for (;;) {
     if ((j & 15) == 15 || j + 1 == J) {
-      if (!fits && (j >> 4) == bj && fmax(fabs(s1), fabs(s2)) >= 0x1p-80) {
+      if (!fits && (j >> 4) == bj) {
         u.ck[(cb + bj) * stride + k] = make_float2((float)seed0, (float)nx);
         u.jin[mk] = js;
       }

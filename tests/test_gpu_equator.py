@@ -200,3 +200,21 @@ def test_half_tiles(torch_cuda):
     i, j = (np.concatenate([slots(lmax, l) for l in range(l0 + 1)]) for lmax in (l0, l1))
     for a, b, u in zip(out[0], out[1], (UNIT["f64"], UNIT["df64"])):
         assert np.linalg.norm(a[i] - b[j]) <= 4 * u * np.sqrt(2048) * np.linalg.norm(a)
+
+
+def test_small_terms_f32(torch_cuda, osht):
+    """Terms between 2^-100 and 2^-80 count in FP32 too: m = 20 on the ring next to the
+    pole, where lam_lm first reaches 2^-99 at l = 41 and 2^-92 at l = 51, the end of the
+    analysis' first block.  Tolerance as for the FP32 transforms, of each coefficient."""
+    torch = torch_cuda
+    from paper_1702_08852_gb300 import wf
+    nside, lmax = 64, 128
+    m = np.zeros(12 * nside * nside)
+    m[:4] = [1.0, -2.0, 0.5, 3.0]
+    ls = np.arange(44, 52)
+    ms = np.full(ls.size, 20)
+    ref = 4 * np.pi / m.size * osht.adjoint_modes(m, nside, lmax, ls, ms)
+    with wf.Plan(nside, lmax, np.ones(lmax + 1)) as p:
+        got = p.map2alm_f32(torch.from_numpy(m).cuda()).cpu().numpy()
+    err = np.abs(got[ms * (2 * lmax + 1 - ms) // 2 + ls] - ref)
+    assert np.all(err <= UNIT["f32"] * (64 + 2 * nside * np.sqrt(lmax + 1.0)) * np.abs(ref))
