@@ -70,6 +70,7 @@ wf_status autotune(Plan &P) {
   static const int syn_cand[6] = {1, 2, 4, 2, 4, 2};  // slots 3 .. 5 (FP32): packed
   wf_status st = WF_OK;
   for (int k = 0; k < 2 && st == WF_OK; ++k) {  // 0 = FP64, 1 = FP32
+    if (k ? !P.pt32.ck : !P.pt64.ck) continue;  // no transform of this type can run
     float best = 1e30f;
     int pick = P.syn_np[k];
     for (int ci = 0; ci < 3 && st == WF_OK; ++ci) {

@@ -980,6 +980,12 @@ static int anal_threads(size_t v, int lmax) {
   return 32 * std::max(2, std::min(PANA_MAXWARPS, v == 4 ? nb : 2 * nb));
 }
 
+static wf_status ready(const void *ck) {
+  if (ck) return WF_OK;
+  set_error("transform: Nside is too large for the ring FFTs of this precision");
+  return WF_ERR_CUDA;
+}
+
 template <int NP>
 static void synth64(const Plan &P, const double2 *x, double2 *F, const SolverState *st,
                     int lstatic, int threads) {
@@ -992,6 +998,7 @@ static void synth64(const Plan &P, const double2 *x, double2 *F, const SolverSta
 template <>
 wf_status launch_legendre_synth<double2>(const Plan &P, const double2 *x, double2 *F,
                                          const SolverState *st, int lstatic) {
+  WF_TRY(ready(P.pt64.ck));
   ++P.nlaunch;
   // one or two warps per CTA: an SM's FP64 unit (2 lanes per clock) is full with a
   // few warps, and small CTAs spread small maps over the SMs
@@ -1009,6 +1016,7 @@ template <>
 wf_status launch_legendre_anal<double2>(const Plan &P, const double2 *G, double2 *x,
                                         const SolverState *st, int mode, int lstatic,
                                         const double2 *src, double2 *) {
+  WF_TRY(ready(P.pt64.ck));
   ++P.nlaunch;
   const int tile = anal_tile(8, P.npairs, P.lmax);
   k_pair_anal<double><<<P.lmax + 1, anal_threads(8, P.lmax), anal_smem(8, P.npairs, P.lmax, tile),
@@ -1032,6 +1040,7 @@ static void synth32(const Plan &P, const float2 *x, float2 *F, const SolverState
 template <>
 wf_status launch_legendre_synth<float2>(const Plan &P, const float2 *xs, float2 *F,
                                         const SolverState *st, int lstatic) {
+  WF_TRY(ready(P.pt32.ck));
   ++P.nlaunch;
   switch (P.syn_np[1]) {
     case 1: synth32<1>(P, xs, F, st, lstatic); break;
@@ -1046,6 +1055,7 @@ template <>
 wf_status launch_legendre_anal<float2>(const Plan &P, const float2 *G, double2 *x,
                                        const SolverState *st, int mode, int lstatic,
                                        const double2 *src, float2 *xs_out) {
+  WF_TRY(ready(P.pt32.ck));
   ++P.nlaunch;
   const int tile = anal_tile(4, P.npairs, P.lmax);
   k_pair_anal<float><<<P.lmax + 1, anal_threads(4, P.lmax), anal_smem(4, P.npairs, P.lmax, tile),
@@ -1069,6 +1079,7 @@ static void synth_dd(const Plan &P, const float4 *x, float4 *F, const SolverStat
 
 wf_status launch_legendre_synth_dd(const Plan &P, const float4 *xs, float4 *F,
                                    const SolverState *st, int lstatic) {
+  WF_TRY(ready(P.ptdd.ck));
   ++P.nlaunch;
   if (P.npairs >= 1024)
     synth_dd<2>(P, xs, F, st, lstatic);
@@ -1081,6 +1092,7 @@ wf_status launch_legendre_synth_dd(const Plan &P, const float4 *xs, float4 *F,
 wf_status launch_legendre_anal_dd(const Plan &P, const float4 *G, double2 *x,
                                   const SolverState *st, int mode, int lstatic,
                                   const double2 *src) {
+  WF_TRY(ready(P.ptdd.ck));
   ++P.nlaunch;
   typedef Cx<dd>::type C;
   const int tile = anal_tile(8, P.npairs, P.lmax);
@@ -1214,19 +1226,21 @@ __global__ void k_pair_walk(int npairs, int lmax, const PairTab<double> t_,
   t_.seed[mk] = make_double2(s1, nx);
   u.seed[mk] = make_float2((float)s1, (float)nx);
   const double2 st = make_double2(ldexp(b1, be), ldexp(b2, be));
-  t_.ck[(cb + bj) * stride + k] = st;
+  if (t_.ck) t_.ck[(cb + bj) * stride + k] = st;
+  if (!t_.ck && !u.ck) return;
   const bool fits = fmax(fabs(st.x), fabs(st.y)) >= 0x1p-120;
-  if (fits) u.ck[(cb + bj) * stride + k] = make_float2((float)st.x, (float)st.y);
+  if (fits && u.ck) u.ck[(cb + bj) * stride + k] = make_float2((float)st.x, (float)st.y);
   const double seed0 = s1;
   for (;;) {
     if ((j & 15) == 15 || j + 1 == J) {
-      if (!fits && (j >> 4) == bj) {
+      if (!fits && (j >> 4) == bj && u.ck) {
         u.ck[(cb + bj) * stride + k] = make_float2((float)seed0, (float)nx);
         u.jin[mk] = js;
       }
       if (j + 1 < J) {
-        t_.ck[(cb + (j >> 4) + 1) * stride + k] = make_double2(s1, s2);
-        u.ck[(cb + (j >> 4) + 1) * stride + k] = make_float2((float)s1, (float)s2);
+        const long at = (cb + (j >> 4) + 1) * stride + k;
+        if (t_.ck) t_.ck[at] = make_double2(s1, s2);
+        if (u.ck) u.ck[at] = make_float2((float)s1, (float)s2);
       }
     }
     if (++j >= J) break;
@@ -1253,8 +1267,8 @@ __global__ void k_eq_walk(int npairs, int lmax, const PairTab<double> t_, const 
   double even = ldexp(mant[i], expo[i]), odd = 0.0;  // rec[0].x = 0 leaves lam_mm
   for (int j = 0; j < J; ++j) {
     if ((j & 15) == 0) {
-      t_.ck_e[at] = make_double2(even, odd);
-      u.ck_e[at] = make_float2((float)even, (float)odd);
+      if (t_.ck_e) t_.ck_e[at] = make_double2(even, odd);
+      if (u.ck_e) u.ck_e[at] = make_float2((float)even, (float)odd);
       at += t_.estride;
     }
     const double2 r = rec[j];
@@ -1466,17 +1480,20 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
   WF_CUDA(cudaMalloc(&u.jin, sizeof(int) * mk));
   WF_CUDA(cudaMalloc(&t.seed, sizeof(double2) * mk));
   WF_CUDA(cudaMalloc(&u.seed, sizeof(float2) * mk));
-  WF_CUDA(cudaMalloc(&t.ck, sizeof(double2) * ck));
-  WF_CUDA(cudaMalloc(&u.ck, sizeof(float2) * ck));
-  WF_CUDA(cudaMalloc(&t.ck_e, sizeof(double2) * ce));
-  WF_CUDA(cudaMalloc(&u.ck_e, sizeof(float2) * ce));
+  // the checkpoints are most of a plan (Nside 1024: 3.3 of 5.1 GB, growing as Nside^3):
+  // only for the transforms whose ring FFTs can run
+  auto checkpoints = [&](auto **a, auto **b) {
+    WF_CUDA(cudaMalloc(a, sizeof(**a) * ck));
+    WF_CUDA(cudaMalloc(b, sizeof(**b) * ce));
+    WF_CUDA(cudaMemsetAsync(*a, 0, sizeof(**a) * ck, P.stream));
+    WF_CUDA(cudaMemsetAsync(*b, 0, sizeof(**b) * ce, P.stream));
+    return WF_OK;
+  };
+  if (ring_fits(P, sizeof(double2))) WF_TRY(checkpoints(&t.ck, &t.ck_e));
+  if (ring_fits(P, sizeof(float2))) WF_TRY(checkpoints(&u.ck, &u.ck_e));
   WF_CUDA(cudaMalloc(&t.gfirst, sizeof(int) * nb));
   WF_CUDA(cudaMemsetAsync(t.js, 0x3f, sizeof(int) * mk, P.stream));
   WF_CUDA(cudaMemsetAsync(u.jin, 0x3f, sizeof(int) * mk, P.stream));
-  WF_CUDA(cudaMemsetAsync(t.ck, 0, sizeof(double2) * ck, P.stream));
-  WF_CUDA(cudaMemsetAsync(u.ck, 0, sizeof(float2) * ck, P.stream));
-  WF_CUDA(cudaMemsetAsync(t.ck_e, 0, sizeof(double2) * ce, P.stream));
-  WF_CUDA(cudaMemsetAsync(u.ck_e, 0, sizeof(float2) * ce, P.stream));
   WF_CUDA(cudaMemsetAsync(t.gfirst, 0x7f, sizeof(int) * nb, P.stream));  // none
   u.js = t.js;
   u.gfirst = t.gfirst;
@@ -1484,7 +1501,7 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
   k_pair_walk<<<(unsigned)((n + 127) / 128), 128, 0, P.stream>>>(P.npairs, lmax, t, u, mant,
                                                                  expo);
   WF_CUDA(cudaGetLastError());
-  if (keq < P.npairs) {
+  if (keq < P.npairs && (t.ck_e || u.ck_e)) {
     const long ne = (long)(P.npairs - keq) * (lmax + 1);
     k_eq_walk<<<(unsigned)((ne + 127) / 128), 128, 0, P.stream>>>(P.npairs, lmax, t, u, mant, expo);
     WF_CUDA(cudaGetLastError());

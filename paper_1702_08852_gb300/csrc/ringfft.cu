@@ -420,6 +420,16 @@ template <> struct Tables<ddc> {
   static const void *tp(const Plan &P) { return P.tpdd; }
 };
 
+static size_t ring_bytes(size_t elem, int M, int n, int threads) {
+  return elem * (M + (n < threads ? 2 * threads : 0));
+}
+constexpr int RING_SMEM = 220 * 1024;
+
+bool ring_fits(const Plan &P, size_t elem) {
+  return ring_bytes(elem, P.fftMmax, 0, P.fftMmax >= 8192 ? RING_THREADS_BIG : RING_THREADS) <=
+         RING_SMEM;
+}
+
 template <typename T2, int MODE>
 static wf_status launch_ring_mode(const Plan &P, const typename CT<T2>::G *F,
                                   typename CT<T2>::G *G, const double *in_map,
@@ -444,9 +454,7 @@ static wf_status launch_ring_mode(const Plan &P, const typename CT<T2>::G *F,
   const int Mall = std::max(Mg[0], Mg[1]), nall = std::min(nmin[0], nmin[1]);
   // rings with fewer pixels than threads fold through a partial-sum area of 2 x threads
   // entries placed after the FFT buffer
-  auto bytes = [](int M, int n, int threads) {
-    return sizeof(T2) * (M + (n < threads ? 2 * threads : 0));
-  };
+  auto bytes = [](int M, int n, int threads) { return ring_bytes(sizeof(T2), M, n, threads); };
   constexpr size_t QUARTER = 56 * 1024;
   const size_t all = bytes(Mall, nall, RING_THREADS);
   const bool one = all + sizeof(typename CT<T2>::W) * tab <= QUARTER;
@@ -552,7 +560,7 @@ wf_status launch_to_dd(const Plan &P, const double *in, float2 *out, long n) {
 }
 
 wf_status init_ring_attributes() {
-  const int big = 220 * 1024;
+  const int big = RING_SMEM;
   WF_CUDA(cudaFuncSetAttribute(k_ring<double2, RING_SYNTH>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   WF_CUDA(cudaFuncSetAttribute(k_ring<double2, RING_ANALYSIS>,

@@ -56,7 +56,8 @@ struct PairTab {
   V *w = nullptr;                  // [3][stride]: z^2 - 1, z^2 - 1/2, z^2
   V *z = nullptr, *zl = nullptr;   // [stride]; FP32: z = z + zl
   int *js = nullptr;               // [lmax+1][stride] first j with |Q_j| >= 2^-100, k < keq
-  typename CkVec<V>::type *ck = nullptr;  // [block of 16 j of m][cstride]: k < keq
+  typename CkVec<V>::type *ck = nullptr;  // [block of 16 j of m][cstride]: k < keq; NULL
+                                          // where no transform of this type can run
   int cstride = 0, estride = 0;    // keq rounded up to 64; stride less keq rounded down
   typename CkVec<V>::type *seed = nullptr;  // [lmax+1][stride] (s_js, s_js+1)
   int *jin = nullptr;              // [lmax+1][stride] FP32: j where ck holds the seeds
@@ -354,6 +355,9 @@ wf_status launch_to_dd(const Plan &P, const double *in, float2 *out, long n);
 
 // once per plan (kernel attributes; allowed outside stream capture only)
 wf_status init_ring_attributes();
+// whether the ring FFTs of complex elements of `elem` bytes fit shared memory (16 bytes:
+// up to Nside 1024, 8 bytes: up to 2048)
+bool ring_fits(const Plan &P, size_t elem);
 
 // autotune.cu: time the Legendre launch variants once per geometry
 wf_status autotune(Plan &P);

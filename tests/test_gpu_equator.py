@@ -218,3 +218,24 @@ def test_small_terms_f32(torch_cuda, osht):
         got = p.map2alm_f32(torch.from_numpy(m).cuda()).cpu().numpy()
     err = np.abs(got[ms * (2 * lmax + 1 - ms) // 2 + ls] - ref)
     assert np.all(err <= UNIT["f32"] * (64 + 2 * nside * np.sqrt(lmax + 1.0)) * np.abs(ref))
+
+
+def test_large_plan(torch_cuda):
+    """Nside 2048: only the FP32 ring FFTs fit shared memory, so a plan has no FP64
+    checkpoints.  Without them it holds 6.2 GB (maps 1.4, ring coefficients 0.8, chirps 1.4,
+    FP32 checkpoints 2.2 and less than half a GB of others), with them 10.7 GB."""
+    torch = torch_cuda
+    from paper_1702_08852_gb300 import wf
+    nside, lmax = 2048, 2048
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    with wf.Plan(nside, lmax, np.ones(lmax + 1)) as p:
+        assert free - torch.cuda.mem_get_info()[0] < 8.5e9
+        a = torch.zeros(p.nalm, dtype=torch.complex128, device="cuda")
+        a[3] = 1.0  # l = 3, m = 0
+        with pytest.raises(wf.WFError) as e:
+            p.alm2map(a)
+        assert e.value.status == wf.WF_ERR_CUDA
+        m = p.alm2map_f32(a)
+        b = p.map2alm_f32(m)
+        assert torch.linalg.vector_norm(b - a) < 1e-3  # quadrature
