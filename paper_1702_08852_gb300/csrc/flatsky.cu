@@ -602,6 +602,10 @@ wf_status wf_flat_plan(wf_flat_t *out, int n, double pixel_area, const double *c
       (e = cudaMemcpy(F->tw, tw.data(), sizeof(double2) * tw.size(), cudaMemcpyHostToDevice)) !=
           cudaSuccess)
     return fail("upload", e);
+  if (const wf_status s = uploads_done(); s != WF_OK) {
+    flat_free(F);
+    return s;
+  }
   *out = F;
   return WF_OK;
 }

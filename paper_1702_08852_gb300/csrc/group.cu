@@ -537,6 +537,7 @@ static wf_status build_group(Plan &P) {
                                (int)smem_bytes(2 * G_MAX_MAPS)));
   WF_CUDA(cudaFuncSetAttribute(k_group_mma<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)smem_bytes(2 * G_MAX_MAPS)));
+  WF_TRY(uploads_done());
   dim3 grid((P.npairs + 127) / 128, L + 1);
   ++P.nlaunch;
   k_group_tables<<<grid, 128, 0, P.stream>>>(P.pt64, P.npairs, L, g->ana, g->ana_first, g->syn,

@@ -1464,6 +1464,7 @@ wf_status build_pair_tables(Plan &P, const double *mant, const int *expo) {
   WF_TRY(up(&t.w, w));
   WF_TRY(up(&t.z, z));
   WF_TRY(up(&P.pt32.zl, zl));
+  WF_TRY(uploads_done());
   for (double2 **a : {&t.rec[0], &t.rec[1], &t.rec[2], &t.rec_e})
     WF_CUDA(cudaMalloc(a, sizeof(double2) * nq));
   for (double **a : {&t.se, &t.sn, &t.so, &t.ge, &t.go})

@@ -574,7 +574,7 @@ static wf_status net_alloc(Net &N) {
   const long wout = std::max((long)H * (H + 1), (long)H * 4) * K;
   WF_CUDA(cudaMalloc(&N.wpart, sizeof(float) * wout * NN_PARTS));
   WF_CUDA(cudaMalloc(&N.red, sizeof(double) * 4 * 304 + sizeof(double) * 2 * (P.lmax + 1)));
-  return WF_OK;
+  return uploads_done();
 }
 
 // the kernels' width is a template parameter: f.template operator()<K>()
@@ -801,7 +801,7 @@ wf_status wf_net_set_params(wf_net_t net, const float *host, long n) {
   WF_CUDA(cudaMemset(net->am, 0, sizeof(float) * n));
   WF_CUDA(cudaMemset(net->av, 0, sizeof(float) * n));
   net->step = 0;
-  return WF_OK;
+  return uploads_done();
 }
 
 wf_status wf_net_get_params(wf_net_t net, float *host, long n) {

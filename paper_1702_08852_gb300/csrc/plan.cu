@@ -375,8 +375,8 @@ wf_status build_tables(Plan &P) {
     WF_CUDA(cudaMemcpy(P.cl32, cl32.data(), sizeof(float) * (P.lmax + 1),
                        cudaMemcpyHostToDevice));
   }
-  WF_TRY(make_seeds(P));
-  return WF_OK;
+  WF_TRY(uploads_done());
+  return make_seeds(P);
 }
 
 // ---------------------------------------------------------------- noise

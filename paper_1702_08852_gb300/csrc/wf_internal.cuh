@@ -32,6 +32,14 @@ void set_error_static(const char *msg);
     if (s_ != WF_OK) return s_;         \
   } while (0)
 
+// cudaMemcpy from pageable memory may return, and cudaMemset returns, before the device
+// has the data, and a stream made with cudaStreamNonBlocking does not wait for either: called after
+// a plan's uploads, before kernels on its stream read them.
+inline wf_status uploads_done() {
+  WF_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+  return WF_OK;
+}
+
 // ---------------------------------------------------------------- geometry
 // Tables of the Legendre kernels in the parity-pair basis (legpair.cu), V the
 // arithmetic; indexed by (m, j) except where noted
