@@ -234,7 +234,7 @@ __device__ __forceinline__ V lane_sums(V *v, int lane) {
 //   E_j = se_j a_{m+2j} + sn_j a_{m+2j+2},   O_j = so_j a_{m+2j+1}.
 // F_north = sum_j s_j (E_j + z O_j), F_south the difference.
 constexpr int PSYN_THREADS = 64;     // FP64
-constexpr int PSYN_THREADS32 = 128;  // FP32
+constexpr int PSYN_THREADS32 = 256;  // FP32, at most
 
 template <typename V>
 __host__ __device__ constexpr int synth_forms(int np) {  // forms staged by a CTA
@@ -1030,10 +1030,17 @@ wf_status launch_legendre_anal<double2>(const Plan &P, const double2 *G, double2
 template <int NP>
 static void synth32(const Plan &P, const float2 *x, float2 *F, const SolverState *st,
                     int lstatic) {
-  // small maps: both kinds of pairs in a CTA, so that no part of one idles
-  const SynthGrid g(4, P.npairs, P.pt32.keq, P.lmax, PSYN_THREADS32, NP,
-                    synth_forms<float>(NP), NP % 2 == 0, P.npairs < 1024);
-  k_pair_synth<float, NP><<<dim3(g.ctas, P.lmax + 1), PSYN_THREADS32, g.smem, P.stream>>>(
+  // both kinds of pairs in a CTA while two fit an SM, so that few of its warps idle, and 8
+  // warps on large maps.  4 warps with CTAs of their own for the equatorial pairs: 0.574 ms
+  // at Nside 1024 (a fifth of the warps idle), 0.487 ms with 8 in common ones; transform
+  // at Nside 512 201 and 194 us; at Nside 256 the kernel takes 17.9 us with 4 warps, 19.2
+  // with 8
+  const int np = P.npairs, keq = P.pt32.keq, nf = synth_forms<float>(NP);
+  const int threads = np < 1024 ? PSYN_THREADS32 / 2 : PSYN_THREADS32;
+  constexpr bool packed = NP % 2 == 0;
+  SynthGrid g(4, np, keq, P.lmax, threads, NP, nf, packed, true);
+  if (g.smem > PAIR_SMEM / 2) g = SynthGrid(4, np, keq, P.lmax, threads, NP, nf, packed, false);
+  k_pair_synth<float, NP><<<dim3(g.ctas, P.lmax + 1), threads, g.smem, P.stream>>>(
       P.pt32, P.npairs, P.lmax, x, F, st, lstatic, g.nlow, g.eq_ofs);
 }
 

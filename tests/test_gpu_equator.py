@@ -239,3 +239,21 @@ def test_large_plan(torch_cuda):
         m = p.alm2map_f32(a)
         b = p.map2alm_f32(m)
         assert torch.linalg.vector_norm(b - a) < 1e-3  # quadrature
+
+
+def test_synthesis_in_separate_blocks(torch_cuda):
+    """Nside 1024, lmax 2600: too much shared memory for both kinds of pairs in a block of
+    the FP32 synthesis.  A field of l <= 2048 comes out as from the plan of lmax 2048, whose
+    blocks are common: the same sums."""
+    torch = torch_cuda
+    from paper_1702_08852_gb300 import wf
+    nside, l0, l1 = 1024, 2048, 2600
+    a = rand_alm(l0, 5)
+    b = np.zeros((l1 + 1) * (l1 + 2) // 2, complex)
+    for l in range(l0 + 1):
+        b[slots(l1, l)] = a[slots(l0, l)]
+    out = []
+    for lmax, x in ((l0, a), (l1, b)):
+        with wf.Plan(nside, lmax, np.ones(lmax + 1)) as p:
+            out.append(p.alm2map_f32(torch.from_numpy(x).cuda()))
+    assert torch.linalg.vector_norm(out[0] - out[1]) <= UNIT["f32"] * torch.linalg.vector_norm(out[0])
