@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(PSYN_THREADS32)
 // with the solver's filter, source term and Cauchy sums fused.
 constexpr int PANA_TILE = 2048;
 constexpr int PAIR_SMEM = 220 * 1024;  // dynamic shared memory limit of these kernels
-constexpr int PANA_MAXWARPS = 8;
+constexpr int PANA_MAXWARPS = 16;
 constexpr int CKJ = 16;
 
 // 16 steps of R pairs (one lane's): the recurrence and the four sums of each j; in
@@ -692,7 +692,8 @@ template <typename E> __device__ __forceinline__ E epi_val(E v) { return v; }
 template <typename E> __device__ __forceinline__ double epi_val(dd v) { return dd_val(v); }
 
 template <typename V>
-__global__ void __launch_bounds__(32 * PANA_MAXWARPS, std::is_same<V, double>::value ? 1 : 2)
+__global__ void __launch_bounds__(std::is_same<V, dd>::value ? 32 * PANA_MAXWARPS : 256,
+                                  std::is_same<V, float>::value ? 2 : 1)
     k_pair_anal(const PairTab<V> t, int npairs, int lmax,
                 const double *__restrict__ cl, double omega,
                 const typename Cx<V>::type *__restrict__ G, double2 *__restrict__ x,
@@ -974,10 +975,11 @@ static size_t anal_smem(size_t v, int npairs, int lmax, int tile) {
 static int anal_tile(size_t v, int npairs, int lmax) {
   return anal_smem(v, npairs, lmax, PANA_TILE) <= PAIR_SMEM ? PANA_TILE : PANA_TILE / 2;
 }
-// a warp per item of the CTA of m = 0 (FP64, dd: twice its blocks)
-static int anal_threads(size_t v, int lmax) {
-  const int nb = lmax / 32 + 1;
-  return 32 * std::max(2, std::min(PANA_MAXWARPS, v == 4 ? nb : 2 * nb));
+// a warp per item of the CTA of m = 0 (FP64, dd: twice its blocks), at most 8; dd 16 where
+// one CTA fills an SM's shared memory (Nside 1024: 8 warps 9.9 ms, 16 7.6 ms)
+static int anal_threads(size_t v, int lmax, size_t dd_smem = 0) {
+  const int nb = lmax / 32 + 1, most = dd_smem > PAIR_SMEM / 2 ? PANA_MAXWARPS : 8;
+  return 32 * std::max(2, std::min(most, v == 4 ? nb : 2 * nb));
 }
 
 static wf_status ready(const void *ck) {
@@ -1103,8 +1105,8 @@ wf_status launch_legendre_anal_dd(const Plan &P, const float4 *G, double2 *x,
   ++P.nlaunch;
   typedef Cx<dd>::type C;
   const int tile = anal_tile(8, P.npairs, P.lmax);
-  k_pair_anal<dd><<<P.lmax + 1, anal_threads(8, P.lmax), anal_smem(8, P.npairs, P.lmax, tile),
-                     P.stream>>>(
+  const size_t smem = anal_smem(8, P.npairs, P.lmax, tile);
+  k_pair_anal<dd><<<P.lmax + 1, anal_threads(8, P.lmax, smem), smem, P.stream>>>(
       P.ptdd, P.npairs, P.lmax, P.cl_d, P.omega, reinterpret_cast<const C *>(G), x, P.partials,
       src, nullptr, nullptr, P.pt64.se, P.pt64.sn, P.pt64.so, P.pt64.ge, P.pt64.go, st, mode,
       lstatic, tile);
