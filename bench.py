@@ -140,17 +140,18 @@ def measured_peaks():
 
 # DRAM bytes (read + write, ncu) of one full-band launch of the FP32 analysis
 # at Nside 1024 / lmax 2048 (an ncu capture of the --kernel-case legendre32
-# run); scaled to a live launch by its share of the full band's terms.  None
-# once the kernel changes after a capture, as the parity-pair analysis has.
-ANALYSIS_DRAM_FULL_BAND = {"nside": 1024, "bytes": None,
+# run); scaled to a live launch by its share of the full band's terms.  "variant"
+# is what a plan reports by default: these fields select nothing any more.
+ANALYSIS_DRAM_FULL_BAND = {"nside": 1024, "bytes": 9.93e8,
                            "terms": 3140761977.0,
-                           "variant": {"ana_np": 4, "ana_queue": 0, "ana_packed": 1,
-                                       "ana_global_acc": 1},
-                           "source": "no capture since the kernel changed"}
+                           "variant": {"ana_np": 8, "ana_queue": 0, "ana_packed": 0,
+                                       "ana_global_acc": 0},
+                           "source": "profiles/pair_basis_and_cases.md"}
 
 
 def analysis_variant(tuning):
-    """The FP32 analysis launch variant of a plan's tuning report."""
+    """The FP32 analysis fields of a plan's tuning report (kept as they were set; the
+    analysis is one kernel)."""
     return {"ana_np": tuning["ana_np"][1], "ana_queue": tuning["ana_queue"],
             "ana_packed": tuning["ana_packed"], "ana_global_acc": tuning["ana_global_acc"]}
 
@@ -179,10 +180,11 @@ def alu_peaks(wf):
             "source": "measured live: wf_alu_peak FMA chains on every SM, best of 5"}
 
 
-# FP32 operations of the double-float formulas per (l, m, ring pair) term: 84
-# per step of the parity-pair recurrence (the step and four accumulations of a
-# product), which serves two l
-DD_FLOPS_PER_TERM = 42.0
+# FP32 operations of the double-float formulas per (l, m, ring pair) term, a
+# multiply-add counted as two: 93 per step of the parity-pair recurrence (33 for the
+# step, 15 for each of four accumulated products), which serves two l (the eighth of
+# the pairs next to the equator: 110)
+DD_FLOPS_PER_TERM = 46.5
 KERNEL_NAMES = ["legendre_analysis_f32", "legendre_synthesis_f32", "ring_step_f32",
                 "legendre_synthesis_dd", "legendre_analysis_dd", "ring_step_dd"]
 
@@ -191,7 +193,7 @@ def kernel_rooflines(kern, alu, peaks, peak_src, args, ana_variant):
     """Per-kernel rooflines of the timed solves (wf_kernel_stats, CUDA events
     around every launch) and the dominant kernel's at the top level.
     Legendre kernels: 7 algorithmic flops per term against the measured FP32
-    FMA peak (the double-float ones: the 42 FP32 operations of their formulas per
+    FMA peak (the double-float ones: the 46.5 FP32 operations of their formulas per
     term against the same peak, and their FP64-equivalent 7 flops per term
     beside the measured FP64 peak); ring steps: DRAM bytes they cannot avoid
     against the measured copy bandwidth."""

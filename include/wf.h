@@ -352,7 +352,7 @@ wf_status wf_trace(wf_plan_t plan, int *count, int *stage, double *xi,
  * opts.timing = 1 since plan creation or the last reset.
  *  kernel    0 = Legendre analysis (Omega Y^T with the fused filter),
  *            1 = Legendre synthesis, 2 = ring step (fold, inverse ring
- *            FFTs, the t-update of Eq. 14, forward ring FFTs; both launches)
+ *            FFTs, the t-update of Eq. 14, forward ring FFTs; in one launch or two)
  *            of the captured FP32 / FP64 iterations; 3 = Legendre
  *            synthesis, 4 = Legendre analysis,
  *            5 = ring step, all three in double-float, of the mixed solver's

@@ -91,8 +91,8 @@ __device__ __forceinline__ int sw(int i) {
 // and W_h^j = (W_2h^j)^2, side by side in a table that holds every span's entries at
 // h / 2 - 1 (twiddle_table: Mmax / 2 - 1 entries for lengths up to Mmax), one vector load
 // per butterfly instead of two scattered ones or a complex square (FP32 transform pair at
-// Nside 256: 156 -> 144 us with the chirp tables in shared memory, flat solve at n = 256:
-// 594 -> 540 ms).  The table
+// Nside 256: 156 -> 144 us with the chirp tables in shared memory, flat solve at n = 256
+// 1.10 times as fast).  The table
 // (16 KB in FP32 for 2048 points) stays in L1; computing the pair in FP32 by sincospi
 // took 40 of a butterfly's ~100 instructions.
 template <typename T2>

@@ -24,8 +24,8 @@
 // real rows as one complex row, and keep the filtered spectrum and C in the
 // bit-reversed ky order that the forward column transform leaves, so no permutation
 // pass is made.  FP64 arithmetic (2 multiply-adds per clock and SM) bounds both forms:
-// per iteration at n = 256 it is ~9 us of the h form.  A solve at n = 256 takes 554 ms
-// with the h kernels (740 ms with the general ones and computed twiddles): what is left above the
+// per iteration at n = 256 it is ~9 us of the h form.  A solve at n = 256 takes 548 ms
+// with the h kernels (730 ms with the general ones and computed twiddles): what is left above the
 // arithmetic is the latency of the passes' barriers at 64 threads per CTA.  Other spectra
 // run the general kernels.
 #include <math.h>

@@ -41,17 +41,19 @@
 // l instead of E and O: a map that is zero but on nine rings around the equator comes out
 // to 1.6e-7 in FP32 at Nside 512 (1.3e-4 without it) and to 2e-14 in FP64 (1.9e-13).
 //
-// Bound: the FP64 unit, 2 multiply-adds per clock and SM.  At Nside 1024, lmax 2048
-// (3.14e9 terms) the synthesis takes 16.6 ms (21.4 ms with the one-step recurrence)
-// and the analysis 16.9 ms (29.0 ms), against 15 ms for 3 multiply-adds per term at
-// the unit's measured 1.25 TFLOP/s; at Nside 150, lmax 311, 0.106 and 0.142 ms
-// (0.233 and 0.276 ms).  FP32: the FMA pipe takes 6 clocks per warp and step, 0.26 ms
-// at Nside 1024; measured 0.435 ms (synthesis, from 0.645) and 0.597 ms (analysis,
-// from 0.891), at Nside 256 17.7 and 23 us (from 23 and 38): what is left is the
-// reductions, the loads between the blocks and, on small maps, the largest m's chain.
-// Double-float (84 FP32 operations per step against 116 for two l of the one-step
-// recurrence): Nside 512 synthesis 0.63 ms (0.76), analysis 0.92 ms (0.97 and a combine
-// pass of 0.04), bound by the FP32 pipe's dependent chains at 16 warps per SM.
+// Bound: the FP64 unit, 2 multiply-adds per clock and SM (98 and 92 % busy at Nside 512).
+// At Nside 1024, lmax 2048 (3.14e9 terms) the synthesis takes 16.6 ms (21.4 ms with the
+// one-step recurrence for all pairs) and the analysis 17.7 ms (29.0 ms), against 15.6 ms
+// for 3 multiply-adds per term, 4 for the equatorial eighth, at the unit's measured 1.25
+// TFLOP/s; at Nside 150, lmax 311, 0.104 and 0.137 ms (0.233 and 0.276 ms).  FP32: the
+// FMA pipe takes 6 clocks per warp and step (equatorial 10), 0.28 ms at Nside 1024;
+// measured 0.487 ms (synthesis, from 0.645) and 0.656 ms (analysis, from 0.891), at Nside
+// 256 17.9 and 31.5 us: what is left is the reductions, the loads between the blocks (1.0
+// GB of DRAM at Nside 1024, most of it checkpoints: 0.15 ms) and, on small maps, the
+// largest m's chain.  Double-float (93 FP32 operations per step, 110 equatorial, against
+// 116 for two l of the one-step recurrence; a multiply-add counts as two): Nside 512
+// synthesis 0.61 ms (0.76), analysis 1.05 ms (0.97 and a combine pass of 0.04), Nside 1024
+// 4.4 and 7.6 ms, bound by the FP32 pipe's dependent chains at 16 warps per SM.
 //
 // Checkpoints: ck[(block b of 16 j of m)][pair] holds (s_{16b-1}, s_{16b-2}), so any 16
 // j can be computed on their own: a warp of the analysis owns 16 j of one m, keeps
@@ -1138,7 +1140,7 @@ __global__ void k_alm_to_dd(const double2 *__restrict__ x, long n, float4 *__res
   }
 }
 
-wf_status launch_prescale_dd(const Plan &P, const double2 *x, float4 *xs) {
+wf_status launch_alm_to_dd(const Plan &P, const double2 *x, float4 *xs) {
   ++P.nlaunch;
   const unsigned grid = (unsigned)std::min((P.nalm + 255) / 256, 8L * P.num_sms);
   k_alm_to_dd<<<grid, 256, 0, P.stream>>>(x, P.nalm, xs);

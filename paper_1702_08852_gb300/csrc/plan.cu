@@ -329,10 +329,10 @@ static wf_status make_seeds(Plan &P) {
   WF_CUDA(cudaGetDevice(&dev));
   P.device = dev;
   WF_CUDA(cudaDeviceGetAttribute(&P.num_sms, cudaDevAttrMultiProcessorCount, dev));
-  // FP32 synthesis: one pair per thread on small maps (Nside 90: 6.4 us, 7.5 with two),
-  // two in the middle (Nside 256: 17.0 us, 18.8 with one, 18.7 with four; Nside 512:
-  // 69, 85, 71), four on large ones (Nside 1024: 436 us, 531 with two); FP64 is bound
-  // by its unit and takes one
+  // FP32 synthesis: one pair per thread on small maps, two in the middle, four on large
+  // ones (the transform with one, two and four: Nside 128 39, 42, 44 us; Nside 256 66, 64,
+  // 69; Nside 512 206, 194, 196; Nside 1024 913, 821, 781); FP64 is bound by its unit and
+  // takes one
   P.syn_np[1] = P.npairs >= 1536 ? 4 : P.npairs >= 384 ? 2 : 1;
   return with_diag(P, [&](const double *mant, const int *expo) {
     return build_pair_tables(P, mant, expo);

@@ -352,7 +352,7 @@ static float4 *dd_view(double2 *p) { return reinterpret_cast<float4 *>(p); }
 
 wf_status alm2map_df64(Plan &P, const double *alm, double *map) {
   const double2 *a = reinterpret_cast<const double2 *>(alm);
-  WF_TRY(launch_prescale_dd(P, a, dd_view(P.xs64)));
+  WF_TRY(launch_alm_to_dd(P, a, dd_view(P.xs64)));
   WF_TRY(launch_legendre_synth_dd(P, dd_view(P.xs64), dd_view(P.F64), nullptr, P.lmax));
   WF_TRY(launch_ring_dd(P, RING_SYNTH, dd_view(P.F64), nullptr, nullptr, map, nullptr,
                         P.lmax));
@@ -684,7 +684,7 @@ static wf_status fp64_step(Plan &P, const double2 *x, double2 *gx, double *num,
                           cudaMemcpyHostToDevice, P.stream));
   WF_CUDA(cudaMemcpyAsync(gx, x, sizeof(double2) * P.nalm, cudaMemcpyDeviceToDevice,
                           P.stream));
-  if (dd) WF_TRY(launch_prescale_dd(P, x, dd_view(P.xs64)));
+  if (dd) WF_TRY(launch_alm_to_dd(P, x, dd_view(P.xs64)));
   // opts.timing: events around the double-float synthesis, ring step and
   // analysis (kernels 3, 5, 4 of wf_kernel_stats)
   const bool timed = dd && P.opts.timing;

@@ -276,7 +276,7 @@ struct Plan {
   // optional per-kernel timing inside the captured graphs (opts.timing):
   // events around the Legendre analysis (k = 0) and synthesis (k = 1) of
   // every iteration of a chunk; accumulated over active iterations only
-  // timed kernels: 0 analysis, 1 synthesis, 2 ring step (both launches)
+  // timed kernels: 0 analysis, 1 synthesis, 2 ring step (its launch or two)
   std::vector<cudaEvent_t> tev;     // [3 kernels][2 (start, stop)][chunk]
   int tev_chunk = 0;
   // 3, 4: double-float Legendre synthesis / analysis and 5: FP64 ring step
@@ -327,7 +327,7 @@ void free_pair_tables(Plan &P);
 // pairs (re hi, re lo, im hi, im lo), 16 bytes like an FP64 complex (the
 // plan's F64 / G64 / xs64 buffers hold them in this form), the format of the
 // double-float ring transforms.
-wf_status launch_prescale_dd(const Plan &P, const double2 *x, float4 *xs);
+wf_status launch_alm_to_dd(const Plan &P, const double2 *x, float4 *xs);
 wf_status launch_legendre_synth_dd(const Plan &P, const float4 *xs, float4 *F,
                                    const SolverState *st, int lstatic);
 wf_status launch_legendre_anal_dd(const Plan &P, const float4 *G, double2 *x,
