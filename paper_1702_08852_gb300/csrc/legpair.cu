@@ -39,7 +39,7 @@
 // and in FP64 CTAs, of their own, so no number of pairs per thread and no Nside mixes the
 // two kinds.  In the analysis a block's sums over them are separate ones, of even and odd
 // l instead of E and O: a map that is zero but on nine rings around the equator comes out
-// to 1.6e-7 in FP32 at Nside 512 (1.3e-4 without it) and to 2e-14 in FP64 (1.9e-13).
+// to 1.6e-7 in FP32 at Nside 512 (1.3e-4 without it) and to 6.5e-16 in FP64 (1.8e-13).
 //
 // Bound: the FP64 unit, 2 multiply-adds per clock and SM (98 and 92 % busy at Nside 512).
 // At Nside 1024, lmax 2048 (3.14e9 terms) the synthesis takes 16.6 ms (21.4 ms with the
